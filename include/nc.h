@@ -376,9 +376,11 @@ nc_status nc_design_map(nc_ctx* ctx, long long n, const double* in, const unsign
  * x -/+ 0.5 (xmax - xmin) and then widen by 1.2 / narrow by 0.7 where a variable
  * moves monotonically / oscillates; move limits 0.1 of the way to the
  * asymptotes and `move` of the box; Svanberg's convex approximation of both
- * functions; the subproblem is solved through its dual, bisection on the
- * multiplier to floating-point resolution (the multiplier goes to
- * *lambda_host, and max_j |x_new - x| to *change_host; either may be NULL).
+ * functions; the subproblem is solved through its dual, a bracketing search for
+ * the multiplier down to a few units in its last place (the multiplier, at which
+ * the approximated constraint holds, goes to *lambda_host, and max_j |x_new - x|
+ * to *change_host; either may be NULL).  A workspace of 9 values per variable is
+ * kept by the context (not allocated where the device would keep less than 8 GB).
  * Synchronous.  NC_ERR_ARG for invalid sizes or options, NC_ERR_NAN for a
  * non-finite value. */
 nc_status nc_mma_update(nc_ctx* ctx, long long n, int iter, double* x, double* xold1,

@@ -203,6 +203,7 @@ void nc_destroy(nc_ctx* ctx) {
   cudaFree(ctx->pub_lin);
   cudaFree(ctx->ref_lin);
   cudaFree(ctx->asm_lin);
+  cudaFree(ctx->mma_ws);
   if (ctx->cap) cudaStreamDestroy(ctx->cap);
   delete ctx;
 }
