@@ -7,14 +7,31 @@
 // T_{n,e} = int_e N_n = h^3/8.  P is symmetric, so the same call applies the
 // chain rule dPhi/drho = P dPhi/dgamma~.
 //
-// On a uniform grid every element matrix is the same, so r^2 K + M is applied
-// node by node as a sum over the node's (up to 8) elements of the closed-form
-// Q1 entries (stiffness h/3, 0, -h/12, -h/12 and mass h^3/216 * 2^(shared
-// coordinates), by the number of coordinates in which the two corners differ).
-// The SPD system is solved by Jacobi-preconditioned conjugate gradients in FP64.
+// On a uniform grid r^2 K + M is a sum of products of the 1-D stiffness and mass
+// matrices.  Both have a boundary row that is half the interior row with the
+// missing neighbour mirrored, so the operator is one symmetric 27-point stencil
+// with four weights (by the number of coordinates that differ) on mirrored
+// neighbours, halved once per boundary coordinate; its diagonal is a constant
+// halved the same way.  The SPD system is solved by Jacobi-preconditioned
+// conjugate gradients in FP64.
+//
+// An iteration is two kernels, and no scalar returns to the host: alpha, beta and
+// the stopping test are taken by the block that ends a reduction, and the host
+// enqueues batches of iterations (those after convergence return at once).
+//  * k_cg_apply forms p = r / d + beta p on the fly while it loads its tile, then
+//    q = A p and <p, q>: per plane, the four edge and four corner neighbours are
+//    summed once and meet their weights afterwards, 15 FP64 operations per node
+//    with the update of p, where a sum over the eight elements takes 64;
+//  * k_cg_update takes the steps of x and r with <r, r> and <r, r/d>.
+// FP64 operations bound both (two FP64 lanes per SM).  80x80x160 (1.06M nodes, 19
+// iterations): 1.86 ms, k_cg_apply 67 us and k_cg_update 23 us an iteration; 5.75 ms
+// with one kernel per vector operation, a 64-term product (146 us) and three host
+// reads per iteration.
+#include <algorithm>
 #include <cmath>
 
 #include "nc_internal.cuh"
+#include "nc_reduce.cuh"
 
 namespace nc {
 nc_status set_err(nc_ctx* ctx, nc_status st, const std::string& msg);
@@ -29,60 +46,213 @@ constexpr int FT = 256;
 
 inline unsigned fblocks(long long n) { return (unsigned)((n + FT - 1) / FT); }
 
+// Weights of the mirrored 27-point stencil by the number of coordinates in which the
+// neighbour differs, and the reciprocal of the diagonal w[0] (interior values).
 struct HelmCoef {
-  double A[4];  // entry of r^2 K_e + M_e by the number of differing coordinates
+  double w[4], inv_d;
 };
 
 HelmCoef helm_coef(double h, double R) {
   const double r2 = R * R / 12.0;
-  const double K[4] = {h / 3.0, 0.0, -h / 12.0, -h / 12.0};
-  const double M[4] = {8.0, 4.0, 2.0, 1.0};
+  const double K[4] = {h / 3.0, 0.0, -h / 12.0, -h / 12.0};  // element stiffness entries
+  const double M[4] = {8.0, 4.0, 2.0, 1.0};                  // element mass entries, x h^3/216
+  const double elems[4] = {8.0, 4.0, 2.0, 1.0};              // elements that share both nodes
   HelmCoef c;
-  for (int q = 0; q < 4; ++q) c.A[q] = r2 * K[q] + M[q] * h * h * h / 216.0;
+  for (int q = 0; q < 4; ++q) c.w[q] = elems[q] * (r2 * K[q] + M[q] * h * h * h / 216.0);
+  c.inv_d = 1.0 / c.w[0];
   return c;
 }
 
-// y = (r^2 K + M) x, one thread per node; diag receives the diagonal if not null.
-__global__ void k_helm_apply(LevelDev d, HelmCoef c, const double* __restrict__ x,
-                             double* __restrict__ y, double* __restrict__ diag) {
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (n >= d.Nn) return;
-  int i, j, k;
-  node_ijk(d, n, i, j, k);
-  const long long sy = d.nx + 1, sz = (long long)(d.nx + 1) * (d.ny + 1);
-  double acc = 0.0, dg = 0.0;
-  for (int a = 0; a < 8; ++a) {  // the node is local corner a of element (i-ia, j-ja, k-ka)
-    const int ia = a & 1, ja = (a >> 1) & 1, ka = (a >> 2) & 1;
-    const int ie = i - ia, je = j - ja, ke = k - ka;
-    if (ie < 0 || je < 0 || ke < 0 || ie >= d.nx || je >= d.ny || ke >= d.nz) continue;
-    const long long n0 = ie + sy * (je + (long long)(d.ny + 1) * ke);
-    for (int b = 0; b < 8; ++b) {
-      const long long m = n0 + (b & 1) + ((b >> 1) & 1) * sy + ((b >> 2) & 1) * sz;
-      acc += c.A[__popc(a ^ b)] * (x ? x[m] : 0.0);
+// State of one solve, on the device.
+struct CgState {
+  double bb, tol2, rr, rz, alpha, beta;
+  int it, done;  // done: 0 running, 1 converged, 2 iteration limit, 3 non-finite input
+  unsigned ticket, pad;
+};
+constexpr int CG_MAX_IT = 1000;
+
+__device__ __forceinline__ int on_face(int i, int n) { return i == 0 || i == n; }
+// 2^b, from the exponent bits (an integer conversion would take the FP64 pipe)
+__device__ __forceinline__ double pow2(int b) { return __hiloint2double((1023 + b) << 20, 0); }
+
+// b_n = sum over the node's elements of rho_e h^3 / 8; r = b, x = 0, <b, b>, <b, b/d>.
+__global__ void __launch_bounds__(FT) k_cg_rhs(LevelDev d, HelmCoef c, const double* __restrict__ rho,
+                                               double* __restrict__ r, double* __restrict__ x,
+                                               double* partial, CgState* s) {
+  const double w = d.h * d.h * d.h * 0.125;
+  double bb = 0.0, bz = 0.0;
+  for (long long n = blockIdx.x * (long long)FT + threadIdx.x; n < d.Nn; n += (long long)gridDim.x * FT) {
+    int i, j, k;
+    node_ijk(d, n, i, j, k);
+    double acc = 0.0;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+      const int ie = i - (a & 1), je = j - ((a >> 1) & 1), ke = k - ((a >> 2) & 1);
+      if (ie < 0 || je < 0 || ke < 0 || ie >= d.nx || je >= d.ny || ke >= d.nz) continue;
+      acc += rho[ie + (long long)d.nx * (je + (long long)d.ny * ke)];
     }
-    dg += c.A[0];
+    acc *= w;
+    r[n] = acc;
+    x[n] = 0.0;
+    bb += acc * acc;
+    bz += acc * acc * pow2(on_face(i, d.nx) + on_face(j, d.ny) + on_face(k, d.nz));
   }
-  if (y) y[n] = acc;
-  if (diag) diag[n] = dg;
+  bb = block_fold<false, FT>(bb);
+  if (threadIdx.x == 0) partial[blockIdx.x] = bb;
+  bz = block_fold<false, FT>(bz);
+  if (threadIdx.x == 0) partial[gridDim.x + blockIdx.x] = bz;
+  if (!last_block(&s->ticket)) return;
+  bb = fold_partials<false, FT>(gridDim.x, partial);
+  bz = fold_partials<false, FT>(gridDim.x, partial + gridDim.x);
+  if (threadIdx.x == 0) {
+    s->bb = s->rr = bb;
+    s->tol2 = 1e-26 * bb;  // ||r|| <= 1e-13 ||b||
+    s->rz = bz * c.inv_d;
+    s->beta = 0.0;
+    s->it = 0;
+    s->done = !isfinite(bb) ? 3 : (bb > 0.0 ? 0 : 1);
+  }
 }
 
-// b_n = sum over the node's elements of rho_e h^3 / 8
-__global__ void k_helm_rhs(LevelDev d, const double* __restrict__ rho, double* __restrict__ b) {
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (n >= d.Nn) return;
-  int i, j, k;
-  node_ijk(d, n, i, j, k);
-  double acc = 0.0;
-  for (int a = 0; a < 8; ++a) {
-    const int ie = i - (a & 1), je = j - ((a >> 1) & 1), ke = k - ((a >> 2) & 1);
-    if (ie < 0 || je < 0 || ke < 0 || ie >= d.nx || je >= d.ny || ke >= d.nz) continue;
-    acc += rho[ie + (long long)d.nx * (je + (long long)d.ny * ke)];
+// Index of grid line position g, mirrored at both ends (and kept inside for the
+// positions of a ragged tile that no owned node reads).
+__device__ __forceinline__ int mirror(int g, int n) {
+  g = g < 0 ? -g : (g > n ? 2 * n - g : g);
+  return g < 0 ? 0 : (g > n ? n : g);
+}
+
+// p = r/d + beta p_old, q = A p, alpha = <r, r/d> / <p, q>.
+// A block marches a 32 x 8 node tile over zc planes; a plane of p with its halo is
+// formed in shared memory (two buffers, one barrier per plane), the loads of the
+// next plane in flight meanwhile.  P and Q are a plane's contributions to its own and
+// to the adjacent planes' products.
+constexpr int HTX = 32, HTY = FT / HTX, HW = HTX + 2, HSLOTS = HW * (HTY + 2);
+__global__ void __launch_bounds__(FT) k_cg_apply(LevelDev d, HelmCoef c, int zc, long long items,
+                                                 int tiles_x, int tiles_y,
+                                                 const double* __restrict__ r,
+                                                 const double* __restrict__ p_old,
+                                                 double* __restrict__ p_new, double* __restrict__ q,
+                                                 double* partial, CgState* s) {
+  if (s->done) return;
+  const double beta = s->beta;
+  const bool first = s->it == 0;  // p_old is not set yet
+  __shared__ double sm[2][HSLOTS];
+  const int tx = threadIdx.x % HTX, ty = threadIdx.x / HTX;
+  const long long sy = d.nx + 1, sz = (long long)(d.nx + 1) * (d.ny + 1);
+  static_assert(HSLOTS <= 2 * FT, "two tile slots per thread");
+  double pq = 0.0;
+  for (long long item = blockIdx.x; item < items; item += gridDim.x) {
+    const int bx = (int)(item % tiles_x), by = (int)(item / tiles_x % tiles_y);
+    const int k0 = (int)(item / tiles_x / tiles_y) * zc, k1 = min(k0 + zc, d.nz + 1);
+    long long at[2];  // node of the slot in plane 0
+    double wxy[2], wxy2[2];  // 1/d on an inner and on a boundary plane
+    bool own[2];      // the slot is a node of this tile
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int t = threadIdx.x + u * FT, sx = t % HW, s2 = t / HW;
+      const int gi = bx * HTX + sx - 1, gj = by * HTY + s2 - 1;
+      const int mi = mirror(gi, d.nx), mj = mirror(gj, d.ny);
+      at[u] = mi + sy * mj;
+      wxy[u] = c.inv_d * pow2(on_face(mi, d.nx) + on_face(mj, d.ny));
+      wxy2[u] = 2.0 * wxy[u];
+      own[u] = sx >= 1 && sx <= HTX && s2 >= 1 && s2 <= HTY && gi <= d.nx && gj <= d.ny;
+    }
+    const bool two = threadIdx.x + FT < HSLOTS;
+    const int i = bx * HTX + tx, j = by * HTY + ty;
+    const bool in = i <= d.nx && j <= d.ny;
+    const int faces_xy = on_face(i, d.nx) + on_face(j, d.ny);
+    double rv[2] = {0.0, 0.0}, pv[2] = {0.0, 0.0};
+    auto load = [&](int kk) {
+      const long long off = sz * mirror(kk, d.nz);
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (u == 0 || two) {
+          rv[u] = r[at[u] + off];
+          pv[u] = first ? 0.0 : p_old[at[u] + off];
+        }
+    };
+    double P = 0.0, Q1 = 0.0, Q2 = 0.0, cp = 0.0;  // P, Q of plane kk - 1, Q of kk - 2, p of kk - 1
+    load(k0 - 1);
+    for (int kk = k0 - 1; kk <= k1; ++kk) {
+      double* b = sm[kk & 1];
+      const int gk = mirror(kk, d.nz);
+      const bool face = on_face(gk, d.nz);
+#pragma unroll
+      for (int u = 0; u < 2; ++u)
+        if (u == 0 || two) {
+          const double v = rv[u] * (face ? wxy2[u] : wxy[u]) + beta * pv[u];
+          b[threadIdx.x + u * FT] = v;
+          if (own[u] && kk >= k0 && kk < k1) p_new[at[u] + sz * gk] = v;
+        }
+      if (kk < k1) load(kk + 1);
+      __syncthreads();
+      const double* m = b + (ty + 1) * HW + tx + 1;
+      const double cc = m[0];
+      const double e = (m[-1] + m[1]) + (m[-HW] + m[HW]);
+      const double dg = (m[-HW - 1] + m[-HW + 1]) + (m[HW - 1] + m[HW + 1]);
+      const double Q = c.w[1] * cc + (c.w[2] * e + c.w[3] * dg);
+      if (kk > k0 && in) {
+        const int kp = kk - 1;
+        double y = P + (Q2 + Q);
+        const int faces = faces_xy + on_face(kp, d.nz);
+        if (faces) y *= pow2(-faces);
+        q[i + sy * j + sz * kp] = y;
+        pq += cp * y;
+      }
+      if (kk >= k0 && kk < k1) P = c.w[0] * cc + (c.w[1] * e + c.w[2] * dg);
+      Q2 = Q1;
+      Q1 = Q;
+      cp = cc;
+    }
+    __syncthreads();  // the next tile writes the buffers
   }
-  b[n] = acc * d.h * d.h * d.h * 0.125;
+  pq = block_fold<false, FT>(pq);
+  if (threadIdx.x == 0) partial[blockIdx.x] = pq;
+  if (!last_block(&s->ticket)) return;
+  pq = fold_partials<false, FT>(gridDim.x, partial);
+  if (threadIdx.x == 0) {
+    s->alpha = s->rz / pq;
+    if (!(pq > 0.0)) s->done = 1;
+  }
+}
+
+// x += alpha p, r -= alpha q, beta = the ratio of the new <r, r/d> to the old.
+__global__ void __launch_bounds__(FT) k_cg_update(LevelDev d, HelmCoef c, const double* __restrict__ p,
+                                                  const double* __restrict__ q, double* __restrict__ x,
+                                                  double* __restrict__ r, double* partial, CgState* s) {
+  if (s->done) return;
+  const double alpha = s->alpha;
+  double rr = 0.0, rz = 0.0;
+  for (long long n = blockIdx.x * (long long)FT + threadIdx.x; n < d.Nn; n += (long long)gridDim.x * FT) {
+    int i, j, k;
+    node_ijk(d, n, i, j, k);
+    x[n] += alpha * p[n];
+    const double v = r[n] - alpha * q[n];
+    r[n] = v;
+    rr += v * v;
+    rz += v * (v * pow2(on_face(i, d.nx) + on_face(j, d.ny) + on_face(k, d.nz)));
+  }
+  rr = block_fold<false, FT>(rr);
+  if (threadIdx.x == 0) partial[blockIdx.x] = rr;
+  rz = block_fold<false, FT>(rz);
+  if (threadIdx.x == 0) partial[gridDim.x + blockIdx.x] = rz;
+  if (!last_block(&s->ticket)) return;
+  rr = fold_partials<false, FT>(gridDim.x, partial);
+  rz = fold_partials<false, FT>(gridDim.x, partial + gridDim.x) * c.inv_d;
+  if (threadIdx.x == 0) {
+    s->rr = rr;
+    s->beta = rz / s->rz;
+    s->rz = rz;
+    if (++s->it >= CG_MAX_IT) s->done = 2;
+    if (rr <= s->tol2) s->done = 1;
+  }
 }
 
 // gamma~_e = mean of the element's eight nodal values
-__global__ void k_elem_mean(LevelDev d, const double* __restrict__ x, double* __restrict__ g) {
+// (once the solve has converged)
+__global__ void k_elem_mean(LevelDev d, const double* __restrict__ x, double* __restrict__ g,
+                            const CgState* s) {
+  if (s->done != 1) return;
   const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (e >= d.E) return;
   int i, j, k;
@@ -90,17 +260,26 @@ __global__ void k_elem_mean(LevelDev d, const double* __restrict__ x, double* __
   const long long sy = d.nx + 1, sz = (long long)(d.nx + 1) * (d.ny + 1);
   const long long n0 = i + sy * (j + (long long)(d.ny + 1) * k);
   double acc = 0.0;
+#pragma unroll
   for (int a = 0; a < 8; ++a) acc += x[n0 + (a & 1) + ((a >> 1) & 1) * sy + ((a >> 2) & 1) * sz];
   g[e] = 0.125 * acc;
 }
 
-nc_status dot(nc_ctx* ctx, long long n, const double* a, const double* b, double* out,
-              cudaStream_t s) {
-  vmdot(n, 1, a, 0, b, ctx->dscal, ctx->partial, s);
-  nc_status st = cuda_check(ctx, cudaMemcpyAsync(out, ctx->dscal, sizeof(double),
-                                                 cudaMemcpyDeviceToHost, s), "filter dot");
-  if (st != NC_OK) return st;
-  return cuda_check(ctx, cudaStreamSynchronize(s), "filter sync");
+// Planes per tile march of k_cg_apply: the count that leaves the busiest SM the least
+// work, a march of zc planes costing zc + 2 halo planes, blocks spread over 152 SMs
+// (short marches for small grids, where whole columns would leave SMs idle).
+int planes_per_block(long long tiles, int planes) {
+  int best = 1;
+  double cost = 1e300;
+  for (int zc = 1; zc <= planes && zc <= 64; ++zc) {
+    const long long blocks = tiles * ((planes + zc - 1) / zc);
+    const double t = (double)((blocks + 151) / 152) * (zc + 2);
+    if (t < cost) {
+      cost = t;
+      best = zc;
+    }
+  }
+  return best;
 }
 
 }  // namespace
@@ -114,43 +293,42 @@ extern "C" nc_status nc_filter(nc_ctx* ctx, const double* rho, double* gamma_f, 
   const LevelDev& d = L.d;
   const long long Nn = d.Nn;
   nc_status st;
-  for (int q = 0; q < 6; ++q)
+  for (int q = 0; q < 5; ++q)
     if (!ctx->filt[q] &&
         (st = cuda_check(ctx, cudaMalloc((void**)&ctx->filt[q], sizeof(double) * Nn),
                          "cudaMalloc filter")) != NC_OK)
       return st;
-  double *x = ctx->filt[0], *r = ctx->filt[1], *z = ctx->filt[2], *p = ctx->filt[3],
-         *q = ctx->filt[4], *dg = ctx->filt[5];
+  double *x = ctx->filt[0], *r = ctx->filt[1], *q = ctx->filt[2], *p[2] = {ctx->filt[3], ctx->filt[4]};
   const HelmCoef c = helm_coef(d.h, radius);
-  k_helm_apply<<<fblocks(Nn), FT, 0, s>>>(d, c, nullptr, nullptr, dg);
-  k_helm_rhs<<<fblocks(Nn), FT, 0, s>>>(d, rho, r);  // r = b (x = 0)
-  vzero(Nn, x, s);
-  double bb, rz, pq, rr;
-  if ((st = dot(ctx, Nn, r, r, &bb, s)) != NC_OK) return st;
-  if (!std::isfinite(bb)) return set_err(ctx, NC_ERR_NAN, "nc_filter: non-finite design");
-  const double tol2 = 1e-26 * bb;  // ||r|| <= 1e-13 ||b||
-  if (bb > 0.0) {
-    vdiv(Nn, (const double*)r, (const double*)dg, z, s);
-    vcopy(Nn, (const double*)z, p, s);
-    if ((st = dot(ctx, Nn, r, z, &rz, s)) != NC_OK) return st;
-    int it = 0;
-    for (; it < 1000; ++it) {
-      k_helm_apply<<<fblocks(Nn), FT, 0, s>>>(d, c, p, q, nullptr);
-      if ((st = dot(ctx, Nn, p, q, &pq, s)) != NC_OK) return st;
-      if (!(pq > 0.0)) break;
-      const double alpha = rz / pq;
-      vaxpy(Nn, alpha, (const double*)p, x, s);
-      vaxpy(Nn, -alpha, (const double*)q, r, s);
-      if ((st = dot(ctx, Nn, r, r, &rr, s)) != NC_OK) return st;
-      if (rr <= tol2) break;
-      vdiv(Nn, (const double*)r, (const double*)dg, z, s);
-      double rz_new;
-      if ((st = dot(ctx, Nn, r, z, &rz_new, s)) != NC_OK) return st;
-      vxpay(Nn, (const double*)z, rz_new / rz, p, s);  // p = z + beta p
-      rz = rz_new;
+  CgState* cg = (CgState*)ctx->dscal;
+  static_assert(sizeof(CgState) <= sizeof(double) * (MAX_RESTART + 2) * 4, "dscal holds the state");
+  cudaMemsetAsync(cg, 0, sizeof(CgState), s);
+  const unsigned vb = (unsigned)std::min<long long>((Nn + FT - 1) / FT, RED_BLOCKS_MAX);
+  k_cg_rhs<<<vb, FT, 0, s>>>(d, c, rho, r, x, ctx->partial, cg);
+  const int tiles_x = (d.nx + HTX) / HTX, tiles_y = (d.ny + HTY) / HTY;
+  const long long tiles = (long long)tiles_x * tiles_y;
+  const int zc = planes_per_block(tiles, d.nz + 1);
+  const long long items = tiles * ((d.nz + zc) / zc);
+  const unsigned ab = (unsigned)std::min<long long>(items, (long long)MAX_RESTART * RED_BLOCKS_MAX);
+  CgState h;
+  int m = 0, batch = 16;  // a radius of 2.5 h takes about 19 iterations
+  do {
+    for (int i = 0; i < batch; ++i, ++m) {
+      k_cg_apply<<<ab, FT, 0, s>>>(d, c, zc, items, tiles_x, tiles_y, r, p[m & 1], p[(m + 1) & 1], q,
+                                   ctx->partial, cg);
+      k_cg_update<<<vb, FT, 0, s>>>(d, c, p[(m + 1) & 1], q, x, r, ctx->partial, cg);
     }
-    if (it >= 1000) return set_err(ctx, NC_ERR_MAXIT, "nc_filter: CG did not converge");
-  }
-  k_elem_mean<<<fblocks(d.E), FT, 0, s>>>(d, x, gamma_f);
-  return cuda_check(ctx, cudaStreamSynchronize(s), "nc_filter");
+    k_elem_mean<<<fblocks(d.E), FT, 0, s>>>(d, x, gamma_f, cg);
+    if ((st = cuda_check(ctx, cudaMemcpyAsync(&h, cg, sizeof(h), cudaMemcpyDeviceToHost, s),
+                         "nc_filter")) != NC_OK ||
+        (st = cuda_check(ctx, cudaStreamSynchronize(s), "nc_filter")) != NC_OK)
+      return st;
+    // the rest at the rate seen so far
+    const double rate = std::log(h.rr / h.bb) / m;
+    const double need = rate < 0.0 ? std::log(h.tol2 / h.rr) / rate + 1.0 : 32.0;
+    batch = need >= 1.0 && need < 32.0 ? (int)need : 32;
+  } while (!h.done);
+  if (h.done == 3) return set_err(ctx, NC_ERR_NAN, "nc_filter: non-finite design");
+  if (h.done == 2) return set_err(ctx, NC_ERR_MAXIT, "nc_filter: CG did not converge");
+  return NC_OK;
 }

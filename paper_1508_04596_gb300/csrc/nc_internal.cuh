@@ -130,7 +130,7 @@ struct nc_ctx {
   double* cjel = nullptr;     // coarsest-level element Jacobians (40 x 40 per element)
   long long cjel_elems = 0;
   cudaStream_t cap = nullptr; // stream used to capture the V-cycle graph
-  double* filt[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};  // filter CG
+  double* filt[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // filter CG
   double* pub_lin = nullptr;  // linearisation of nc_linearize (level 0, FP64)
   double* asm_lin = nullptr;  // linearisation used by nc_assemble (level 0, FP64)
   double* ref_lin = nullptr;  // linearisation of the mixed adjoint's FP64 refinement (level 0)

@@ -1,0 +1,63 @@
+// Deterministic reductions that end in the kernel that computes them: every block
+// writes one partial per value, and the block that finishes last folds the
+// partials in index order (no second launch).  The result does not depend on which
+// block that is.
+#pragma once
+#include <cuda_runtime.h>
+
+namespace nc {
+
+template <bool MAX, typename T>
+__device__ __forceinline__ T warp_fold(T v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const T w = __shfl_down_sync(0xffffffffu, v, o);
+    v = MAX ? (v > w ? v : w) : v + w;
+  }
+  return v;
+}
+
+// Block sum (or maximum) of one value per thread, THREADS threads, valid in thread 0.
+template <bool MAX, int THREADS, typename T>
+__device__ __forceinline__ T block_fold(T v) {
+  __shared__ T sh[THREADS / 32];
+  v = warp_fold<MAX>(v);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  __syncthreads();  // sh may still be read from a previous call
+  if (lane == 0) sh[wid] = v;
+  __syncthreads();
+  if (wid == 0) {
+    v = lane < THREADS / 32 ? sh[lane] : T(0);
+    v = warp_fold<MAX>(v);
+  }
+  return v;
+}
+
+// Whether the calling block is the last of its grid to get here.  Its threads then
+// see what every other block wrote before its own call.  The ticket, 0 on entry,
+// is left at 0.
+__device__ __forceinline__ bool last_block(unsigned* ticket) {
+  __shared__ bool last;
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    last = atomicAdd(ticket, 1u) == gridDim.x * gridDim.y * gridDim.z - 1;
+    if (last) *ticket = 0;
+  }
+  __syncthreads();
+  if (last) __threadfence();
+  return last;
+}
+
+// Sum (or maximum) of nb partials in a fixed order, valid in thread 0 (one block).
+template <bool MAX, int THREADS>
+__device__ __forceinline__ double fold_partials(int nb, const double* partial) {
+  double v = 0.0;
+  for (int b = threadIdx.x; b < nb; b += THREADS) {
+    const double q = __ldcg(partial + b);
+    v = MAX ? (v > q ? v : q) : v + q;
+  }
+  return block_fold<MAX, THREADS>(v);
+}
+
+}  // namespace nc
