@@ -379,7 +379,7 @@ nc_status nc_design_map(nc_ctx* ctx, long long n, const double* in, const unsign
  * functions; the subproblem is solved through its dual, a bracketing search for
  * the multiplier down to a few units in its last place (the multiplier, at which
  * the approximated constraint holds, goes to *lambda_host, and max_j |x_new - x|
- * to *change_host; either may be NULL).  A workspace of 9 values per variable is
+ * to *change_host; either may be NULL).  A workspace of 12 values per variable is
  * kept by the context (not allocated where the device would keep less than 8 GB).
  * Synchronous.  NC_ERR_ARG for invalid sizes or options, NC_ERR_NAN for a
  * non-finite value. */

@@ -28,13 +28,17 @@
 // The host enqueues a batch of passes and reads the state once: passes after the
 // search has ended return at once.  Measured at 80x80x160 (1.02M variables, 432k
 // active): 57 bisection passes of 117 us, each followed by a host read, took 8.1 ms
-// for the volume and the update; now 1.22 ms.  10-15 passes are needed, and each takes
-// the coefficients of the active variables, computed once per call, from a
-// compacted workspace (9 values per active variable; two square roots and two
-// divisions per variable and pass, bound by the FP64 pipe).
+// for the volume and the update.  10-15 passes are needed now, and each takes the
+// coefficients of the active variables, computed once per call, from a compacted
+// workspace.  A pass is bound by the FP64 pipe; for a variable inside its limits
+//   p1/(U - y) + q1/(y - L) = (sqrt P + sqrt Q) (p1/sqrt P + q1/sqrt Q) / (U - L),
+// and at a limit the term does not depend on lam, so a pass takes two reciprocal
+// square roots per variable and no division: 49 us a pass, 0.92 ms for the volume
+// and the update (73 us and 1.22 ms with two square roots and two divisions).
 #include <cmath>
 
 #include "nc_internal.cuh"
+#include "nc_reduce.cuh"
 
 namespace nc {
 nc_status set_err(nc_ctx* ctx, nc_status st, const std::string& msg);
@@ -57,67 +61,11 @@ inline unsigned mma_blocks(long long n) {
   return (unsigned)(b < RED_BLOCKS_MAX ? b : RED_BLOCKS_MAX);
 }
 
-__device__ __forceinline__ double warp_sum_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
-__device__ __forceinline__ double warp_max_d(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, o));
-  return v;
-}
-
 // Block sum (or maximum) of one value per thread -> partial[blockIdx.x].
 template <bool MAX>
 __device__ __forceinline__ void block_partial(double v, double* partial) {
-  __shared__ double sh[MT / 32];
-  v = MAX ? warp_max_d(v) : warp_sum_d(v);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    v = lane < MT / 32 ? sh[lane] : 0.0;
-    v = MAX ? warp_max_d(v) : warp_sum_d(v);
-    if (lane == 0) partial[blockIdx.x] = v;
-  }
-}
-
-// Whether the calling block is the last of its grid to get here.  Its threads then
-// see what every other block wrote before its own call.  The ticket is left at 0.
-__device__ __forceinline__ bool last_block(unsigned* ticket) {
-  __shared__ bool last;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    if (last) *ticket = 0;
-  }
-  __syncthreads();
-  if (last) __threadfence();
-  return last;
-}
-
-// Sum (or maximum) of nb partials in a fixed order, valid in thread 0 (one block).
-template <bool MAX>
-__device__ __forceinline__ double fold_block(int nb, const double* partial) {
-  __shared__ double sh[MT / 32];
-  double v = 0.0;
-  for (int b = threadIdx.x; b < nb; b += MT) {
-    const double q = __ldcg(partial + b);
-    v = MAX ? fmax(v, q) : v + q;
-  }
-  v = MAX ? warp_max_d(v) : warp_sum_d(v);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  __syncthreads();
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  if (wid == 0) {
-    v = lane < MT / 32 ? sh[lane] : 0.0;
-    v = MAX ? warp_max_d(v) : warp_sum_d(v);
-  }
-  return v;
+  v = block_fold<MAX, MT>(v);
+  if (threadIdx.x == 0) partial[blockIdx.x] = v;
 }
 
 // out[0], out[1]: sums of (1 - gamma_e) and of the active count over the variables
@@ -131,12 +79,10 @@ __global__ void __launch_bounds__(MT) k_volume(long long n, const double* __rest
     cnt += 1.0;
   }
   block_partial<false>(acc, partial);
-  __syncthreads();
   block_partial<false>(cnt, partial + gridDim.x);
   if (!last_block(ticket)) return;
-  const double s0 = fold_block<false>(gridDim.x, partial);
-  __syncthreads();
-  const double s1 = fold_block<false>(gridDim.x, partial + gridDim.x);
+  const double s0 = fold_partials<false, MT>(gridDim.x, partial);
+  const double s1 = fold_partials<false, MT>(gridDim.x, partial + gridDim.x);
   if (threadIdx.x == 0) {
     out[0] = s0;
     out[1] = s1;
@@ -146,9 +92,12 @@ __global__ void __launch_bounds__(MT) k_volume(long long n, const double* __rest
 // dg = -1/(vf count) on active entries, 0 elsewhere; nothing without an active one
 __global__ void k_volume_grad(long long n, const unsigned char* __restrict__ active,
                               const double* __restrict__ sums, double vf, double* __restrict__ dg) {
+  __shared__ double sh;
+  if (threadIdx.x == 0) sh = -(1.0 / (vf * sums[1]));  // one FP64 division per block
+  __syncthreads();
+  const double dgval = sh;
   const long long j = blockIdx.x * (long long)MT + threadIdx.x;
   if (j >= n || !(sums[1] > 0.0)) return;
-  const double dgval = -(1.0 / (vf * sums[1]));
   dg[j] = (!active || active[j]) ? dgval : 0.0;
 }
 
@@ -174,16 +123,18 @@ __device__ __forceinline__ void mma_asym(long long j, int k, double xj,
   upp[j] = u;
 }
 
-// What the separable Lagrangian of one variable needs for any multiplier; c is
-// its term of the approximated constraint at y = x.
+// What the separable Lagrangian of one variable needs for any multiplier.  w =
+// 1/(u - l); c, ta, tb: the variable's term p1/(u - y) + q1/(y - l) of the
+// approximated constraint at y = x, and at alpha and beta less c.
 struct MmaCoef {
-  double l, u, alpha, beta, p0, q0, p1, q1, c;
+  double l, u, alpha, beta, p0, q0, p1, q1, w, c, ta, tb;
 };
-constexpr int MMA_COEFS = 9;
+constexpr int MMA_COEFS = 12;
 
-__device__ __forceinline__ MmaCoef mma_coef(double xj, double l, double u, double a0, double a1,
-                                            double xmin, double xmax, double move) {
-  const double d = xmax - xmin, r = 1e-5 / d;
+// The coefficients but for w, c, ta and tb, which only the evaluations need.
+__device__ __forceinline__ MmaCoef mma_coef_y(double xj, double l, double u, double a0, double a1,
+                                              double xmin, double xmax, double move, double r) {
+  const double d = xmax - xmin;
   const double a0p = fmax(a0, 0.0), a0m = fmax(-a0, 0.0);
   const double a1p = fmax(a1, 0.0), a1m = fmax(-a1, 0.0);
   const double ux2 = (u - xj) * (u - xj), xl2 = (xj - l) * (xj - l);
@@ -196,19 +147,36 @@ __device__ __forceinline__ MmaCoef mma_coef(double xj, double l, double u, doubl
   m.q1 = xl2 * (0.001 * a1p + 1.001 * a1m + r);
   m.alpha = fmax(fmax(xmin, l + 0.1 * (xj - l)), xj - move * d);
   m.beta = fmin(fmin(xmax, u - 0.1 * (u - xj)), xj + move * d);
-  m.c = m.p1 / (u - xj) + m.q1 / (xj - l);
   return m;
 }
 
-// Minimiser y_j(lam) of the separable Lagrangian, and its term of the
-// approximated constraint (both fractions over one denominator).
+__device__ __forceinline__ double mma_term_at(const MmaCoef& m, double y) {
+  const double a = m.u - y, b = y - m.l;
+  return (m.p1 * b + m.q1 * a) / (a * b);
+}
+
+__device__ __forceinline__ MmaCoef mma_coef(double xj, double l, double u, double a0, double a1,
+                                            double xmin, double xmax, double move, double r) {
+  MmaCoef m = mma_coef_y(xj, l, u, a0, a1, xmin, xmax, move, r);
+  m.w = 1.0 / (u - l);
+  m.c = mma_term_at(m, xj);
+  m.ta = mma_term_at(m, m.alpha) - m.c;
+  m.tb = mma_term_at(m, m.beta) - m.c;
+  return m;
+}
+
+// Minimiser y_j(lam) of the separable Lagrangian, clipped to [alpha, beta].
 __device__ __forceinline__ double mma_y(const MmaCoef& m, double lam) {
   const double sP = sqrt(m.p0 + lam * m.p1), sQ = sqrt(m.q0 + lam * m.q1);
   return fmin(fmax((m.l * sP + m.u * sQ) / (sP + sQ), m.alpha), m.beta);
 }
+// Its term of the approximated constraint (P, Q > 0: the approximation adds 1e-5 / d).
 __device__ __forceinline__ double mma_term(const MmaCoef& m, double lam) {
-  const double y = mma_y(m, lam), a = m.u - y, b = y - m.l;
-  return (m.p1 * b + m.q1 * a) / (a * b) - m.c;
+  const double P = m.p0 + lam * m.p1, Q = m.q0 + lam * m.q1;
+  const double rP = rsqrt(P), rQ = rsqrt(Q), sP = P * rP, sQ = Q * rQ;
+  const double den = sP + sQ, num = m.l * sP + m.u * sQ;  // y = num / den
+  const double t = (den * m.w) * (m.p1 * rP + m.q1 * rQ) - m.c;
+  return num <= m.alpha * den ? m.ta : (num >= m.beta * den ? m.tb : t);
 }
 
 // The search for the multiplier.  a is the newest point, b the end of the bracket
@@ -321,6 +289,8 @@ __device__ __forceinline__ int tile_slot(bool act, int& total) {
   return pos;
 }
 
+// entry i of the workspace; EVAL: what an evaluation takes, else what y takes
+template <bool EVAL>
 __device__ __forceinline__ MmaCoef ws_load(const MmaWs& w, long long i) {
   const long long st = (long long)gridDim.x * w.seg;
   MmaCoef m;
@@ -332,7 +302,12 @@ __device__ __forceinline__ MmaCoef ws_load(const MmaWs& w, long long i) {
   m.q0 = w.v[i + 5 * st];
   m.p1 = w.v[i + 6 * st];
   m.q1 = w.v[i + 7 * st];
-  m.c = w.v[i + 8 * st];
+  if (EVAL) {
+    m.w = w.v[i + 8 * st];
+    m.c = w.v[i + 9 * st];
+    m.ta = w.v[i + 10 * st];
+    m.tb = w.v[i + 11 * st];
+  }
   return m;
 }
 
@@ -340,7 +315,7 @@ __device__ __forceinline__ MmaCoef ws_load(const MmaWs& w, long long i) {
 __device__ __forceinline__ void mma_finish(double acc, double f1, double* partial, MmaSearch* s) {
   block_partial<false>(acc, partial);
   if (!last_block(&s->ticket)) return;
-  const double sum = fold_block<false>(gridDim.x, partial);
+  const double sum = fold_partials<false, MT>(gridDim.x, partial);
   if (threadIdx.x == 0) {
     MmaSearch t = *s;
     mma_advance(t, f1 + sum);
@@ -353,7 +328,7 @@ struct MmaArgs {
   const double *x, *xo1, *xo2, *df0, *df1;
   double *low, *upp;
   const unsigned char* active;
-  double xmin, xmax, move, scale0, f1;
+  double xmin, xmax, move, r, scale0, f1;  // r = 1e-5 / (xmax - xmin)
 };
 
 // Asymptotes of the iteration, the coefficients into the workspace (STORE), and the
@@ -373,10 +348,11 @@ __global__ void __launch_bounds__(MT) k_mma_begin(MmaArgs a, int iter, MmaWs w, 
       const double xj = a.x[j];
       mma_asym(j, iter, xj, a.xo1, a.xo2, a.low, a.upp, a.xmin, a.xmax);
       const MmaCoef m = mma_coef(xj, a.low[j], a.upp[j], a.scale0 * a.df0[j], a.df1[j], a.xmin,
-                                 a.xmax, a.move);
+                                 a.xmax, a.move, a.r);
       acc += mma_term(m, 0.0);
       if (STORE) {
-        const double q[MMA_COEFS] = {m.l, m.u, m.alpha, m.beta, m.p0, m.q0, m.p1, m.q1, m.c};
+        const double q[MMA_COEFS] = {m.l, m.u, m.alpha, m.beta, m.p0, m.q0,
+                                     m.p1, m.q1, m.w, m.c, m.ta, m.tb};
 #pragma unroll
         for (int r = 0; r < MMA_COEFS; ++r)
           w.v[r * (long long)gridDim.x * w.seg + base + cnt + pos] = q[r];
@@ -397,12 +373,12 @@ __global__ void __launch_bounds__(MT) k_mma_dual(MmaArgs a, MmaWs w, double* par
   if (STORE) {
     const int cnt = w.cnt[blockIdx.x];
     const long long base = (long long)blockIdx.x * w.seg;
-    for (int i = threadIdx.x; i < cnt; i += MT) acc += mma_term(ws_load(w, base + i), lam);
+    for (int i = threadIdx.x; i < cnt; i += MT) acc += mma_term(ws_load<true>(w, base + i), lam);
   } else {
     for (long long j = blockIdx.x * (long long)MT + threadIdx.x; j < a.n; j += (long long)gridDim.x * MT)
       if (!a.active || a.active[j])
         acc += mma_term(mma_coef(a.x[j], a.low[j], a.upp[j], a.scale0 * a.df0[j], a.df1[j], a.xmin,
-                                 a.xmax, a.move), lam);
+                                 a.xmax, a.move, a.r), lam);
   }
   mma_finish(acc, a.f1, partial, s);
 }
@@ -425,9 +401,9 @@ __global__ void __launch_bounds__(MT) k_mma_commit(MmaArgs a, MmaWs w, double* x
       const double xj = x[j];
       double y = xj;
       if (act)
-        y = mma_y(STORE ? ws_load(w, at + pos)
-                        : mma_coef(xj, a.low[j], a.upp[j], a.scale0 * a.df0[j], a.df1[j], a.xmin,
-                                   a.xmax, a.move), lam);
+        y = mma_y(STORE ? ws_load<false>(w, at + pos)
+                        : mma_coef_y(xj, a.low[j], a.upp[j], a.scale0 * a.df0[j], a.df1[j], a.xmin,
+                                     a.xmax, a.move, a.r), lam);
       xo2[j] = xo1[j];
       xo1[j] = xj;
       x[j] = y;
@@ -437,7 +413,7 @@ __global__ void __launch_bounds__(MT) k_mma_commit(MmaArgs a, MmaWs w, double* x
   }
   block_partial<true>(mx, partial);
   if (!last_block(&s->ticket)) return;
-  const double v = fold_block<true>(gridDim.x, partial);
+  const double v = fold_partials<true, MT>(gridDim.x, partial);
   if (threadIdx.x == 0) s->change = v;
 }
 
@@ -546,7 +522,7 @@ nc_status nc_mma_update(nc_ctx* ctx, long long n, int iter, double* x, double* x
   MmaWs w;
   const bool store = mma_workspace(ctx, n, nb, w);
   const MmaArgs a{n, x, xold1, xold2, df0, df1, low, upp, active, o.xmin, o.xmax, o.move,
-                  o.df0_scale, f1};
+                  1e-5 / (o.xmax - o.xmin), o.df0_scale, f1};
   MmaSearch* srch = (MmaSearch*)ctx->dscal;
   static_assert(sizeof(MmaSearch) <= sizeof(double) * (MAX_RESTART + 2) * 4, "dscal holds the search");
   cudaMemsetAsync(srch, 0, sizeof(MmaSearch), s);
