@@ -375,7 +375,7 @@ nc_status nc_linearize(nc_ctx* ctx, const double* x, const double* gam, void* st
   if (!ctx->pub_lin &&
       (st = dev_alloc(ctx, &ctx->pub_lin, (long long)LIN_SLOTS * L.d.E)) != NC_OK)
     return st;
-  op_linearize<double>(L.d, L.c64, x, gam, L.f64.src, ctx->pub_lin, (cudaStream_t)stream);
+  op_linearize(L.d, L.c64, x, gam, L.f64.src, ctx->pub_lin, (cudaStream_t)stream);
   ctx->pub_x = x;
   ctx->pub_gam = gam;
   return cuda_check(ctx, cudaGetLastError(), "nc_linearize");
@@ -385,7 +385,7 @@ nc_status nc_jvp_lin(nc_ctx* ctx, const double* v, double* Jv, void* stream) {
   if (!ctx || !v || !Jv) return set_err(ctx, NC_ERR_ARG, "nc_jvp_lin: bad argument");
   if (!ctx->pub_x) return set_err(ctx, NC_ERR_ARG, "nc_jvp_lin: call nc_linearize first");
   const Level& L = ctx->lv[0];
-  op_jvp_cached<double>(L.d, L.c64, ctx->pub_x, ctx->pub_gam, L.f64.src, ctx->pub_lin, v, Jv,
+  op_jvp_cached(L.d, L.c64, ctx->pub_x, ctx->pub_gam, L.f64.src, ctx->pub_lin, v, Jv,
                         ctx->Y, (cudaStream_t)stream);
   return cuda_check(ctx, cudaGetLastError(), "nc_jvp_lin");
 }
@@ -394,7 +394,7 @@ nc_status nc_jtvp_lin(nc_ctx* ctx, const double* w, double* JTw, void* stream) {
   if (!ctx || !w || !JTw) return set_err(ctx, NC_ERR_ARG, "nc_jtvp_lin: bad argument");
   if (!ctx->pub_x) return set_err(ctx, NC_ERR_ARG, "nc_jtvp_lin: call nc_linearize first");
   const Level& L = ctx->lv[0];
-  op_jtvp_cached<double>(L.d, L.c64, ctx->pub_x, ctx->pub_gam, L.f64.src, ctx->pub_lin, w, JTw,
+  op_jtvp_cached(L.d, L.c64, ctx->pub_x, ctx->pub_gam, L.f64.src, ctx->pub_lin, w, JTw,
                          ctx->Y, (cudaStream_t)stream);
   return cuda_check(ctx, cudaGetLastError(), "nc_jtvp_lin");
 }
@@ -410,7 +410,7 @@ nc_status nc_assemble(nc_ctx* ctx, const void* x, const void* gam, void* S, int 
     if (!ctx->asm_lin &&
         (st = dev_alloc(ctx, &ctx->asm_lin, (long long)LIN_SLOTS * L.d.E)) != NC_OK)
       return st;
-    op_linearize<double>(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src,
+    op_linearize(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src,
                          ctx->asm_lin, s);
     op_assemble<double>(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src,
                         ctx->asm_lin, (double*)S, ctx->Y, s);

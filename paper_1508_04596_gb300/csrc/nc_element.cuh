@@ -200,15 +200,10 @@ NC_HD void scale_coef(ElemCoef<R>& k, const ElemConst<R>& c) {
   k.wK = c.wh * k.K;
 }
 
+// Coefficients of an element with u_e^T u_e = S.
 template <typename R>
-NC_HD ElemCoef<R> elem_coef(const R xe[5][8], R gam, R s, const ElemConst<R>& c, R& S) {
+NC_HD ElemCoef<R> coef_of(R S, R gam, R s, const ElemConst<R>& c) {
   ElemCoef<R> k;
-  R acc = R(0);
-#pragma unroll
-  for (int i = 0; i < 3; ++i)
-#pragma unroll
-    for (int a = 0; a < 8; ++a) acc += xe[i][a] * xe[i][a];
-  S = acc;
   k.alpha = c.h * alpha_of(gam, c);
   k.K = c.inv_h * K_of(gam, c);
   // (tau_e/h)^-2 = h^2 (S/(4h)^2 + (4 Pr/h^2)^2 + alpha_e^2) and
@@ -218,6 +213,17 @@ NC_HD ElemCoef<R> elem_coef(const R xe[5][8], R gam, R s, const ElemConst<R>& c,
   k.s = c.h * s;
   scale_coef(k, c);
   return k;
+}
+
+template <typename R>
+NC_HD ElemCoef<R> elem_coef(const R xe[5][8], R gam, R s, const ElemConst<R>& c, R& S) {
+  R acc = R(0);
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int a = 0; a < 8; ++a) acc += xe[i][a] * xe[i][a];
+  S = acc;
+  return coef_of(S, gam, s, c);
 }
 
 // Strong residuals at a quadrature point; body = rM without the pressure
@@ -464,6 +470,24 @@ NC_HD R point_sens(const QP<R>& q, const QP<R>& t, const ElemCoef<R>& k, R dalph
 // slot s of an element is stored at cache[s * stride].
 constexpr int LIN_GP = 19;
 constexpr int LIN_SLOTS = 8 * LIN_GP + 4;
+
+template <typename R>
+NC_HD void store_point(const QP<R>& q, const ElemCoef<R>& k, const ElemConst<R>& c, R* o,
+                       long long stride) {
+  R body[3], rM[3], rT;
+  strong(q, k, c, body, rM, rT);
+#pragma unroll
+  for (int i = 0; i < 3; ++i) o[i * stride] = q.u[i];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+#pragma unroll
+    for (int j = 0; j < 3; ++j) o[(3 + 3 * i + j) * stride] = q.G[i][j];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) o[(12 + j) * stride] = q.gT[j];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) o[(15 + i) * stride] = k.wtau * rM[i];
+  o[18 * stride] = k.wtauT * rT;
+}
 
 template <typename R>
 NC_HD void load_lin_pair(const R* cache, long long stride, int P, QP<R> q[2], R rM[2][3], R rT[2]) {
@@ -826,22 +850,8 @@ NC_HD void elem_linearize(const R xe[5][8], R gam, R s, const ElemConst<R>& c, R
   QP<R> q[8];
   interp_all8<R>(xe, q);
 #pragma unroll
-  for (int p = 0; p < 8; ++p) {
-    R body[3], rM[3], rT;
-    strong(q[p], k, c, body, rM, rT);
-    R* o = cache + (long long)(p * LIN_GP) * stride;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) o[i * stride] = q[p].u[i];
-#pragma unroll
-    for (int i = 0; i < 3; ++i)
-#pragma unroll
-      for (int j = 0; j < 3; ++j) o[(3 + 3 * i + j) * stride] = q[p].G[i][j];
-#pragma unroll
-    for (int j = 0; j < 3; ++j) o[(12 + j) * stride] = q[p].gT[j];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) o[(15 + i) * stride] = k.wtau * rM[i];
-    o[18 * stride] = k.wtauT * rT;
-  }
+  for (int p = 0; p < 8; ++p)
+    store_point(q[p], k, c, cache + (long long)(p * LIN_GP) * stride, stride);
   cache[(long long)(8 * LIN_GP) * stride] = k.tau;
   cache[(long long)(8 * LIN_GP + 1) * stride] = k.tauT;
   cache[(long long)(8 * LIN_GP + 2) * stride] = k.alpha;

@@ -143,14 +143,27 @@ struct nc_ctx {
 
 namespace nc {
 
-// Element-row scratch: the 40 rows (f, a) of the element kernels, in blocks of
-// YB consecutive elements: row r = 8 f + a of element e sits at
-// Y[(e / YB) * 40 YB + r YB + e % YB].  A warp's 32 elements write each row as
-// one contiguous 128-byte (FP32) or 256-byte (FP64) segment, and the 40 rows of an
-// element lie at fixed offsets from its first (offsets known at compile time, so
-// no per-row address arithmetic).  Holds 40 * round_up(E, YB) values.
+// Element-row scratch of the operators that keep a row per element, diag(J) and the
+// assembly: the 40 rows (f, a) in blocks of YB consecutive elements, row r = 8 f + a
+// of element e at Y[(e / YB) * 40 YB + r YB + e % YB].  A warp's 32 elements write
+// each row as one contiguous 128-byte (FP32) or 256-byte (FP64) segment, and the 40
+// rows of an element lie at fixed offsets from its first.  Holds 40 * round_up(E, YB)
+// values.  The marching operators (MarchPlan) use the same array and never more of it.
 constexpr int YB = 32;
 inline long long scratch_len(long long E) { return 40 * ((E + YB - 1) / YB * YB); }
+
+// How the marching element kernels (nc_march.cuh) cut a grid: the element rows j into
+// runs of rc, and the x-node faces of the element layers, l = i + (nx + 1) k, into
+// chunks of `stride`: nchunk chunks for every run, or, with rc = 1 and `flat`, over
+// all runs together, l = i + (nx + 1) (k + nz j).  A chunk writes 10 sums per lane
+// (32) and node row (rc + 1 of a run).
+struct MarchPlan {
+  long long nchunk;
+  int runs, rc, stride, flat;
+  __host__ __device__ long long warps() const { return flat ? nchunk : nchunk * runs; }
+  long long scratch() const { return warps() * (rc + 1) * 320; }
+};
+MarchPlan march_plan(const LevelDev& d, bool fp64);
 
 // ---- element operators (nc_kernels.cu); Y is scratch of scratch_len(E) elements of R
 template <typename R>
@@ -164,15 +177,12 @@ void op_jtvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam,
              const R* w, R* out, R* Y, cudaStream_t s);
 // linearisation cache (LIN_SLOTS values per element, slot-major) and the
 // products that read it
-template <typename R>
-void op_linearize(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
-                  R* cache, cudaStream_t s);
-template <typename R>
-void op_jvp_cached(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam,
-                   const R* src, const R* cache, const R* v, R* out, R* Y, cudaStream_t s);
-template <typename R>
-void op_jtvp_cached(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam,
-                    const R* src, const R* cache, const R* w, R* out, R* Y, cudaStream_t s);
+void op_linearize(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam, const double* src,
+                  double* cache, cudaStream_t s);
+void op_jvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
+                   const double* src, const double* cache, const double* v, double* out, double* Y, cudaStream_t s);
+void op_jtvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
+                    const double* src, const double* cache, const double* w, double* out, double* Y, cudaStream_t s);
 template <typename R>
 void op_diag(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
              R* out, R* Y, cudaStream_t s);

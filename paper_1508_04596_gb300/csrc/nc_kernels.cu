@@ -1,14 +1,15 @@
 // Element operators, assembly by node-owner gather, and grid transfers.
 //
-// Assembly is colouring-free and deterministic: one thread per element writes
-// its 40 element rows (f, a) to a scratch array (blocked by YB elements, see
-// nc_internal.cuh); one thread per node then sums the rows of its (up to) eight
-// elements in the fixed local order a = 0..7.  No atomics, so results are
-// bitwise reproducible.
+// Assembly is colouring-free and deterministic: the element kernels write sums per
+// node and element layer (the marching operators, nc_march.cuh) or 40 rows per element
+// (diag(J) and the assembled Jacobian) to a scratch array, and one thread per node
+// adds those of its node in a fixed order.  No atomics, so results are bitwise
+// reproducible.
 #include <type_traits>
 
 #include "nc_element_f2.cuh"
 #include "nc_internal.cuh"
+#include "nc_march.cuh"
 
 namespace nc {
 
@@ -50,20 +51,6 @@ __device__ __forceinline__ long long elem_node(const LevelDev& d, long long e, i
   return node_id(d, i + (a & 1), j + ((a >> 1) & 1), k + ((a >> 2) & 1));
 }
 
-// nodal velocities of the state (the only state data the cached products read)
-template <typename R>
-__device__ __forceinline__ void load_vel(const LevelDev& d, const R* __restrict__ x, long long e,
-                                         R ue[3][8]) {
-  const long long n0 = elem_node(d, e, 0);
-  const long long sy = d.nx + 1, sz = (long long)(d.nx + 1) * (d.ny + 1);
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const long long n = n0 + (a & 1) + ((a >> 1) & 1) * sy + ((a >> 2) & 1) * sz;
-#pragma unroll
-    for (int f = 0; f < 3; ++f) ue[f][a] = x[f * d.Nn + n];
-  }
-}
-
 // first row of element e in the blocked scratch; row r = 8 f + a is at + r YB
 __device__ __forceinline__ long long yrow0(long long e) {
   static_assert(YB == 32, "yrow0 takes the block by a shift");
@@ -78,86 +65,6 @@ __device__ __forceinline__ void store_elem(long long E, long long e, const R out
   for (int f = 0; f < 5; ++f)
 #pragma unroll
     for (int a = 0; a < 8; ++a) y[(f * 8 + a) * YB] = out[f][a];
-}
-
-template <typename R>
-__global__ void __launch_bounds__(ELEM_THREADS) k_elem_res(LevelDev d, ElemConst<R> c,
-                                                           const R* __restrict__ x,
-                                                           const R* __restrict__ gam,
-                                                           const R* __restrict__ src, R* Y) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e >= d.E) return;
-  R xe[5][8], out[5][8];
-  load_elem(d, x, e, xe, false);
-  elem_residual<R>(xe, gam[e], src ? src[e] : R(0), c, out);
-  store_elem(d.E, e, out, Y);
-}
-
-// Two blocks per SM, up to 255 registers: both products then run without
-// spilling.  J^T w, whose fluxes keep more values live, is 10 % faster in FP32
-// than at three blocks (168 registers, spilled); J v, with fewer values live, is
-// 1.5 % faster at 192x192x384 than at three blocks (where it spills 300 bytes a
-// thread), 0.4 % at 128^3, and as fast as 64-thread blocks at five per SM.
-// FP32 takes the packed-pair element routines (two lanes of FP32 arithmetic per
-// instruction).  The nodal loads stay node by node with 64-bit indices: per-field
-// base pointers with 32-bit row offsets cut the FP32 J v's instructions by 12 %
-// but made it 10 % slower (more long-scoreboard stalls).
-template <typename R, bool TRANSPOSE>
-__global__ void __launch_bounds__(ELEM_THREADS, 2) k_elem_lin(LevelDev d, ElemConst<R> c,
-                                                           const R* __restrict__ x,
-                                                           const R* __restrict__ gam,
-                                                           const R* __restrict__ src,
-                                                           const R* __restrict__ v, R* Y) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e >= d.E) return;
-  R xe[5][8], ve[5][8], out[5][8];
-  load_elem(d, x, e, xe, false);
-  load_elem(d, v, e, ve, true);  // Dirichlet columns removed
-  const R g = gam[e], s = src ? src[e] : R(0);
-  if constexpr (std::is_same<R, float>::value) {
-    if (TRANSPOSE)
-      elem_jtvp_f2(xe, ve, g, s, c, out);
-    else
-      elem_jvp_f2(xe, ve, g, s, c, out);
-  } else {
-    if (TRANSPOSE)
-      elem_jtvp<R>(xe, ve, g, s, c, out);
-    else
-      elem_jvp<R>(xe, ve, g, s, c, out);
-  }
-  store_elem(d.E, e, out, Y);
-}
-
-template <typename R>
-__global__ void __launch_bounds__(ELEM_THREADS) k_elem_linearize(LevelDev d, ElemConst<R> c,
-                                                                 const R* __restrict__ x,
-                                                                 const R* __restrict__ gam,
-                                                                 const R* __restrict__ src,
-                                                                 R* cache) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e >= d.E) return;
-  R xe[5][8];
-  load_elem(d, x, e, xe, false);
-  elem_linearize<R>(xe, gam[e], src ? src[e] : R(0), c, cache + e, d.E);
-}
-
-// J v / J^T w from the linearisation cache: only the direction and the nodal
-// velocities of the state are gathered.
-template <typename R, bool TRANSPOSE>
-__global__ void __launch_bounds__(ELEM_THREADS) k_elem_lin_cached(
-    LevelDev d, ElemConst<R> c, const R* __restrict__ x, const R* __restrict__ gam,
-    const R* __restrict__ src, const R* __restrict__ cache, const R* __restrict__ v, R* Y) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e >= d.E) return;
-  R ue[3][8], ve[5][8], out[5][8];
-  load_vel(d, x, e, ue);
-  load_elem(d, v, e, ve, true);  // Dirichlet columns removed
-  const R g = gam[e], s = src ? src[e] : R(0);
-  if (TRANSPOSE)
-    elem_jtvp_lin<R>(cache + e, d.E, ue, ve, g, s, c, out);
-  else
-    elem_jvp_lin<R>(cache + e, d.E, ue, ve, g, s, c, out);
-  store_elem(d.E, e, out, Y);
 }
 
 // Column col = 5 b + g of every element Jacobian: the element product with the
@@ -253,20 +160,6 @@ __global__ void __launch_bounds__(ELEM_THREADS) k_elem_diag(LevelDev d, ElemCons
   store_elem(d.E, e, out, Y);
 }
 
-__global__ void __launch_bounds__(ELEM_THREADS) k_elem_sens(LevelDev d, ElemConst<double> c,
-                                                            const double* __restrict__ x,
-                                                            const double* __restrict__ gam,
-                                                            const double* __restrict__ src,
-                                                            const double* __restrict__ lam,
-                                                            double* out) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e >= d.E) return;
-  double xe[5][8], le[5][8];
-  load_elem(d, x, e, xe, false);
-  load_elem(d, lam, e, le, true);  // Dirichlet rows excluded
-  out[e] = elem_sens<double>(xe, le, gam[e], src ? src[e] : 0.0, c);
-}
-
 enum GatherMode { G_RES = 0, G_LIN = 1, G_DIAG = 2 };
 
 __device__ __forceinline__ int patch_face_count(const LevelDev& d, int i, int j, int k) {
@@ -282,22 +175,10 @@ __device__ __forceinline__ int patch_face_count(const LevelDev& d, int i, int j,
   return cnt;
 }
 
+// Row values of node n from the sums acc of its elements: Dirichlet rows, patch flux.
 template <typename R, int MODE>
-__global__ void __launch_bounds__(NODE_THREADS) k_gather(LevelDev d, const R* __restrict__ Y,
-                                                         const R* __restrict__ xv, R* out) {
-  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (n >= d.Nn) return;
-  int i, j, k;
-  node_ijk(d, n, i, j, k);
-  R acc[5] = {R(0), R(0), R(0), R(0), R(0)};
-#pragma unroll
-  for (int a = 0; a < 8; ++a) {
-    const int ie = i - (a & 1), je = j - ((a >> 1) & 1), ke = k - ((a >> 2) & 1);
-    if (ie < 0 || je < 0 || ke < 0 || ie >= d.nx || je >= d.ny || ke >= d.nz) continue;
-    const long long e = ie + (long long)d.nx * (je + (long long)d.ny * ke);
-#pragma unroll
-    for (int f = 0; f < 5; ++f) acc[f] += Y[yrow0(e) + (f * 8 + a) * YB];
-  }
+__device__ __forceinline__ void node_rows(const LevelDev& d, long long n, int i, int j, int k, R acc[5],
+                                          const R* __restrict__ xv, R* __restrict__ out) {
   const uint8_t fl = d.flag[n];
   if (MODE == G_RES) {
     const int pc = patch_face_count(d, i, j, k);
@@ -318,6 +199,41 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather(LevelDev d, const R* __
     }
     out[f * d.Nn + n] = v;
   }
+}
+
+// Gather of the 40 element rows (diag(J)).
+template <typename R, int MODE>
+__global__ void __launch_bounds__(NODE_THREADS) k_gather(LevelDev d, const R* __restrict__ Y,
+                                                         const R* __restrict__ xv, R* out) {
+  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (n >= d.Nn) return;
+  int i, j, k;
+  node_ijk(d, n, i, j, k);
+  R acc[5] = {R(0), R(0), R(0), R(0), R(0)};
+#pragma unroll
+  for (int a = 0; a < 8; ++a) {
+    const int ie = i - (a & 1), je = j - ((a >> 1) & 1), ke = k - ((a >> 2) & 1);
+    if (ie < 0 || je < 0 || ke < 0 || ie >= d.nx || je >= d.ny || ke >= d.nz) continue;
+    const long long e = ie + (long long)d.nx * (je + (long long)d.ny * ke);
+#pragma unroll
+    for (int f = 0; f < 5; ++f) acc[f] += Y[yrow0(e) + (f * 8 + a) * YB];
+  }
+  node_rows<R, MODE>(d, n, i, j, k, acc, xv, out);
+}
+
+// Gather of the marching kernels' sums.
+template <typename R, int MODE>
+__global__ void __launch_bounds__(NODE_THREADS) k_gather_march(LevelDev d, MarchPlan mp,
+                                                               const R* __restrict__ Y,
+                                                               const R* __restrict__ xv,
+                                                               R* __restrict__ out) {
+  const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (n >= d.Nn) return;
+  int i, j, k;
+  node_ijk(d, n, i, j, k);
+  R acc[5] = {R(0), R(0), R(0), R(0), R(0)};
+  march::node_sums(d, mp, i, j, k, Y, acc);
+  node_rows<R, MODE>(d, n, i, j, k, acc, xv, out);
 }
 
 template <typename R, bool ZERO>
@@ -454,47 +370,100 @@ __global__ void k_coarsen_elem(LevelDev f, const R* __restrict__ gf, LevelDev c,
 
 }  // namespace
 
+// Chunks of 31 faces share their end faces; 32 where a layer's row of faces divides 32
+// and no element straddles two chunks.  The run length is the one that takes the
+// fewest steps on the busiest scheduler.  FP32 kernels are bound by latency at 8 warps
+// on each of 152 SMs, which finish a run in about the time one takes; a run of rc rows
+// costs its steps and 0.6 of one for the first row's loads and the extra row of sums.
+// FP64 steps pass the 608 schedulers' FP64 units one after the other, so there the
+// runs per scheduler count.  (96^3: FP32 J v 119, 92, 86, 84 us with runs of 1, 4, 8, 24
+// rows; 64^3, FP64 J v from the store: 680, 703, 673, 694, 683, 811 us with 1 to 6.)  Runs
+// of several rows are taken only where their sums fit the element-row scratch; single
+// rows, cut into chunks all together, always do: 640 values per 31 faces (2 rows of 10
+// sums per lane) against 40 per element, or per 32 faces with one element across.
+MarchPlan march_plan(const LevelDev& d, bool fp64) {
+  const long long slots = fp64 ? 608 : 8 * 152;
+  const double extra = fp64 ? 0.15 : 0.6;
+  MarchPlan p;
+  p.stride = 32 % (d.nx + 1) == 0 ? 32 : 31;
+  const long long faces = (long long)(d.nx + 1) * d.nz;
+  p.flat = 1;
+  p.rc = 1;
+  p.runs = d.ny;
+  p.nchunk = (faces * d.ny + p.stride - 1) / p.stride;
+  auto steps = [&](const MarchPlan& m) {  // a lone run per FP64 unit hides no latency
+    const long long turns = (m.warps() + slots - 1) / slots;
+    return (m.rc + extra) * (fp64 && turns == 1 ? 1.12 : (double)turns);
+  };
+  double cost = steps(p);
+  MarchPlan q = p;
+  q.flat = 0;
+  q.nchunk = (faces + p.stride - 1) / p.stride;
+  for (q.rc = 2; q.rc <= 24 && q.rc <= d.ny; ++q.rc) {
+    q.runs = (d.ny + q.rc - 1) / q.rc;
+    const double t = steps(q);
+    if (t < cost && q.scratch() <= scratch_len(d.E)) {
+      cost = t;
+      p = q;
+    }
+  }
+  return p;
+}
+
+// A warp for every chunk of faces and run of rows, four to a block: one on each
+// scheduler (blocks of one warp leave schedulers idle, FP64 23 % slower at 64^3).
+template <typename R, int K>
+static void run_march(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
+                      const R* cache, const R* v, R* out, cudaStream_t s) {
+  const MarchPlan mp = march_plan(d, sizeof(R) == 8);
+  march::k_march<R, K><<<nblocks(mp.warps(), march::WARPS), 32 * march::WARPS, 0, s>>>(
+      d, c, mp, x, gam, src, cache, v, out);
+}
+
+template <typename R, int MODE>
+static void run_gather(const LevelDev& d, const R* Y, const R* xv, R* out, cudaStream_t s) {
+  k_gather_march<R, MODE><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(
+      d, march_plan(d, sizeof(R) == 8), Y, xv, out);
+}
+
 template <typename R>
 void op_residual(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
                  R* r, R* Y, cudaStream_t s) {
-  k_elem_res<R><<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src, Y);
-  k_gather<R, G_RES><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, Y, x, r);
+  run_march<R, march::RES>(d, c, x, gam, src, nullptr, nullptr, Y, s);
+  run_gather<R, G_RES>(d, Y, x, r, s);
 }
 
 template <typename R>
 void op_jvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
             const R* v, R* out, R* Y, cudaStream_t s) {
-  k_elem_lin<R, false><<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src, v, Y);
-  k_gather<R, G_LIN><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, Y, v, out);
+  run_march<R, march::JVP>(d, c, x, gam, src, nullptr, v, Y, s);
+  run_gather<R, G_LIN>(d, Y, v, out, s);
 }
 
 template <typename R>
 void op_jtvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
              const R* w, R* out, R* Y, cudaStream_t s) {
-  k_elem_lin<R, true><<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src, w, Y);
-  k_gather<R, G_LIN><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, Y, w, out);
+  run_march<R, march::JTVP>(d, c, x, gam, src, nullptr, w, Y, s);
+  run_gather<R, G_LIN>(d, Y, w, out, s);
 }
 
-template <typename R>
-void op_linearize(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
-                  R* cache, cudaStream_t s) {
-  k_elem_linearize<R><<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src, cache);
+void op_linearize(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
+                  const double* src, double* cache, cudaStream_t s) {
+  run_march<double, march::LINEARIZE>(d, c, x, gam, src, nullptr, nullptr, cache, s);
 }
 
-template <typename R>
-void op_jvp_cached(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam,
-                   const R* src, const R* cache, const R* v, R* out, R* Y, cudaStream_t s) {
-  k_elem_lin_cached<R, false><<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src,
-                                                                                 cache, v, Y);
-  k_gather<R, G_LIN><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, Y, v, out);
+void op_jvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
+                   const double* src, const double* cache, const double* v, double* out, double* Y,
+                   cudaStream_t s) {
+  run_march<double, march::JVP_LIN>(d, c, x, gam, src, cache, v, Y, s);
+  run_gather<double, G_LIN>(d, Y, v, out, s);
 }
 
-template <typename R>
-void op_jtvp_cached(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam,
-                    const R* src, const R* cache, const R* w, R* out, R* Y, cudaStream_t s) {
-  k_elem_lin_cached<R, true><<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src,
-                                                                                cache, w, Y);
-  k_gather<R, G_LIN><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, Y, w, out);
+void op_jtvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
+                    const double* src, const double* cache, const double* w, double* out, double* Y,
+                    cudaStream_t s) {
+  run_march<double, march::JTVP_LIN>(d, c, x, gam, src, cache, w, Y, s);
+  run_gather<double, G_LIN>(d, Y, w, out, s);
 }
 
 template <typename R>
@@ -528,7 +497,7 @@ void op_assemble(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* 
 
 void op_sens(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
              const double* src, const double* lam, double* out, cudaStream_t s) {
-  k_elem_sens<<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src, lam, out);
+  run_march<double, march::SENS>(d, c, x, gam, src, nullptr, lam, out, s);
 }
 
 template <typename R>
@@ -587,12 +556,6 @@ void op_coarsen_elem(const LevelDev& fine, const R* gf, const LevelDev& coarse, 
                            const R*, R*, R*, cudaStream_t);                                     \
   template void op_diag<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*, const R*,  \
                            R*, R*, cudaStream_t);                                               \
-  template void op_linearize<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*,       \
-                                const R*, R*, cudaStream_t);                                    \
-  template void op_jvp_cached<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*,      \
-                                 const R*, const R*, const R*, R*, R*, cudaStream_t);           \
-  template void op_jtvp_cached<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*,     \
-                                  const R*, const R*, const R*, R*, R*, cudaStream_t);          \
   template void op_assemble<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*,        \
                                const R*, const R*, R*, R*, cudaStream_t);                       \
   template void op_impose<R>(const LevelDev&, R*, cudaStream_t);                                \

@@ -15,6 +15,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include "nc_internal.cuh"
 
@@ -123,12 +124,14 @@ void level_apply(nc_ctx* ctx, int l, bool tr, const R* v, R* out, cudaStream_t s
     op_stencil<R>(L.d, B.gst, tr, v, out, s);
     return;
   }
-  if (B.lin) {  // FP64 levels: products from the linearisation cache
-    if (tr)
-      op_jtvp_cached<R>(L.d, cst<R>(L), B.x, B.gam, B.src, B.lin, v, out, (R*)ctx->Y, s);
-    else
-      op_jvp_cached<R>(L.d, cst<R>(L), B.x, B.gam, B.src, B.lin, v, out, (R*)ctx->Y, s);
-    return;
+  if constexpr (std::is_same<R, double>::value) {
+    if (B.lin) {  // FP64 levels: products from the linearisation cache
+      if (tr)
+        op_jtvp_cached(L.d, L.c64, B.x, B.gam, B.src, B.lin, v, out, ctx->Y, s);
+      else
+        op_jvp_cached(L.d, L.c64, B.x, B.gam, B.src, B.lin, v, out, ctx->Y, s);
+      return;
+    }
   }
   if (tr)
     op_jtvp<R>(L.d, cst<R>(L), B.x, B.gam, B.src, v, out, (R*)ctx->Y, s);
@@ -282,13 +285,15 @@ nc_status linearize(nc_ctx* ctx, int nlev, const double* x, const double* gam, c
       galerkin_build<R>(ctx, l, s);
       op_stencil_diag<R>(L.d, B.gst, B.diag, s);
     } else if (assembled) {
-      if (B.lin) op_linearize<R>(L.d, cst<R>(L), B.x, B.gam, B.src, B.lin, s);
+      if constexpr (std::is_same<R, double>::value)
+        if (B.lin) op_linearize(L.d, L.c64, B.x, B.gam, B.src, B.lin, s);
       op_assemble<R>(L.d, cst<R>(L), B.x, B.gam, B.src, B.lin, B.gst, (R*)ctx->Y, s);
       op_stencil_diag<R>(L.d, B.gst, B.diag, s);
     } else {
       // diag(J^T) = diag(J)
       op_diag<R>(L.d, cst<R>(L), B.x, B.gam, B.src, B.diag, (R*)ctx->Y, s);
-      if (B.lin) op_linearize<R>(L.d, cst<R>(L), B.x, B.gam, B.src, B.lin, s);
+      if constexpr (std::is_same<R, double>::value)
+        if (B.lin) op_linearize(L.d, L.c64, B.x, B.gam, B.src, B.lin, s);
     }
     if (l == nlev - 1 && coarse_dense_dofs(L) <= COARSE_DENSE_MAX) {
       const nc_status st = B.use_gst ? coarse_setup_stencil<R>(ctx, L, B.gst, &B.inv, s)
@@ -918,13 +923,13 @@ nc_status nc_adjoint_solve(nc_ctx* ctx, const double* x, const double* gam, cons
       if (!mixed) {
         store = L.f64.lin;
       } else if (refine_store(ctx, L.d.E)) {
-        op_linearize<double>(L.d, L.c64, x, gam, ctx->src64, ctx->ref_lin, s);
+        op_linearize(L.d, L.c64, x, gam, ctx->src64, ctx->ref_lin, s);
         store = ctx->ref_lin;
       }
     }
     auto jt64 = [&](const double* w, double* out) {
       if (store)
-        op_jtvp_cached<double>(L.d, L.c64, x, gam, ctx->src64, store, w, out, ctx->Y, s);
+        op_jtvp_cached(L.d, L.c64, x, gam, ctx->src64, store, w, out, ctx->Y, s);
       else
         op_jtvp<double>(L.d, L.c64, x, gam, ctx->src64, w, out, ctx->Y, s);
     };
