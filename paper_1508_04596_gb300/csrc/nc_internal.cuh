@@ -160,6 +160,7 @@ inline long long scratch_len(long long E) { return 40 * ((E + YB - 1) / YB * YB)
 struct MarchPlan {
   long long nchunk;
   int runs, rc, stride, flat;
+  int split;  // a flat plan whose chunks four warps share (nc_split.cuh)
   __host__ __device__ long long warps() const { return flat ? nchunk : nchunk * runs; }
   long long scratch() const { return warps() * (rc + 1) * 320; }
 };

@@ -10,6 +10,7 @@
 #include "nc_element_f2.cuh"
 #include "nc_internal.cuh"
 #include "nc_march.cuh"
+#include "nc_split.cuh"
 
 namespace nc {
 
@@ -407,6 +408,10 @@ MarchPlan march_plan(const LevelDev& d, bool fp64) {
       p = q;
     }
   }
+  // Four warps per chunk while that keeps the schedulers short of work (FP64: at most two
+  // chunks' quarters each): residual FP64 at 12^3 27 us against 51, at 20^3 39 against
+  // 51, at 24^3 68 against 51; FP32 J v 10.3 against 12.4 at 16^3, even at 32^3.
+  p.split = p.flat && p.nchunk <= (fp64 ? 304 : 750);
   return p;
 }
 
@@ -416,6 +421,12 @@ template <typename R, int K>
 static void run_march(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
                       const R* cache, const R* v, R* out, cudaStream_t s) {
   const MarchPlan mp = march_plan(d, sizeof(R) == 8);
+  if constexpr (march::Traits<K>::TEST) {
+    if (mp.split) {
+      march::k_split<R, K><<<(unsigned)mp.nchunk, 128, 0, s>>>(d, c, mp, x, gam, src, cache, v, out);
+      return;
+    }
+  }
   march::k_march<R, K><<<nblocks(mp.warps(), march::WARPS), 32 * march::WARPS, 0, s>>>(
       d, c, mp, x, gam, src, cache, v, out);
 }

@@ -58,8 +58,10 @@ def test_small_grids(nc, dims):
     assert rel(gp.jtvp_lin(dev(v)).cpu().numpy(), J.T @ v) <= 1e-12
 
 
-# runs of several rows (5 and 6 here), the last one shorter
-@pytest.mark.parametrize("dims,runs", [((40, 19, 220), 5), ((20, 27, 300), 6)])
+# runs of several rows (5 and 6 here), the last one shorter; single rows, a warp per chunk (the
+# smaller grids of this file share a chunk between four warps)
+@pytest.mark.parametrize("dims,runs", [((40, 19, 220), 5), ((20, 27, 300), 6),
+                                       ((32, 30, 31), 1), ((24, 24, 24), 1)])
 @pytest.mark.parametrize("dt", [torch.float64, torch.float32])
 def test_runs_of_rows(nc, dims, runs, dt):
     nx, ny, nz = dims
@@ -73,7 +75,7 @@ def test_runs_of_rows(nc, dims, runs, dt):
     vi = np.where(prob.dmask, 0.0, v)
     pick = []
     for j in (1, runs - 1, runs, runs + 1, 2 * runs, ny - 2, ny - 1):
-        for face in (31, 62, 31 * 40, 31 * 77, 31 * 150 + 30):  # chunk ends
+        for face in (31, 62, 31 * 20, 31 * 40, 31 * 77, 31 * 150 + 30):  # chunk ends
             i, k = face % (nx + 1), face // (nx + 1)
             if 0 < i < nx and 0 < k < nz:
                 pick.append(i + (nx + 1) * (j + (ny + 1) * k))
