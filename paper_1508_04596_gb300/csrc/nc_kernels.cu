@@ -10,7 +10,9 @@
 #include "nc_element_f2.cuh"
 #include "nc_internal.cuh"
 #include "nc_march.cuh"
+#include "nc_reduce.cuh"
 #include "nc_split.cuh"
+#include "nc_transfer.cuh"
 
 namespace nc {
 
@@ -237,6 +239,54 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_march(LevelDev d, March
   node_rows<R, MODE>(d, n, i, j, k, acc, xv, out);
 }
 
+// The same for a product w = A v with the dots <V_q, w>, q < k <= KB, that the smoother
+// takes of it next: the result is not read back, and no multi-dot is launched (a third
+// of the reduction launches; on a small level a launch costs more than its work).
+// Two accumulators per column; partials fold in the last block.
+template <typename R, int KB>
+__global__ void __launch_bounds__(NODE_THREADS) k_gather_dots(LevelDev d, MarchPlan mp,
+                                                              const R* __restrict__ Y,
+                                                              const R* __restrict__ xv,
+                                                              R* __restrict__ out, int k,
+                                                              const R* __restrict__ V, long long ld,
+                                                              double* partial, double* dots,
+                                                              unsigned* ticket) {
+  R a0[KB], a1[KB];
+#pragma unroll
+  for (int q = 0; q < KB; ++q) a0[q] = a1[q] = R(0);
+  for (long long n = blockIdx.x * (long long)NODE_THREADS + threadIdx.x; n < d.Nn;
+       n += (long long)gridDim.x * NODE_THREADS) {
+    int i, j, kk;
+    node_ijk(d, n, i, j, kk);
+    R acc[5] = {R(0), R(0), R(0), R(0), R(0)};
+    march::node_sums(d, mp, i, j, kk, Y, acc);
+    const uint8_t fl = d.flag[n];
+#pragma unroll
+    for (int f = 0; f < 5; ++f) {
+      const R w = (fl >> f) & 1 ? xv[f * d.Nn + n] : acc[f];
+      out[f * d.Nn + n] = w;
+      acc[f] = w;
+    }
+#pragma unroll
+    for (int q = 0; q < KB; ++q)
+      if (q < k) {
+        const R* p = V + q * ld + n;
+        R u[5];
+#pragma unroll
+        for (int f = 0; f < 5; ++f) u[f] = p[f * d.Nn];
+        a0[q] = fma(u[0], acc[0], fma(u[2], acc[2], fma(u[4], acc[4], a0[q])));
+        a1[q] = fma(u[1], acc[1], fma(u[3], acc[3], a1[q]));
+      }
+  }
+#pragma unroll
+  for (int q = 0; q < KB; ++q)
+    if (q < k) {
+      const R t = block_fold<false, NODE_THREADS>(a0[q] + a1[q]);
+      if (threadIdx.x == 0) partial[q * gridDim.x + blockIdx.x] = double(t);
+    }
+  if (last_block(ticket)) fold_values(k, gridDim.x, partial, dots);
+}
+
 template <typename R, bool ZERO>
 __global__ void k_impose(LevelDev d, R* x) {
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -279,69 +329,27 @@ __global__ void k_source_grad(LevelDev d, const double* __restrict__ src, double
   g[4 * d.Nn + n] = acc * d.h * d.h * d.h * 0.125;
 }
 
-// ---- transfers between a fine level and the next coarser one (factor 2)
-// 1-D Q1 prolongation weight of coarse node I for fine node i: 1 if i == 2I,
-// 1/2 if |i - 2I| == 1.
+// A thread per node and field (blockIdx.y): with a thread per node the coarse levels
+// are too few threads to hide the latency of 27 x 5 loads (64^3 -> 32^3: 21 us, 9 now).
 template <typename R>
-__global__ void k_restrict(LevelDev f, const R* __restrict__ rf, LevelDev c, R* rc) {
+__global__ void k_restrict(LevelDev f, const R* __restrict__ rf, LevelDev c, R* __restrict__ rc) {
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= c.Nn) return;
+  const int q = blockIdx.y;
   int I, J, K;
   node_ijk(c, n, I, J, K);
-  const uint8_t cfl = c.flag[n];
-  R acc[5] = {R(0), R(0), R(0), R(0), R(0)};
-  for (int dk = -1; dk <= 1; ++dk) {
-    const int k = 2 * K + dk;
-    if (k < 0 || k > f.nz) continue;
-    const R wk = dk ? R(0.5) : R(1);
-    for (int dj = -1; dj <= 1; ++dj) {
-      const int j = 2 * J + dj;
-      if (j < 0 || j > f.ny) continue;
-      const R wj = dj ? R(0.5) : R(1);
-      for (int di = -1; di <= 1; ++di) {
-        const int i = 2 * I + di;
-        if (i < 0 || i > f.nx) continue;
-        const R w = wk * wj * (di ? R(0.5) : R(1));
-        const long long m = node_id(f, i, j, k);
-        const uint8_t ffl = f.flag[m];
-#pragma unroll
-        for (int q = 0; q < 5; ++q)
-          if (!((ffl >> q) & 1)) acc[q] += w * rf[q * f.Nn + m];
-      }
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 5; ++q) rc[q * c.Nn + n] = ((cfl >> q) & 1) ? R(0) : acc[q];
+  rc[q * c.Nn + n] = restrict_value(f, rf + q * f.Nn, q, c.flag[n], I, J, K);
 }
 
 template <typename R>
 __global__ void k_prolong_add(LevelDev c, const R* __restrict__ zc, LevelDev f, R* zf) {
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= f.Nn) return;
+  const int q = blockIdx.y;
   int i, j, k;
   node_ijk(f, n, i, j, k);
-  const uint8_t ffl = f.flag[n];
-  const int i0 = i >> 1, i1 = (i + 1) >> 1, j0 = j >> 1, j1 = (j + 1) >> 1, k0 = k >> 1,
-            k1 = (k + 1) >> 1;
-  const R wi = (i & 1) ? R(0.5) : R(1), wj = (j & 1) ? R(0.5) : R(1), wk = (k & 1) ? R(0.5) : R(1);
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    if ((ffl >> q) & 1) continue;
-    const R* z = zc + q * c.Nn;
-    R acc;
-    if (!(i & 1) && !(j & 1) && !(k & 1)) {
-      acc = z[node_id(c, i0, j0, k0)];
-    } else {
-      acc = R(0);
-      const int is[2] = {i0, i1}, js[2] = {j0, j1}, ks[2] = {k0, k1};
-      const int ni = (i & 1) ? 2 : 1, nj = (j & 1) ? 2 : 1, nk = (k & 1) ? 2 : 1;
-      for (int a = 0; a < nk; ++a)
-        for (int b = 0; b < nj; ++b)
-          for (int cc = 0; cc < ni; ++cc) acc += z[node_id(c, is[cc], js[b], ks[a])];
-      acc *= wi * wj * wk;
-    }
-    zf[q * f.Nn + n] += acc;
-  }
+  if ((f.flag[n] >> q) & 1) return;
+  zf[q * f.Nn + n] += prolong_value(c, zc + q * c.Nn, i, j, k);
 }
 
 template <typename R>
@@ -432,9 +440,22 @@ static void run_march(const LevelDev& d, const ElemConst<R>& c, const R* x, cons
 }
 
 template <typename R, int MODE>
-static void run_gather(const LevelDev& d, const R* Y, const R* xv, R* out, cudaStream_t s) {
-  k_gather_march<R, MODE><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(
-      d, march_plan(d, sizeof(R) == 8), Y, xv, out);
+static void run_gather(const LevelDev& d, const R* Y, const R* xv, R* out, cudaStream_t s,
+                       const Dots<R>* dots = nullptr) {
+  const MarchPlan mp = march_plan(d, sizeof(R) == 8);
+  const unsigned nb = nblocks(d.Nn, NODE_THREADS);
+  if (dots && dots->k <= 8) {
+    const unsigned rb = nb < RED_BLOCKS_MAX ? nb : RED_BLOCKS_MAX;
+    if (dots->k <= 4)
+      k_gather_dots<R, 4><<<rb, NODE_THREADS, 0, s>>>(d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
+                                                      dots->partial, dots->out, red_ticket(dots->partial));
+    else
+      k_gather_dots<R, 8><<<rb, NODE_THREADS, 0, s>>>(d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
+                                                      dots->partial, dots->out, red_ticket(dots->partial));
+    return;
+  }
+  k_gather_march<R, MODE><<<nb, NODE_THREADS, 0, s>>>(d, mp, Y, xv, out);
+  if (dots) vmdot(5 * d.Nn, dots->k, dots->V, dots->ld, (const R*)out, dots->out, dots->partial, s);
 }
 
 template <typename R>
@@ -446,16 +467,16 @@ void op_residual(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* 
 
 template <typename R>
 void op_jvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
-            const R* v, R* out, R* Y, cudaStream_t s) {
+            const R* v, R* out, R* Y, cudaStream_t s, const Dots<R>* dots) {
   run_march<R, march::JVP>(d, c, x, gam, src, nullptr, v, Y, s);
-  run_gather<R, G_LIN>(d, Y, v, out, s);
+  run_gather<R, G_LIN>(d, Y, v, out, s, dots);
 }
 
 template <typename R>
 void op_jtvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
-             const R* w, R* out, R* Y, cudaStream_t s) {
+             const R* w, R* out, R* Y, cudaStream_t s, const Dots<R>* dots) {
   run_march<R, march::JTVP>(d, c, x, gam, src, nullptr, w, Y, s);
-  run_gather<R, G_LIN>(d, Y, w, out, s);
+  run_gather<R, G_LIN>(d, Y, w, out, s, dots);
 }
 
 void op_linearize(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
@@ -465,16 +486,16 @@ void op_linearize(const LevelDev& d, const ElemConst<double>& c, const double* x
 
 void op_jvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
                    const double* src, const double* cache, const double* v, double* out, double* Y,
-                   cudaStream_t s) {
+                   cudaStream_t s, const Dots<double>* dots) {
   run_march<double, march::JVP_LIN>(d, c, x, gam, src, cache, v, Y, s);
-  run_gather<double, G_LIN>(d, Y, v, out, s);
+  run_gather<double, G_LIN>(d, Y, v, out, s, dots);
 }
 
 void op_jtvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
                     const double* src, const double* cache, const double* w, double* out, double* Y,
-                    cudaStream_t s) {
+                    cudaStream_t s, const Dots<double>* dots) {
   run_march<double, march::JTVP_LIN>(d, c, x, gam, src, cache, w, Y, s);
-  run_gather<double, G_LIN>(d, Y, w, out, s);
+  run_gather<double, G_LIN>(d, Y, w, out, s, dots);
 }
 
 template <typename R>
@@ -541,12 +562,12 @@ void op_objective_grad(const LevelDev& d, double* g, cudaStream_t s) {
 
 template <typename R>
 void op_restrict(const LevelDev& fine, const R* rf, const LevelDev& coarse, R* rc, cudaStream_t s) {
-  k_restrict<R><<<nblocks(coarse.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(fine, rf, coarse, rc);
+  k_restrict<R><<<dim3(nblocks(coarse.Nn, NODE_THREADS), NF), NODE_THREADS, 0, s>>>(fine, rf, coarse, rc);
 }
 template <typename R>
 void op_prolong_add(const LevelDev& coarse, const R* zc, const LevelDev& fine, R* zf,
                     cudaStream_t s) {
-  k_prolong_add<R><<<nblocks(fine.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(coarse, zc, fine, zf);
+  k_prolong_add<R><<<dim3(nblocks(fine.Nn, NODE_THREADS), NF), NODE_THREADS, 0, s>>>(coarse, zc, fine, zf);
 }
 template <typename R>
 void op_inject(const LevelDev& fine, const R* xf, const LevelDev& coarse, R* xc, cudaStream_t s) {
@@ -562,9 +583,9 @@ void op_coarsen_elem(const LevelDev& fine, const R* gf, const LevelDev& coarse, 
   template void op_residual<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*,        \
                                const R*, R*, R*, cudaStream_t);                                 \
   template void op_jvp<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*, const R*,   \
-                          const R*, R*, R*, cudaStream_t);                                      \
+                          const R*, R*, R*, cudaStream_t, const Dots<R>*);                      \
   template void op_jtvp<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*, const R*,  \
-                           const R*, R*, R*, cudaStream_t);                                     \
+                           const R*, R*, R*, cudaStream_t, const Dots<R>*);                     \
   template void op_diag<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*, const R*,  \
                            R*, R*, cudaStream_t);                                               \
   template void op_assemble<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*,        \

@@ -60,4 +60,17 @@ __device__ __forceinline__ double fold_partials(int nb, const double* partial) {
   return block_fold<MAX, THREADS>(v);
 }
 
+// out[q] = the sum of partial[q * nb ...] for q < cnt (or its square root), a warp per
+// value, in a fixed order.
+__device__ __forceinline__ void fold_values(int cnt, int nb, const double* partial, double* out,
+                                            int take_sqrt = 0) {
+  const int lane = threadIdx.x & 31;
+  for (int q = threadIdx.x >> 5; q < cnt; q += blockDim.x >> 5) {
+    double v = 0.0;
+    for (int b = lane; b < nb; b += 32) v += __ldcg(partial + (long long)q * nb + b);
+    v = warp_fold<false>(v);
+    if (lane == 0) out[q] = take_sqrt ? sqrt(v > 0.0 ? v : 0.0) : v;
+  }
+}
+
 }  // namespace nc

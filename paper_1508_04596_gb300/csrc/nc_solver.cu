@@ -28,12 +28,6 @@ using namespace nc;
 
 namespace {
 
-constexpr int LDH = MAX_RESTART + 1;            // leading dimension of device Hessenbergs
-constexpr int HD_Y = LDH * LDH;                   // y, then g, then the rotations
-constexpr int HD_BETA = HD_Y + 4 * LDH;           // scalar slots
-constexpr int HD_SIG2 = HD_BETA + 8;              // squared norms of the smoother basis
-constexpr int HD_SIZE = HD_SIG2 + LDH;
-
 template <typename R> LevelBuf<R>& buf(Level& L);
 template <> LevelBuf<double>& buf<double>(Level& L) { return L.f64; }
 template <> LevelBuf<float>& buf<float>(Level& L) { return L.f32; }
@@ -47,105 +41,40 @@ nc_status alloc(nc_ctx* ctx, R** p, long long n) {
   return cuda_check(ctx, cudaMalloc((void**)p, sizeof(R) * (size_t)n), "cudaMalloc");
 }
 
-// Least squares of the smoother's Arnoldi process, on the device.  Column j of
-// Hd holds the raw dots g_ij = <v_i, w_j> (i <= j) of the unnormalised basis
-// v_i (squared norms sig2_i in Hd[HD_SIG2..]), built so that
-//   A D^-1 v_j = sum_i g_ij / sig2_i v_i + sigma_j v_{j+1}.
-// With q_i = v_i / sigma_i this is the usual Arnoldi relation with the
-// Hessenberg entries H_ij = g_ij / (sigma_i sigma_j), H_{j+1,j} = sigma_{j+1},
-// and beta = sigma_0.  Solve min || beta e1 - H y || by Givens rotations (in
-// place), then store the coefficients of the correction on the raw basis,
-// y_j / sigma_j -> Hd[HD_Y + j].  A vanishing norm or pivot (an exhausted
-// Krylov space) contributes zero.  One warp stages the k columns and the norms
-// in shared memory, then one thread solves there: the elimination is a chain of
-// dependent operations, and in shared memory each costs tens of cycles instead
-// of a round trip to L2.
-constexpr int LS_THREADS = 32;
-__global__ void __launch_bounds__(LS_THREADS) k_small_ls(double* Hd_g, int k) {
-  __shared__ double Hd[HD_SIZE];
-  for (int t = threadIdx.x; t < k * LDH; t += LS_THREADS) Hd[t] = Hd_g[t];
-  for (int t = threadIdx.x; t <= k; t += LS_THREADS) Hd[HD_SIG2 + t] = Hd_g[HD_SIG2 + t];
-  __syncwarp();
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double* g = Hd + HD_Y + LDH;  // right-hand side, k + 1 entries
-  const double* sig2 = Hd + HD_SIG2;
-  auto inv_sig = [&](int i) {
-    const double s2 = sig2[i];
-    return (s2 > 0.0 && s2 < 1e300) ? 1.0 / sqrt(s2) : 0.0;
-  };
-  const double beta = sqrt(fmax(sig2[0], 0.0));
-  Hd[HD_BETA] = beta;
-  for (int i = 0; i <= k; ++i) g[i] = 0.0;
-  g[0] = (beta > 0.0 && beta < 1e300) ? beta : 0.0;
-  for (int j = 0; j < k; ++j) {  // raw dots -> normalised Hessenberg
-    double* hj = Hd + j * LDH;
-    const double ij = inv_sig(j);
-    for (int i = 0; i <= j; ++i) hj[i] *= inv_sig(i) * ij;
-    hj[j + 1] = (ij > 0.0) ? sqrt(fmax(sig2[j + 1], 0.0)) : 0.0;
-  }
-  double rmax = 0.0;
-  for (int j = 0; j < k; ++j) {
-    double* hj = Hd + j * LDH;
-    // apply the previous rotations (kept after g) to column j
-    for (int q = 0; q < j; ++q) {
-      const double c = Hd[HD_Y + 2 * LDH + 2 * q], s = Hd[HD_Y + 2 * LDH + 2 * q + 1];
-      const double t1 = hj[q], t2 = hj[q + 1];
-      hj[q] = c * t1 + s * t2;
-      hj[q + 1] = -s * t1 + c * t2;
-    }
-    const double a = hj[j], b = hj[j + 1];
-    const double r = hypot(a, b);
-    const double c = r > 0.0 ? a / r : 1.0, s = r > 0.0 ? b / r : 0.0;
-    Hd[HD_Y + 2 * LDH + 2 * j] = c;
-    Hd[HD_Y + 2 * LDH + 2 * j + 1] = s;
-    hj[j] = r;
-    hj[j + 1] = 0.0;
-    const double g1 = g[j], g2 = g[j + 1];
-    g[j] = c * g1 + s * g2;
-    g[j + 1] = -s * g1 + c * g2;
-    rmax = fmax(rmax, fabs(r));
-  }
-  for (int j = k - 1; j >= 0; --j) {
-    double acc = g[j];
-    for (int q = j + 1; q < k; ++q) acc -= Hd[j + q * LDH] * Hd[HD_Y + q];
-    const double d = Hd[j + j * LDH];
-    Hd[HD_Y + j] = (fabs(d) > 1e-14 * rmax && isfinite(acc)) ? acc / d : 0.0;
-  }
-  for (int j = 0; j < k; ++j) Hd_g[HD_Y + j] = Hd[HD_Y + j] * inv_sig(j);
-  Hd_g[HD_BETA] = Hd[HD_BETA];
-}
-
 // ------------------------------------------------------------------ level operators
 template <typename R>
-void level_apply(nc_ctx* ctx, int l, bool tr, const R* v, R* out, cudaStream_t s) {
+void level_apply(nc_ctx* ctx, int l, bool tr, const R* v, R* out, cudaStream_t s,
+                 const Dots<R>* dots = nullptr) {
   Level& L = ctx->lv[l];
   LevelBuf<R>& B = buf<R>(L);
   if (B.use_gst) {  // assembled or Galerkin operator
     op_stencil<R>(L.d, B.gst, tr, v, out, s);
+    if (dots)
+      vmdot(5 * L.d.Nn, dots->k, dots->V, dots->ld, (const R*)out, dots->out, dots->partial, s);
     return;
   }
   if constexpr (std::is_same<R, double>::value) {
     if (B.lin) {  // FP64 levels: products from the linearisation cache
       if (tr)
-        op_jtvp_cached(L.d, L.c64, B.x, B.gam, B.src, B.lin, v, out, ctx->Y, s);
+        op_jtvp_cached(L.d, L.c64, B.x, B.gam, B.src, B.lin, v, out, ctx->Y, s, dots);
       else
-        op_jvp_cached(L.d, L.c64, B.x, B.gam, B.src, B.lin, v, out, ctx->Y, s);
+        op_jvp_cached(L.d, L.c64, B.x, B.gam, B.src, B.lin, v, out, ctx->Y, s, dots);
       return;
     }
   }
   if (tr)
-    op_jtvp<R>(L.d, cst<R>(L), B.x, B.gam, B.src, v, out, (R*)ctx->Y, s);
+    op_jtvp<R>(L.d, cst<R>(L), B.x, B.gam, B.src, v, out, (R*)ctx->Y, s, dots);
   else
-    op_jvp<R>(L.d, cst<R>(L), B.x, B.gam, B.src, v, out, (R*)ctx->Y, s);
+    op_jvp<R>(L.d, cst<R>(L), B.x, B.gam, B.src, v, out, (R*)ctx->Y, s, dots);
 }
 
 // Right Jacobi-preconditioned GMRES(k) on level l:  z += D^-1 V y  approximately
 // solving A z = b.  With zero_init the initial guess is 0.  The basis is kept
 // unnormalised (each new vector is divided by the previous vector's norm, so
-// magnitudes stay bounded); k_small_ls turns the raw dots and norms into the
-// normalised Hessenberg.  Per Arnoldi step: the operator on t = D^-1 v_j, one
-// multi-dot, and one pass that orthogonalises, rescales, forms the next t and
-// the new norm.
+// magnitudes stay bounded); small_ls turns the raw dots and norms into the
+// normalised Hessenberg.  Per Arnoldi step three kernels: the element product of
+// t = D^-1 v_j, the gather of w with its dots, and one pass that orthogonalises,
+// rescales, forms the next t and the new norm.
 template <typename R>
 void smooth(nc_ctx* ctx, int l, bool tr, int k, bool zero_init, cudaStream_t s) {
   Level& L = ctx->lv[l];
@@ -163,13 +92,13 @@ void smooth(nc_ctx* ctx, int l, bool tr, int k, bool zero_init, cudaStream_t s) 
   }
   for (int j = 0; j < k; ++j) {
     R* w = V + (j + 1) * ld;
-    level_apply<R>(ctx, l, tr, B.t, w, s);
     double* hcol = Hd + j * LDH;
-    vmdot(n, j + 1, (const R*)V, ld, (const R*)w, hcol, ctx->partial, s);
+    const Dots<R> dots{j + 1, V, ld, hcol, ctx->partial};
+    level_apply<R>(ctx, l, tr, B.t, w, s, &dots);
     varnoldi_update(n, j + 1, (const R*)V, ld, hcol, Hd + HD_SIG2, (const R*)B.diag, w,
                     j + 1 < k ? B.t : (R*)nullptr, Hd + HD_SIG2 + j + 1, ctx->partial, s);
   }
-  k_small_ls<<<1, LS_THREADS, 0, s>>>(Hd, k);
+  small_ls(Hd, k, s);
   // z (+)= D^-1 (V y)
   vcombine(n, k, (const R*)V, ld, Hd + HD_Y, (const R*)B.diag, B.z, !zero_init, s);
 }
