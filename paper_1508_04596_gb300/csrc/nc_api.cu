@@ -59,6 +59,24 @@ bool valid_bcs(const nc_params& p, const nc_bcs* b, std::string& why) {
   return true;
 }
 
+template <typename R>
+R* assembly_store(nc_ctx* ctx, long long E) {
+  const size_t need = sizeof(R) * (size_t)LIN_SLOTS * (size_t)E;
+  if (ctx->asm_lin_bytes < need) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, need) != cudaSuccess) {
+      cudaGetLastError();
+      return nullptr;
+    }
+    cudaFree(ctx->asm_lin);
+    ctx->asm_lin = p;
+    ctx->asm_lin_bytes = need;
+  }
+  return (R*)ctx->asm_lin;
+}
+template double* assembly_store<double>(nc_ctx*, long long);
+template float* assembly_store<float>(nc_ctx*, long long);
+
 }  // namespace nc
 
 namespace {
@@ -376,7 +394,7 @@ nc_status nc_linearize(nc_ctx* ctx, const double* x, const double* gam, void* st
   if (!ctx->pub_lin &&
       (st = dev_alloc(ctx, &ctx->pub_lin, (long long)LIN_SLOTS * L.d.E)) != NC_OK)
     return st;
-  op_linearize(L.d, L.c64, x, gam, L.f64.src, ctx->pub_lin, (cudaStream_t)stream);
+  op_linearize<double>(L.d, L.c64, x, gam, L.f64.src, ctx->pub_lin, (cudaStream_t)stream);
   ctx->pub_x = x;
   ctx->pub_gam = gam;
   return cuda_check(ctx, cudaGetLastError(), "nc_linearize");
@@ -407,17 +425,16 @@ nc_status nc_assemble(nc_ctx* ctx, const void* x, const void* gam, void* S, int 
   const Level& L = ctx->lv[0];
   cudaStream_t s = (cudaStream_t)stream;
   if (prec == NC_FP64) {
-    nc_status st;
-    if (!ctx->asm_lin &&
-        (st = dev_alloc(ctx, &ctx->asm_lin, (long long)LIN_SLOTS * L.d.E)) != NC_OK)
-      return st;
-    op_linearize(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src,
-                         ctx->asm_lin, s);
-    op_assemble<double>(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src,
-                        ctx->asm_lin, (double*)S, ctx->Y, s);
+    double* lin = assembly_store<double>(ctx, L.d.E);
+    if (!lin) return set_err(ctx, NC_ERR_OOM, "nc_assemble: linearisation store");
+    op_linearize<double>(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src, lin, s);
+    op_assemble<double>(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src, lin, (double*)S,
+                        ctx->Y, s);
   } else {
-    op_assemble<float>(L.d, L.c32, (const float*)x, (const float*)gam, L.f32.src, nullptr,
-                       (float*)S, (float*)ctx->Y, s);
+    float* lin = assembly_store<float>(ctx, L.d.E);
+    if (lin) op_linearize<float>(L.d, L.c32, (const float*)x, (const float*)gam, L.f32.src, lin, s);
+    op_assemble<float>(L.d, L.c32, (const float*)x, (const float*)gam, L.f32.src, lin, (float*)S,
+                       (float*)ctx->Y, s);
   }
   return cuda_check(ctx, cudaGetLastError(), "nc_assemble");
 }

@@ -132,7 +132,8 @@ struct nc_ctx {
   cudaStream_t cap = nullptr; // stream used to capture the V-cycle graph
   double* filt[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // filter CG
   double* pub_lin = nullptr;  // linearisation of nc_linearize (level 0, FP64)
-  double* asm_lin = nullptr;  // linearisation used by nc_assemble (level 0, FP64)
+  void* asm_lin = nullptr;    // linearisation store of an assembly (FP64: nc_assemble; FP32: any level)
+  size_t asm_lin_bytes = 0;
   double* ref_lin = nullptr;  // linearisation of the mixed adjoint's FP64 refinement (level 0)
   void* mma_ws = nullptr;     // coefficient workspace of nc_mma_update
   size_t mma_ws_bytes = 0;
@@ -188,8 +189,9 @@ void op_jtvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam,
              const R* w, R* out, R* Y, cudaStream_t s, const Dots<R>* dots = nullptr);
 // linearisation cache (LIN_SLOTS values per element, slot-major) and the
 // products that read it
-void op_linearize(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam, const double* src,
-                  double* cache, cudaStream_t s);
+template <typename R>
+void op_linearize(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
+                  R* cache, cudaStream_t s);
 void op_jvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
                    const double* src, const double* cache, const double* v, double* out, double* Y, cudaStream_t s, const Dots<double>* dots = nullptr);
 void op_jtvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
@@ -294,12 +296,17 @@ void vcombine(long long n, int k, const R* X, long long ld, const double* coef, 
 // coarse operators.  S holds 675 * Nn entries, S[((o*5 + f)*5 + g)*Nn + n] couples
 // (n, f) to (n + offset o, g), o = (dx+1) + 3 (dy+1) + 9 (dz+1)
 constexpr int STENCIL_VALUES = 675;
-// S = J(x, gamma) of one level, from its element Jacobians (nc_kernels.cu): 40
-// element products with unit directions (reading `cache` when not null), each
-// summed into S per node; Dirichlet rows identity, Dirichlet columns zero.
+// S = J(x, gamma) of one level, from its element Jacobians: from the linearisation
+// store `cache` (nc_assemble.cuh), or without one by 40 element products with unit
+// directions, each summed into S per node; Dirichlet rows identity, Dirichlet columns
+// zero.
 template <typename R>
 void op_assemble(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
                  const R* cache, R* S, R* Y, cudaStream_t s);
+// The context's linearisation store for assemblies, LIN_SLOTS * E values of R; null if
+// there is no memory for it (nc_api.cu).
+template <typename R>
+R* assembly_store(nc_ctx* ctx, long long E);
 template <typename R>
 void op_stencil(const LevelDev& d, const R* S, bool tr, const R* v, R* out, cudaStream_t s);
 template <typename R>

@@ -2,11 +2,12 @@
 //
 // Assembly is colouring-free and deterministic: the element kernels write sums per
 // node and element layer (the marching operators, nc_march.cuh) or 40 rows per element
-// (diag(J) and the assembled Jacobian) to a scratch array, and one thread per node
-// adds those of its node in a fixed order.  No atomics, so results are bitwise
-// reproducible.
+// (diag(J)) to a scratch array, and one thread per node adds those of its node in a
+// fixed order; the assembled Jacobian takes one contribution per entry and launch
+// (nc_assemble.cuh).  Results are bitwise reproducible.
 #include <type_traits>
 
+#include "nc_assemble.cuh"
 #include "nc_element_f2.cuh"
 #include "nc_internal.cuh"
 #include "nc_march.cuh"
@@ -72,7 +73,8 @@ __device__ __forceinline__ void store_elem(long long E, long long e, const R out
 
 // Column col = 5 b + g of every element Jacobian: the element product with the
 // unit direction on unknown g of local node b, or zero where that unknown is
-// Dirichlet (Dirichlet columns are removed).  Re-interpolates the state.
+// Dirichlet (Dirichlet columns are removed).  Re-interpolates the state: the way
+// to assemble where there is no memory for a linearisation store.
 template <typename R>
 __global__ void __launch_bounds__(ELEM_THREADS) k_elem_column(
     LevelDev d, ElemConst<R> c, const R* __restrict__ x, const R* __restrict__ gam,
@@ -96,28 +98,6 @@ __global__ void __launch_bounds__(ELEM_THREADS) k_elem_column(
     for (int a = 0; a < 8; ++a) ve[f][a] = (f == g && a == b) ? R(1) : R(0);
   load_elem(d, x, e, xe, false);
   elem_jvp<R>(xe, ve, gam[e], src ? src[e] : R(0), c, out);
-  store_elem(d.E, e, out, Y);
-}
-
-// The same column from the linearisation store with the unit direction written
-// out (elem_column_lin): unknown G, local node b.
-template <typename R, int G>
-__global__ void __launch_bounds__(ELEM_THREADS) k_elem_column_lin(
-    LevelDev d, ElemConst<R> c, const R* __restrict__ x, const R* __restrict__ gam,
-    const R* __restrict__ src, const R* __restrict__ cache, int b, R* Y) {
-  const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (e >= d.E) return;
-  R out[5][8];
-  const long long nb = elem_node(d, e, b);
-  if ((d.flag[nb] >> G) & 1) {
-#pragma unroll
-    for (int f = 0; f < 5; ++f)
-#pragma unroll
-      for (int a = 0; a < 8; ++a) out[f][a] = R(0);
-  } else {
-    const R ub = G < 3 ? x[G * d.Nn + nb] : R(0);
-    elem_column_lin<R, G>(cache + e, d.E, ub, b, gam[e], src ? src[e] : R(0), c, out);
-  }
   store_elem(d.E, e, out, Y);
 }
 
@@ -479,9 +459,10 @@ void op_jtvp(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam,
   run_gather<R, G_LIN>(d, Y, w, out, s, dots);
 }
 
-void op_linearize(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
-                  const double* src, double* cache, cudaStream_t s) {
-  run_march<double, march::LINEARIZE>(d, c, x, gam, src, nullptr, nullptr, cache, s);
+template <typename R>
+void op_linearize(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
+                  R* cache, cudaStream_t s) {
+  run_march<R, march::LINEARIZE>(d, c, x, gam, src, nullptr, nullptr, cache, s);
 }
 
 void op_jvp_cached(const LevelDev& d, const ElemConst<double>& c, const double* x, const double* gam,
@@ -509,20 +490,13 @@ template <typename R>
 void op_assemble(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
                  const R* cache, R* S, R* Y, cudaStream_t s) {
   cudaMemsetAsync(S, 0, sizeof(R) * (size_t)STENCIL_VALUES * (size_t)d.Nn, s);
-  const unsigned eb = nblocks(d.E, ELEM_THREADS);
-  for (int col = 0; col < 40; ++col) {
-    const int b = col / 5;
-    if (cache) {
-      switch (col % 5) {
-        case 0: k_elem_column_lin<R, 0><<<eb, ELEM_THREADS, 0, s>>>(d, c, x, gam, src, cache, b, Y); break;
-        case 1: k_elem_column_lin<R, 1><<<eb, ELEM_THREADS, 0, s>>>(d, c, x, gam, src, cache, b, Y); break;
-        case 2: k_elem_column_lin<R, 2><<<eb, ELEM_THREADS, 0, s>>>(d, c, x, gam, src, cache, b, Y); break;
-        case 3: k_elem_column_lin<R, 3><<<eb, ELEM_THREADS, 0, s>>>(d, c, x, gam, src, cache, b, Y); break;
-        default: k_elem_column_lin<R, 4><<<eb, ELEM_THREADS, 0, s>>>(d, c, x, gam, src, cache, b, Y);
-      }
-    } else
-      k_elem_column<R><<<eb, ELEM_THREADS, 0, s>>>(d, c, x, gam, src, col, Y);
-    k_assemble_column<R><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, col, Y, S);
+  if (cache) {
+    for (int a = 0; a < 8; ++a) rows::k_assemble_rows<R><<<nblocks(d.E, 128), 128, 0, s>>>(d, c, rows::row_const(c, a), x, cache, a, S);
+  } else {
+    for (int col = 0; col < 40; ++col) {
+      k_elem_column<R><<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src, col, Y);
+      k_assemble_column<R><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, col, Y, S);
+    }
   }
   stencil_dirichlet<R>(d, S, s);
 }
@@ -588,6 +562,8 @@ void op_coarsen_elem(const LevelDev& fine, const R* gf, const LevelDev& coarse, 
                            const R*, R*, R*, cudaStream_t, const Dots<R>*);                     \
   template void op_diag<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*, const R*,  \
                            R*, R*, cudaStream_t);                                               \
+  template void op_linearize<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*,       \
+                                const R*, R*, cudaStream_t);                                    \
   template void op_assemble<R>(const LevelDev&, const ElemConst<R>&, const R*, const R*,        \
                                const R*, const R*, R*, R*, cudaStream_t);                       \
   template void op_impose<R>(const LevelDev&, R*, cudaStream_t);                                \

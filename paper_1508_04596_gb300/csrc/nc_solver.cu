@@ -214,15 +214,16 @@ nc_status linearize(nc_ctx* ctx, int nlev, const double* x, const double* gam, c
       galerkin_build<R>(ctx, l, s);
       op_stencil_diag<R>(L.d, B.gst, B.diag, s);
     } else if (assembled) {
-      if constexpr (std::is_same<R, double>::value)
-        if (B.lin) op_linearize(L.d, L.c64, B.x, B.gam, B.src, B.lin, s);
-      op_assemble<R>(L.d, cst<R>(L), B.x, B.gam, B.src, B.lin, B.gst, (R*)ctx->Y, s);
+      R* lin = B.lin;
+      if (!lin && sizeof(R) == sizeof(float)) lin = assembly_store<R>(ctx, L.d.E);
+      if (lin) op_linearize<R>(L.d, cst<R>(L), B.x, B.gam, B.src, lin, s);
+      op_assemble<R>(L.d, cst<R>(L), B.x, B.gam, B.src, lin, B.gst, (R*)ctx->Y, s);
       op_stencil_diag<R>(L.d, B.gst, B.diag, s);
     } else {
       // diag(J^T) = diag(J)
       op_diag<R>(L.d, cst<R>(L), B.x, B.gam, B.src, B.diag, (R*)ctx->Y, s);
       if constexpr (std::is_same<R, double>::value)
-        if (B.lin) op_linearize(L.d, L.c64, B.x, B.gam, B.src, B.lin, s);
+        if (B.lin) op_linearize<double>(L.d, L.c64, B.x, B.gam, B.src, B.lin, s);
     }
     if (l == nlev - 1 && coarse_dense_dofs(L) <= COARSE_DENSE_MAX) {
       const nc_status st = B.use_gst ? coarse_setup_stencil<R>(ctx, L, B.gst, &B.inv, s)
@@ -852,7 +853,7 @@ nc_status nc_adjoint_solve(nc_ctx* ctx, const double* x, const double* gam, cons
       if (!mixed) {
         store = L.f64.lin;
       } else if (refine_store(ctx, L.d.E)) {
-        op_linearize(L.d, L.c64, x, gam, ctx->src64, ctx->ref_lin, s);
+        op_linearize<double>(L.d, L.c64, x, gam, ctx->src64, ctx->ref_lin, s);
         store = ctx->ref_lin;
       }
     }
