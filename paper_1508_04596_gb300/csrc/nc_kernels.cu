@@ -207,9 +207,12 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather(LevelDev d, const R* __
 // Gather of the marching kernels' sums.
 template <typename R, int MODE>
 __global__ void __launch_bounds__(NODE_THREADS) k_gather_march(LevelDev d, MarchPlan mp,
-                                                               const R* __restrict__ Y,
-                                                               const R* __restrict__ xv,
+                                                               const R* __restrict__ Y_,
+                                                               const R* __restrict__ xv_,
                                                                R* __restrict__ out) {
+  chained();
+  const R* const Y = fresh(Y_);
+  const R* const xv = fresh(xv_);
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= d.Nn) return;
   int i, j, k;
@@ -225,12 +228,16 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_march(LevelDev d, March
 // Two accumulators per column; partials fold in the last block.
 template <typename R, int KB>
 __global__ void __launch_bounds__(NODE_THREADS) k_gather_dots(LevelDev d, MarchPlan mp,
-                                                              const R* __restrict__ Y,
-                                                              const R* __restrict__ xv,
+                                                              const R* __restrict__ Y_,
+                                                              const R* __restrict__ xv_,
                                                               R* __restrict__ out, int k,
-                                                              const R* __restrict__ V, long long ld,
+                                                              const R* __restrict__ V_, long long ld,
                                                               double* partial, double* dots,
                                                               unsigned* ticket) {
+  chained();
+  const R* const Y = fresh(Y_);
+  const R* const xv = fresh(xv_);
+  const R* const V = fresh(V_);
   R a0[KB], a1[KB];
 #pragma unroll
   for (int q = 0; q < KB; ++q) a0[q] = a1[q] = R(0);
@@ -411,11 +418,11 @@ static void run_march(const LevelDev& d, const ElemConst<R>& c, const R* x, cons
   const MarchPlan mp = march_plan(d, sizeof(R) == 8);
   if constexpr (march::Traits<K>::TEST) {
     if (mp.split) {
-      march::k_split<R, K><<<(unsigned)mp.nchunk, 128, 0, s>>>(d, c, mp, x, gam, src, cache, v, out);
+      launch(march::k_split<R, K>, (unsigned)mp.nchunk, 128, 0, s, d, c, mp, x, gam, src, cache, v, out);
       return;
     }
   }
-  march::k_march<R, K><<<nblocks(mp.warps(), march::WARPS), 32 * march::WARPS, 0, s>>>(
+  launch(march::k_march<R, K>, nblocks(mp.warps(), march::WARPS), 32 * march::WARPS, 0, s, 
       d, c, mp, x, gam, src, cache, v, out);
 }
 
@@ -427,14 +434,14 @@ static void run_gather(const LevelDev& d, const R* Y, const R* xv, R* out, cudaS
   if (dots && dots->k <= 8) {
     const unsigned rb = nb < RED_BLOCKS_MAX ? nb : RED_BLOCKS_MAX;
     if (dots->k <= 4)
-      k_gather_dots<R, 4><<<rb, NODE_THREADS, 0, s>>>(d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
+      launch(k_gather_dots<R, 4>, rb, NODE_THREADS, 0, s, d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
                                                       dots->partial, dots->out, red_ticket(dots->partial));
     else
-      k_gather_dots<R, 8><<<rb, NODE_THREADS, 0, s>>>(d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
+      launch(k_gather_dots<R, 8>, rb, NODE_THREADS, 0, s, d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
                                                       dots->partial, dots->out, red_ticket(dots->partial));
     return;
   }
-  k_gather_march<R, MODE><<<nb, NODE_THREADS, 0, s>>>(d, mp, Y, xv, out);
+  launch(k_gather_march<R, MODE>, nb, NODE_THREADS, 0, s, d, mp, Y, xv, out);
   if (dots) vmdot(5 * d.Nn, dots->k, dots->V, dots->ld, (const R*)out, dots->out, dots->partial, s);
 }
 

@@ -119,11 +119,15 @@ template <typename R, int K> struct Stage {
 
 template <typename R, int K>
 __global__ void __launch_bounds__(WARPS * 32, 2) k_march(LevelDev d, ElemConst<R> c, MarchPlan mp,
-                                                        const R* __restrict__ x,
+                                                        const R* __restrict__ x_,
                                                         const R* __restrict__ gam,
                                                         const R* __restrict__ srcs,
-                                                        const R* cache,
-                                                        const R* __restrict__ v, R* out) {
+                                                        const R* cache_,
+                                                        const R* __restrict__ v_, R* out) {
+  chained();
+  const R* const x = fresh(x_);
+  const R* const cache = fresh(cache_);
+  const R* const v = fresh(v_);
   typedef Traits<K> TR;
   typedef typename Stage<R, K>::T T;
   typedef PR<R> P;
@@ -554,11 +558,11 @@ __device__ __forceinline__ void node_sums(const LevelDev& d, const MarchPlan& mp
       const long long w = chunk + (mp.flat ? 0 : (run - t) * mp.nchunk);
       const R* p = Y + (w * rows + (t ? mp.rc : r)) * ROW_LEN + z * 160 + lane;
 #pragma unroll
-      for (int f = 0; f < 5; ++f) acc[f] += p[f * 32];
+      for (int f = 0; f < 5; ++f) acc[f] += __ldcg(p + f * 32);  // read once
       if (lane == 0 && i > 0) {  // the left element's share, in lane 31 of the chunk before
         p += mp.stride - (long long)rows * ROW_LEN;
 #pragma unroll
-        for (int f = 0; f < 5; ++f) acc[f] += p[f * 32];
+        for (int f = 0; f < 5; ++f) acc[f] += __ldcg(p + f * 32);  // read once
       }
     }
   }

@@ -260,9 +260,13 @@ __device__ __forceinline__ void split_chunk(const LevelDev& d, const ElemConst<R
 
 template <typename R, int K>
 __global__ void __launch_bounds__(128) k_split(LevelDev d, ElemConst<R> c, MarchPlan mp,
-                                               const R* __restrict__ x, const R* __restrict__ gam,
-                                               const R* __restrict__ srcs, const R* __restrict__ cache,
-                                               const R* __restrict__ v, R* Y) {
+                                               const R* __restrict__ x_, const R* __restrict__ gam,
+                                               const R* __restrict__ srcs, const R* __restrict__ cache_,
+                                               const R* __restrict__ v_, R* Y) {
+  chained();
+  const R* const x = fresh(x_);
+  const R* const cache = fresh(cache_);
+  const R* const v = fresh(v_);
   __shared__ QuadSums<R> sums;
   split_chunk<R, K, false>(d, c, mp, blockIdx.x, threadIdx.x >> 5, x, gam, srcs, cache, v, Y, sums,
                            [] { __syncthreads(); });
