@@ -13,6 +13,7 @@
 // order (nc_reduce.cuh; a second kernel for that cost 3.7 us per reduction, of 9.7 us
 // in all on a vector of 10^5).  Results are bitwise reproducible from run to run.
 #include <cstdint>
+#include <type_traits>
 
 #include "nc_internal.cuh"
 #include "nc_reduce.cuh"
@@ -189,78 +190,113 @@ __device__ __forceinline__ void finish(int cnt, const double* partial, double* o
   if (last_block(ticket)) fold_values(cnt, gridDim.x, partial, out, take_sqrt);
 }
 
-// partial[i * nb + b] = sum over block b's chunks of X_i . y for i < k, and with
-// self also partial[k * nb + b] = y . y  (per-thread sums in R, partials in double)
+// One pass of a multi-dot over y: NC columns from X on, and with SELF y . y.  All
+// columns' packets of a chunk are loaded before any is used: with a test of the
+// column count around each load one was in flight at a time (FP64, 10 columns of 10.7M:
+// 315 us against 225 now and 176 at the FP64 pipe's rate; the whole Gram-Schmidt step
+// 1063 -> 868 us, FP32 401 -> 369).  FP32 sums go to two accumulators per column.
+template <typename R, bool VEC, int NC, bool SELF>
+__device__ __forceinline__ void mdot_pass(long long n, const R* __restrict__ X, long long ld,
+                                          const R* __restrict__ y, double* partial, double* partial_self) {
+  constexpr int CH = 16 / sizeof(R), NA = sizeof(R) == 4 ? 2 : 1;
+  struct __align__(16) Pk {
+    R v[CH];
+  };
+  const long long nc = n / CH;
+  const long long gid = blockIdx.x * (long long)RED_THREADS + threadIdx.x;
+  const long long gs = (long long)gridDim.x * RED_THREADS;
+  auto get = [&](const R* p, long long c, R o[CH]) {
+    if (VEC) {
+      const Pk t = reinterpret_cast<const Pk*>(p)[c];
+#pragma unroll
+      for (int u = 0; u < CH; ++u) o[u] = t.v[u];
+    } else {
+#pragma unroll
+      for (int u = 0; u < CH; ++u) o[u] = p[CH * c + u];
+    }
+  };
+  R acc[NC][NA], accs = R(0);
+#pragma unroll
+  for (int q = 0; q < NC; ++q)
+#pragma unroll
+    for (int t = 0; t < NA; ++t) acc[q][t] = R(0);
+  for (long long c = gid; c < nc; c += gs) {
+    R yv[CH], xv[NC][CH];
+    get(y, c, yv);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) get(X + q * ld, c, xv[q]);
+#pragma unroll
+    for (int u = 0; u < CH; ++u) {
+      if (SELF) accs = fma(yv[u], yv[u], accs);
+#pragma unroll
+      for (int q = 0; q < NC; ++q) acc[q][u % NA] = fma(xv[q][u], yv[u], acc[q][u % NA]);
+    }
+  }
+  if (gid < n - nc * CH) {
+    const long long i = nc * CH + gid;
+    const R yt = y[i];
+    if (SELF) accs = fma(yt, yt, accs);
+#pragma unroll
+    for (int q = 0; q < NC; ++q) acc[q][0] = fma(X[q * ld + i], yt, acc[q][0]);
+  }
+  R v[NC];
+#pragma unroll
+  for (int q = 0; q < NC; ++q) v[q] = NA == 2 ? acc[q][0] + acc[q][NA - 1] : acc[q][0];
+  block_values<RED_THREADS>(v, NC, partial);
+  if (SELF) {
+    const R w[1] = {accs};
+    block_values<RED_THREADS>(w, 1, partial_self);
+  }
+}
+
+// Columns of one pass over y: FP64 is bound by the FP64 pipe (one FMA per 8 bytes), FP32
+// by HBM.
+template <typename R> constexpr int mdot_cols() { return sizeof(R) == 8 ? 4 : 8; }
+
+// out[i] = X_i . y for i < k, and with self out[k] = y . y (per-thread sums in R, partials
+// in double), in passes of nearly equal numbers of columns
 template <typename R, bool VEC>
-__global__ void __launch_bounds__(RED_THREADS) k_mdot_partial(long long n, int k,
-                                                              const R* __restrict__ X, long long ld,
-                                                              const R* __restrict__ y, int self,
-                                                              double* partial, double* out,
-                                                              int take_sqrt, unsigned* ticket) {
-  constexpr int KB = sizeof(R) == 8 ? 4 : 8;  // columns per pass over y (FP64: fewer live loads)
-  const int nb = gridDim.x;
-  const long long n4 = n >> 2;
-  const long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long gs = (long long)nb * blockDim.x;
-  const int passes = k > 0 ? (k + KB - 1) / KB : 1;
-  for (int p = 0; p < passes; ++p) {
-    const int i0 = p * KB;
-    const bool do_self = self && p == 0;
-    // FP32 (HBM-bound): two chunks per iteration and two accumulators per column
-    // keep more loads in flight and shorten the FMA chains.  FP64 runs at 1/64 of
-    // the FP32 rate on this GPU, so an FP64 multi-dot is bound by its FMA count:
-    // one FMA per element, one chunk per iteration.
-    constexpr int CU = sizeof(R) == 4 ? 2 : 1;
-    R acc[KB], acc2[KB], accs = R(0);
+__global__ void __launch_bounds__(RED_THREADS, 4) k_mdot(long long n, int k, const R* __restrict__ X,
+                                                         long long ld, const R* __restrict__ y, int self,
+                                                         double* partial, double* out, int take_sqrt,
+                                                         unsigned* ticket) {
+  constexpr int KB = mdot_cols<R>();
+  const int passes = (k + KB - 1) / KB;
+  double* const ps = partial + (long long)k * gridDim.x;
+  if (k == 0) {
+    R acc[1] = {R(0)};
+    chunk_loop(n, [&](long long c) {
+      R a[4];
+      ld4<R, VEC>(y, c, a);
 #pragma unroll
-    for (int q = 0; q < KB; ++q) acc[q] = acc2[q] = R(0);
-    for (long long c0 = gid; c0 < n4; c0 += CU * gs) {
-#pragma unroll
-      for (int h = 0; h < CU; ++h) {
-        const long long c = c0 + h * gs;
-        if (c >= n4) break;
-        R yv[4];
-        ld4<R, VEC>(y, c, yv);
-        if (do_self) {
-#pragma unroll
-          for (int u = 0; u < 4; ++u) accs = fma(yv[u], yv[u], accs);
-        }
-#pragma unroll
-        for (int q = 0; q < KB; ++q) {
-          if (i0 + q < k) {
-            R xv[4];
-            ld4<R, VEC>(X + (i0 + q) * ld, c, xv);
-            if (CU == 2) {
-              acc[q] = fma(xv[0], yv[0], acc[q]);
-              acc2[q] = fma(xv[1], yv[1], acc2[q]);
-              acc[q] = fma(xv[2], yv[2], acc[q]);
-              acc2[q] = fma(xv[3], yv[3], acc2[q]);
-            } else {
-#pragma unroll
-              for (int u = 0; u < 4; ++u) acc[q] = fma(xv[u], yv[u], acc[q]);
-            }
-          }
-        }
+      for (int u = 0; u < 4; ++u) acc[0] = fma(a[u], a[u], acc[0]);
+    }, [&](long long i) { acc[0] = fma(y[i], y[i], acc[0]); });
+    block_values<RED_THREADS>(acc, 1, ps);
+  }
+  for (int p = 0, i0 = 0; p < passes; ++p) {
+    const int nc = (k - i0 + passes - p - 1) / (passes - p);
+    const R* const Xp = X + i0 * ld;
+    double* const pp = partial + (long long)i0 * gridDim.x;
+    auto pass = [&](auto c) {
+      constexpr int NC = decltype(c)::value;
+      if constexpr (NC <= KB) {
+        if (self && p == 0)
+          mdot_pass<R, VEC, NC, true>(n, Xp, ld, y, pp, ps);
+        else
+          mdot_pass<R, VEC, NC, false>(n, Xp, ld, y, pp, nullptr);
       }
+    };
+    switch (nc) {
+      case 1: pass(std::integral_constant<int, 1>()); break;
+      case 2: pass(std::integral_constant<int, 2>()); break;
+      case 3: pass(std::integral_constant<int, 3>()); break;
+      case 4: pass(std::integral_constant<int, 4>()); break;
+      case 5: pass(std::integral_constant<int, 5>()); break;
+      case 6: pass(std::integral_constant<int, 6>()); break;
+      case 7: pass(std::integral_constant<int, 7>()); break;
+      default: pass(std::integral_constant<int, 8>());
     }
-    if (gid < (n & 3)) {
-      const long long i = n4 * 4 + gid;
-      const R yt = y[i];
-      if (do_self) accs += yt * yt;
-#pragma unroll
-      for (int q = 0; q < KB; ++q)
-        if (i0 + q < k) acc[q] += X[(i0 + q) * ld + i] * yt;
-    }
-#pragma unroll
-    for (int q = 0; q < KB; ++q) {
-      if (i0 + q >= k) break;
-      const R s = block_sum(acc[q] + acc2[q]);
-      if (threadIdx.x == 0) partial[(i0 + q) * nb + blockIdx.x] = double(s);
-    }
-    if (do_self) {
-      const R s = block_sum(accs);
-      if (threadIdx.x == 0) partial[k * nb + blockIdx.x] = double(s);
-    }
+    i0 += nc;
   }
   finish(k + (self ? 1 : 0), partial, out, take_sqrt, ticket);
 }
@@ -539,10 +575,10 @@ static void mdot(long long n, int k, const R* X, long long ld, const R* y, int s
                  int take_sqrt, double* partial, cudaStream_t s) {
   const int nb = red_blocks(n);
   if ((k == 0 || mv_aligned(X, ld)) && al16(y))
-    k_mdot_partial<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, take_sqrt,
+    k_mdot<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, take_sqrt,
                                                        red_ticket(partial));
   else
-    k_mdot_partial<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, take_sqrt,
+    k_mdot<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, take_sqrt,
                                                         red_ticket(partial));
 }
 template <typename R>

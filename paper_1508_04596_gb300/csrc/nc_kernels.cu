@@ -265,12 +265,10 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_dots(LevelDev d, MarchP
         a1[q] = fma(u[1], acc[1], fma(u[3], acc[3], a1[q]));
       }
   }
+  R v[KB];
 #pragma unroll
-  for (int q = 0; q < KB; ++q)
-    if (q < k) {
-      const R t = block_fold<false, NODE_THREADS>(a0[q] + a1[q]);
-      if (threadIdx.x == 0) partial[q * gridDim.x + blockIdx.x] = double(t);
-    }
+  for (int q = 0; q < KB; ++q) v[q] = q < k ? a0[q] + a1[q] : R(0);
+  block_values<NODE_THREADS>(v, k, partial);
   if (last_block(ticket)) fold_values(k, gridDim.x, partial, dots);
 }
 

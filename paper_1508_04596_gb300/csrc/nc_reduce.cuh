@@ -33,6 +33,54 @@ __device__ __forceinline__ T block_fold(T v) {
   return v;
 }
 
+// Block sums of N values per thread (the first cnt of them) to partial[q * gridDim.x +
+// blockIdx.x].  FP32 folds by shuffles.  An FP64 addition holds a scheduler's unit for
+// 64 cycles whatever the number of active lanes, so FP64 values go through shared
+// memory and one warp adds a value's eight warps before its five shuffle steps: 12
+// additions per value and block instead of 45.
+// N <= 8.
+template <int THREADS, typename T>
+__device__ __forceinline__ T* block_buffer() {  // one for every N
+  __shared__ T sh[sizeof(T) == 8 ? 8 * THREADS : 8 * (THREADS / 32)];
+  return sh;
+}
+template <int THREADS, int N, typename T>
+__device__ __forceinline__ void block_values(const T (&v)[N], int cnt, double* partial) {
+  static_assert(N <= 8, "the buffer holds 8 values");
+  constexpr int W = THREADS / 32;
+  T* const sh = block_buffer<THREADS, T>();
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if constexpr (sizeof(T) == 8) {
+    __syncthreads();  // sh may still be read from a previous call
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (q < cnt) sh[(q * W + wid) * 32 + lane] = v[q];
+    __syncthreads();
+    for (int q = wid; q < cnt; q += W) {
+      T t = sh[q * W * 32 + lane];
+#pragma unroll
+      for (int w = 1; w < W; ++w) t += sh[(q * W + w) * 32 + lane];
+      t = warp_fold<false>(t);
+      if (lane == 0) partial[(long long)q * gridDim.x + blockIdx.x] = double(t);
+    }
+  } else {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < N; ++q)
+      if (q < cnt) {
+        const T t = warp_fold<false>(v[q]);
+        if (lane == 0) sh[wid * 8 + q] = t;
+      }
+    __syncthreads();
+    if ((int)threadIdx.x < cnt) {
+      T t = sh[threadIdx.x];
+#pragma unroll
+      for (int w = 1; w < W; ++w) t += sh[w * 8 + threadIdx.x];
+      partial[(long long)threadIdx.x * gridDim.x + blockIdx.x] = double(t);
+    }
+  }
+}
+
 // Whether the calling block is the last of its grid to get here.  Its threads then
 // see what every other block wrote before its own call.  The ticket, 0 on entry,
 // is left at 0.
