@@ -17,6 +17,7 @@
 
 #include "nc_internal.cuh"
 #include "nc_reduce.cuh"
+#include "nc_smooth.cuh"
 
 namespace nc {
 
@@ -185,9 +186,9 @@ __device__ __forceinline__ T block_sum(T v) {
 }
 
 // The last block's end of a reduction of cnt values (nc_reduce.cuh).
-__device__ __forceinline__ void finish(int cnt, const double* partial, double* out, int take_sqrt,
-                                       unsigned* ticket) {
-  if (last_block(ticket)) fold_values(cnt, gridDim.x, partial, out, take_sqrt);
+template <typename F>
+__device__ __forceinline__ void finish(int cnt, const double* partial, unsigned* ticket, F&& put) {
+  if (last_block(ticket)) fold_values(cnt, gridDim.x, partial, put);
 }
 
 // One pass of a multi-dot over y: NC columns from X on, and with SELF y . y.  All
@@ -254,11 +255,13 @@ __device__ __forceinline__ void mdot_pass(long long n, const R* __restrict__ X, 
 template <typename R> constexpr int mdot_cols() { return sizeof(R) == 8 ? 4 : 8; }
 
 // out[i] = X_i . y for i < k, and with self out[k] = y . y (per-thread sums in R, partials
-// in double), in passes of nearly equal numbers of columns
+// in double), in passes of nearly equal numbers of columns; cf, if not null, gets
+// out[i] / sig2[i]
 template <typename R, bool VEC>
 __global__ void __launch_bounds__(RED_THREADS, 4) k_mdot(long long n, int k, const R* __restrict__ X,
                                                          long long ld, const R* __restrict__ y, int self,
-                                                         double* partial, double* out, int take_sqrt,
+                                                         double* partial, double* out,
+                                                         const double* sig2, double* cf,
                                                          unsigned* ticket) {
   constexpr int KB = mdot_cols<R>();
   const int passes = (k + KB - 1) / KB;
@@ -298,32 +301,30 @@ __global__ void __launch_bounds__(RED_THREADS, 4) k_mdot(long long n, int k, con
     }
     i0 += nc;
   }
-  finish(k + (self ? 1 : 0), partial, out, take_sqrt, ticket);
+  finish(k + (self ? 1 : 0), partial, ticket, [&](int q, double v) {
+    out[q] = v;
+    if (cf) cf[q] = coef_over(v, sig2[q]);
+  });
 }
 
-// One Arnoldi step of the smoother with an unnormalised basis.  With the dots
-// g_i = v_i . w (i < k) and the squared basis norms sig2_i:
-//   w <- (w - sum_i (g_i / sig2_i) v_i) / sqrt(sig2_{k-1}),   t = w / D (if t),
-// and *out = ||w||^2 (the next sig2).
+// One Arnoldi step of the smoother with an unnormalised basis, its k coefficients cf_i
+// and the reciprocal norm of v_{k-1} in Hd (formed once, by the block that ended the
+// dots, and not in every block: an FP64 division or root is a chain of a microsecond):
+//   w <- (w - sum_i cf_i v_i) / ||v_{k-1}||,   t = w / D (if t),
+// the squared norm of w and its reciprocal root into Hd; with ls the block that ends the
+// norm also solves the smoother's least-squares problem (k <= LS_MAX).
+constexpr int LS_MAX = 8;
 template <typename R, bool VEC>
 __global__ void __launch_bounds__(RED_THREADS) k_arnoldi_update(long long n, int k,
                                                                 const R* __restrict__ X, long long ld,
-                                                                const double* __restrict__ g,
-                                                                const double* __restrict__ sig2,
                                                                 const R* __restrict__ D,
                                                                 R* __restrict__ w, R* __restrict__ t,
-                                                                double* partial, double* out,
+                                                                double* Hd, int ls, double* partial,
                                                                 unsigned* ticket) {
   __shared__ R cf[MAX_RESTART + 1];
   __shared__ R sc_sh;
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
-    const double s2 = sig2[i];
-    cf[i] = (s2 > 0.0 && s2 < 1e300) ? R(g[i] / s2) : R(0);
-  }
-  if (threadIdx.x == 0) {  // FP64 scalar work once per block
-    const double sl = sig2[k - 1];
-    sc_sh = (sl > 0.0 && sl < 1e300) ? R(1.0 / sqrt(sl)) : R(0);
-  }
+  for (int i = threadIdx.x; i < k; i += blockDim.x) cf[i] = R(Hd[HD_CF + i]);
+  if (threadIdx.x == RED_THREADS - 1) sc_sh = R(Hd[HD_ISIG + k - 1]);
   __syncthreads();
   const R sc = sc_sh;
   R acc2 = R(0);
@@ -354,16 +355,29 @@ __global__ void __launch_bounds__(RED_THREADS) k_arnoldi_update(long long n, int
   });
   const R s = block_sum(acc2);
   if (threadIdx.x == 0) partial[blockIdx.x] = double(s);
-  finish(1, partial, out, 0, ticket);
+  if (!last_block(ticket)) return;
+  fold_values(1, gridDim.x, partial, [&](int, double v) { put_norm(Hd + HD_SIG2 + k, Hd + HD_ISIG + k, v); });
+  if (ls) {
+    __shared__ double H[LS_MAX * (LS_MAX + 1)], nrm[2][LS_MAX + 1], g[LS_MAX + 1];
+    __syncthreads();
+    for (int q = threadIdx.x; q < k * (k + 1); q += RED_THREADS)
+      H[q] = __ldcg(Hd + (q / (k + 1)) * LDH + q % (k + 1));
+    if ((int)threadIdx.x <= k) {
+      nrm[0][threadIdx.x] = __ldcg(Hd + HD_SIG2 + threadIdx.x);
+      nrm[1][threadIdx.x] = __ldcg(Hd + HD_ISIG + threadIdx.x);
+    }
+    __syncthreads();
+    if (threadIdx.x < 32) warp_least_squares(k, H, k + 1, nrm[0], nrm[1], Hd + HD_Y, g);
+  }
 }
 
 // First basis vector of the smoother: v0 = r (copied unless r is v0 itself),
-// t = r / D, *out = ||r||^2.
+// t = r / D, its norm into Hd.
 template <typename R, bool VEC>
 __global__ void __launch_bounds__(RED_THREADS) k_init_basis(long long n, const R* r,
                                                             const R* __restrict__ D, R* v0,
-                                                            R* __restrict__ t, double* partial,
-                                                            double* out, unsigned* ticket) {
+                                                            R* __restrict__ t, double* Hd,
+                                                            double* partial, unsigned* ticket) {
   const bool copy = r != v0;
   R acc2 = R(0);
   chunk_loop(n, [&](long long c) {
@@ -385,7 +399,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_init_basis(long long n, const R
   });
   const R s = block_sum(acc2);
   if (threadIdx.x == 0) partial[blockIdx.x] = double(s);
-  finish(1, partial, out, 0, ticket);
+  finish(1, partial, ticket, [&](int, double v) { put_norm(Hd + HD_SIG2, Hd + HD_ISIG, v); });
 }
 
 // z (+)= (sum_i coef[i] X_i) / D   (no division when D is null)
@@ -572,47 +586,50 @@ void vscal(long long n, R a, R* y, cudaStream_t s) {
 }
 template <typename R>
 static void mdot(long long n, int k, const R* X, long long ld, const R* y, int self, double* out,
-                 int take_sqrt, double* partial, cudaStream_t s) {
+                 const double* sig2, double* cf, double* partial, cudaStream_t s) {
   const int nb = red_blocks(n);
   if ((k == 0 || mv_aligned(X, ld)) && al16(y))
-    k_mdot<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, take_sqrt,
-                                                       red_ticket(partial));
+    k_mdot<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, sig2, cf,
+                                               red_ticket(partial));
   else
-    k_mdot<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, take_sqrt,
-                                                        red_ticket(partial));
+    k_mdot<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, sig2, cf,
+                                                red_ticket(partial));
 }
 template <typename R>
 void vmdot(long long n, int k, const R* X, long long ld, const R* y, double* out, double* partial,
            cudaStream_t s) {
-  mdot(n, k, X, ld, y, 0, out, 0, partial, s);
+  mdot(n, k, X, ld, y, 0, out, nullptr, nullptr, partial, s);
 }
 template <typename R>
 void vmdot_self(long long n, int k, const R* X, long long ld, const R* y, double* out,
                 double* partial, cudaStream_t s) {
-  mdot(n, k, X, ld, y, 1, out, 0, partial, s);
+  mdot(n, k, X, ld, y, 1, out, nullptr, nullptr, partial, s);
 }
 template <typename R>
-void vinit_basis(long long n, const R* r, const R* D, R* v0, R* t, double* sig2_out,
-                 double* partial, cudaStream_t s) {
+void vmdot_cf(long long n, int k, const R* X, long long ld, const R* y, double* out, const double* sig2,
+              double* cf, double* partial, cudaStream_t s) {
+  mdot(n, k, X, ld, y, 0, out, sig2, cf, partial, s);
+}
+template <typename R>
+void vinit_basis(long long n, const R* r, const R* D, R* v0, R* t, double* Hd, double* partial,
+                 cudaStream_t s) {
   const int nb = red_blocks(n);
   if (al16(r) && al16(D) && al16(v0) && al16(t))
-    k_init_basis<R, true><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, partial, sig2_out,
-                                                     red_ticket(partial));
+    k_init_basis<R, true><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, Hd, partial, red_ticket(partial));
   else
-    k_init_basis<R, false><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, partial, sig2_out,
-                                                      red_ticket(partial));
+    k_init_basis<R, false><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, Hd, partial, red_ticket(partial));
 }
 template <typename R>
-void varnoldi_update(long long n, int k, const R* X, long long ld, const double* g,
-                     const double* sig2, const R* D, R* w, R* t, double* sig2_out,
-                     double* partial, cudaStream_t s) {
-  const int nb = red_blocks(n);
+void varnoldi_update(long long n, int k, const R* X, long long ld, const R* D, R* w, R* t, double* Hd,
+                     bool ls, double* partial, cudaStream_t s) {
+  const int nb = red_blocks(n), fused = ls && k <= LS_MAX;
   if (mv_aligned(X, ld) && al16(D) && al16(w) && al16(t))
-    k_arnoldi_update<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, g, sig2, D, w, t, partial,
-                                                         sig2_out, red_ticket(partial));
+    k_arnoldi_update<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, D, w, t, Hd, fused, partial,
+                                                         red_ticket(partial));
   else
-    k_arnoldi_update<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, g, sig2, D, w, t, partial,
-                                                          sig2_out, red_ticket(partial));
+    k_arnoldi_update<R, false><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, D, w, t, Hd, fused, partial,
+                                                          red_ticket(partial));
+  if (ls && !fused) small_ls(Hd, k, s);
 }
 template <typename R>
 void vcombine(long long n, int k, const R* X, long long ld, const double* coef, const R* D, R* z,
@@ -659,11 +676,12 @@ template void vcast<double, float>(long long, const float*, double*, cudaStream_
                          cudaStream_t);                                                        \
   template void vmdot_self<R>(long long, int, const R*, long long, const R*, double*, double*, \
                               cudaStream_t);                                                   \
+  template void vmdot_cf<R>(long long, int, const R*, long long, const R*, double*,            \
+                            const double*, double*, double*, cudaStream_t);                    \
   template void vinit_basis<R>(long long, const R*, const R*, R*, R*, double*, double*,        \
                                cudaStream_t);                                                  \
-  template void varnoldi_update<R>(long long, int, const R*, long long, const double*,         \
-                                   const double*, const R*, R*, R*, double*, double*,          \
-                                   cudaStream_t);                                              \
+  template void varnoldi_update<R>(long long, int, const R*, long long, const R*, R*, R*,      \
+                                   double*, bool, double*, cudaStream_t);                      \
   template void vcombine<R>(long long, int, const R*, long long, const double*, const R*, R*,  \
                             bool, cudaStream_t);                                               \
   template void vmaxpy<R>(long long, int, const R*, long long, const double*, double, R*,      \

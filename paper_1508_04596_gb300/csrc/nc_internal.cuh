@@ -202,14 +202,19 @@ struct MarchPlan {
 };
 MarchPlan march_plan(const LevelDev& d, bool fp64);
 
-// Dots that a product hands back with its result w: out[q] = <V_q, w> for q < k, V_q =
-// V + q ld; partial: reduction scratch.
+// What a product hands back with its result w: with k > 0 the dots out[q] = <V_q, w>
+// for q < k, V_q = V + q ld, and cf[q] = out[q] / sig2[q] (0 where sig2 vanishes);
+// with b the result is b - w instead.  partial: reduction scratch.
 template <typename R>
 struct Dots {
-  int k;
-  const R* V;
-  long long ld;
-  double *out, *partial;
+  int k = 0;
+  const R* V = nullptr;
+  long long ld = 0;
+  double* out = nullptr;
+  const double* sig2 = nullptr;
+  double* cf = nullptr;
+  double* partial = nullptr;
+  const R* b = nullptr;
 };
 
 // ---- element operators (nc_kernels.cu); Y is scratch of scratch_len(E) elements of R
@@ -302,25 +307,32 @@ void vmaxpy_f32x(long long n, int k, const float* X, long long ld, const double*
 template <typename R>
 void vmaxpy_scale(long long n, int k, const R* X, long long ld, const double* h, const double* q,
                   double* nw_out, R* y, cudaStream_t s);
-// Smoother Arnoldi with an unnormalised basis.  vinit_basis: v0 = r (r may be v0
-// itself), t = r / D, *sig2_out = ||r||^2.  varnoldi_update with the dots
-// g[i] = <v_i, w> (i < k) and the squared norms sig2[i]:
-// w <- (w - sum_i g[i]/sig2[i] v_i) / sqrt(sig2[k-1]), t = w / D (t may be null),
-// *sig2_out = ||w||^2.
+// as vmdot, and cf[i] = out[i] / sig2[i] (0 where sig2 vanishes or is not finite)
 template <typename R>
-void vinit_basis(long long n, const R* r, const R* D, R* v0, R* t, double* sig2_out,
-                 double* partial, cudaStream_t s);
+void vmdot_cf(long long n, int k, const R* X, long long ld, const R* y, double* out, const double* sig2,
+              double* cf, double* partial, cudaStream_t s);
+// Smoother Arnoldi with an unnormalised basis; Hd its device scalars.  vinit_basis:
+// v0 = r (r may be v0 itself), t = r / D, norm 0 into Hd.  varnoldi_update, with k
+// basis vectors and the coefficients of the step in Hd:
+// w <- (w - sum_i cf[i] v_i) / ||v_{k-1}||, t = w / D (t may be null), norm k into Hd;
+// with ls the least-squares problem of k steps is solved as well (as small_ls).
 template <typename R>
-void varnoldi_update(long long n, int k, const R* X, long long ld, const double* g,
-                     const double* sig2, const R* D, R* w, R* t, double* sig2_out,
-                     double* partial, cudaStream_t s);
+void vinit_basis(long long n, const R* r, const R* D, R* v0, R* t, double* Hd, double* partial,
+                 cudaStream_t s);
+template <typename R>
+void varnoldi_update(long long n, int k, const R* X, long long ld, const R* D, R* w, R* t, double* Hd,
+                     bool ls, double* partial, cudaStream_t s);
 // z = (sum_i coef[i] X_i) / D (D may be null: no division), or z += ... with accumulate
 // Device scalars of a smoother: the Hessenberg columns of raw dots (leading dimension
-// LDH), the coefficients of the correction and the squared norms of the basis.
+// LDH), the coefficients of the correction, the squared norms of the basis and their
+// reciprocal roots (0 for a vanishing or non-finite norm), and the coefficients
+// <v_i, w> / ||v_i||^2 of the step in progress.
 constexpr int LDH = MAX_RESTART + 1;
 constexpr int HD_Y = LDH * LDH;
 constexpr int HD_SIG2 = HD_Y + LDH;
-constexpr int HD_SIZE = HD_SIG2 + LDH;
+constexpr int HD_ISIG = HD_SIG2 + LDH;
+constexpr int HD_CF = HD_ISIG + LDH;
+constexpr int HD_SIZE = HD_CF + LDH;
 // The smoother's small least-squares problem (nc_smooth.cu): Hd[HD_Y..] from the rest.
 void small_ls(double* Hd, int k, cudaStream_t s);
 template <typename R>

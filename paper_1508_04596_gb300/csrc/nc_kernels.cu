@@ -209,6 +209,7 @@ template <typename R, int MODE>
 __global__ void __launch_bounds__(NODE_THREADS) k_gather_march(LevelDev d, MarchPlan mp,
                                                                const R* __restrict__ Y_,
                                                                const R* __restrict__ xv_,
+                                                               const R* __restrict__ b_,
                                                                R* __restrict__ out) {
   chained();
   const R* const Y = fresh(Y_);
@@ -219,6 +220,14 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_march(LevelDev d, March
   node_ijk(d, n, i, j, k);
   R acc[5] = {R(0), R(0), R(0), R(0), R(0)};
   march::node_sums(d, mp, i, j, k, Y, acc);
+  if (MODE == G_LIN && b_) {  // b - A v
+    const R* const b = fresh(b_);
+    const uint8_t fl = d.flag[n];
+#pragma unroll
+    for (int f = 0; f < 5; ++f)
+      out[f * d.Nn + n] = b[f * d.Nn + n] - ((fl >> f) & 1 ? xv[f * d.Nn + n] : acc[f]);
+    return;
+  }
   node_rows<R, MODE>(d, n, i, j, k, acc, xv, out);
 }
 
@@ -233,6 +242,7 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_dots(LevelDev d, MarchP
                                                               R* __restrict__ out, int k,
                                                               const R* __restrict__ V_, long long ld,
                                                               double* partial, double* dots,
+                                                              const double* sig2, double* cf,
                                                               unsigned* ticket) {
   chained();
   const R* const Y = fresh(Y_);
@@ -269,7 +279,11 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_dots(LevelDev d, MarchP
 #pragma unroll
   for (int q = 0; q < KB; ++q) v[q] = q < k ? a0[q] + a1[q] : R(0);
   block_values<NODE_THREADS>(v, k, partial);
-  if (last_block(ticket)) fold_values(k, gridDim.x, partial, dots);
+  if (last_block(ticket))
+    fold_values(k, gridDim.x, partial, [&](int q, double t) {
+      dots[q] = t;
+      cf[q] = coef_over(t, sig2[q]);
+    });
 }
 
 template <typename R, bool ZERO>
@@ -429,18 +443,20 @@ static void run_gather(const LevelDev& d, const R* Y, const R* xv, R* out, cudaS
                        const Dots<R>* dots = nullptr) {
   const MarchPlan mp = march_plan(d, sizeof(R) == 8);
   const unsigned nb = nblocks(d.Nn, NODE_THREADS);
-  if (dots && dots->k <= 8) {
+  if (dots && dots->k > 0 && dots->k <= 8) {
     const unsigned rb = nb < RED_BLOCKS_MAX ? nb : RED_BLOCKS_MAX;
     if (dots->k <= 4)
       launch(k_gather_dots<R, 4>, rb, NODE_THREADS, 0, s, d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
-                                                      dots->partial, dots->out, red_ticket(dots->partial));
+             dots->partial, dots->out, dots->sig2, dots->cf, red_ticket(dots->partial));
     else
       launch(k_gather_dots<R, 8>, rb, NODE_THREADS, 0, s, d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
-                                                      dots->partial, dots->out, red_ticket(dots->partial));
+             dots->partial, dots->out, dots->sig2, dots->cf, red_ticket(dots->partial));
     return;
   }
-  launch(k_gather_march<R, MODE>, nb, NODE_THREADS, 0, s, d, mp, Y, xv, out);
-  if (dots) vmdot(5 * d.Nn, dots->k, dots->V, dots->ld, (const R*)out, dots->out, dots->partial, s);
+  launch(k_gather_march<R, MODE>, nb, NODE_THREADS, 0, s, d, mp, Y, xv, dots ? dots->b : nullptr, out);
+  if (dots && dots->k)
+    vmdot_cf(5 * d.Nn, dots->k, dots->V, dots->ld, (const R*)out, dots->out, dots->sig2, dots->cf,
+             dots->partial, s);
 }
 
 template <typename R>

@@ -108,17 +108,25 @@ __device__ __forceinline__ double fold_partials(int nb, const double* partial) {
   return block_fold<MAX, THREADS>(v);
 }
 
-// out[q] = the sum of partial[q * nb ...] for q < cnt (or its square root), a warp per
-// value, in a fixed order.
-__device__ __forceinline__ void fold_values(int cnt, int nb, const double* partial, double* out,
-                                            int take_sqrt = 0) {
+// put(q, the sum of partial[q * nb ...]) for q < cnt, by one lane of the value's warp; a
+// fixed order.
+template <typename F>
+__device__ __forceinline__ void fold_values(int cnt, int nb, const double* partial, F&& put) {
   const int lane = threadIdx.x & 31;
   for (int q = threadIdx.x >> 5; q < cnt; q += blockDim.x >> 5) {
     double v = 0.0;
     for (int b = lane; b < nb; b += 32) v += __ldcg(partial + (long long)q * nb + b);
     v = warp_fold<false>(v);
-    if (lane == 0) out[q] = take_sqrt ? sqrt(v > 0.0 ? v : 0.0) : v;
+    if (lane == 0) put(q, v);
   }
 }
+
+// A smoother's squared norm and its reciprocal root.
+__device__ __forceinline__ bool norm_ok(double s2) { return s2 > 0.0 && s2 < 1e300; }
+__device__ __forceinline__ void put_norm(double* sig2, double* isig, double s2) {
+  *sig2 = s2;
+  *isig = norm_ok(s2) ? rsqrt(s2) : 0.0;
+}
+__device__ __forceinline__ double coef_over(double g, double s2) { return norm_ok(s2) ? g / s2 : 0.0; }
 
 }  // namespace nc

@@ -13,9 +13,12 @@ __global__ void __launch_bounds__(32) k_small_ls(double* Hd, int k) {
   double* isig = sig2 + k + 1;
   double* g = isig + k + 1;
   for (int t = threadIdx.x; t < k * (k + 1); t += 32) H[t] = Hd[(t / (k + 1)) * LDH + t % (k + 1)];
-  for (int t = threadIdx.x; t <= k; t += 32) sig2[t] = Hd[HD_SIG2 + t];
+  for (int t = threadIdx.x; t <= k; t += 32) {
+    sig2[t] = Hd[HD_SIG2 + t];
+    isig[t] = Hd[HD_ISIG + t];
+  }
   __syncwarp();
-  warp_least_squares(k, H, k + 1, sig2, Hd + HD_Y, isig, g);
+  warp_least_squares(k, H, k + 1, sig2, isig, Hd + HD_Y, g);
 }
 
 }  // namespace

@@ -17,15 +17,11 @@ namespace nc {
 // by lane j to column j (and j + 32), the substitution runs by columns with a lane per
 // row.  An FP64 instruction takes a scheduler 64 cycles whatever the number of active
 // lanes: one thread working through the k^2 operations took 40 us for k = 6, this
-// 7 us.  k <= 64; isig (k + 1) and g (k + 1) are scratch.
-__device__ __forceinline__ void warp_least_squares(int k, double* H, int ld, const double* sig2, double* y,
-                                                   double* isig, double* g) {
+// 6 us.  isig: the norms' reciprocal roots, 0 where they vanish; g (k + 1) is scratch.
+__device__ __forceinline__ void warp_least_squares(int k, double* H, int ld, const double* sig2,
+                                                   const double* isig, double* y, double* g) {
   const int lane = threadIdx.x & 31;
-  for (int i = lane; i <= k; i += 32) {
-    const double s2 = sig2[i];
-    isig[i] = (s2 > 0.0 && s2 < 1e300) ? rsqrt(s2) : 0.0;
-    g[i] = 0.0;
-  }
+  for (int i = lane; i <= k; i += 32) g[i] = 0.0;
   __syncwarp();
   if (lane == 0) {
     const double b2 = sig2[0], beta = sqrt(b2 > 0.0 ? b2 : 0.0);

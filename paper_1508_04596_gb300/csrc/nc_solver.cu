@@ -49,8 +49,10 @@ void level_apply(nc_ctx* ctx, int l, bool tr, const R* v, R* out, cudaStream_t s
   LevelBuf<R>& B = buf<R>(L);
   if (B.use_gst) {  // assembled or Galerkin operator
     op_stencil<R>(L.d, B.gst, tr, v, out, s);
-    if (dots)
-      vmdot(5 * L.d.Nn, dots->k, dots->V, dots->ld, (const R*)out, dots->out, dots->partial, s);
+    if (dots && dots->k)
+      vmdot_cf(5 * L.d.Nn, dots->k, dots->V, dots->ld, (const R*)out, dots->out, dots->sig2, dots->cf,
+               dots->partial, s);
+    if (dots && dots->b) vxpay(5 * L.d.Nn, dots->b, R(-1), out, s);
     return;
   }
   if constexpr (std::is_same<R, double>::value) {
@@ -71,8 +73,8 @@ void level_apply(nc_ctx* ctx, int l, bool tr, const R* v, R* out, cudaStream_t s
 // Right Jacobi-preconditioned GMRES(k) on level l:  z += D^-1 V y  approximately
 // solving A z = b.  With zero_init the initial guess is 0.  The basis is kept
 // unnormalised (each new vector is divided by the previous vector's norm, so
-// magnitudes stay bounded); small_ls turns the raw dots and norms into the
-// normalised Hessenberg.  Per Arnoldi step three kernels: the element product of
+// magnitudes stay bounded); the least-squares solve at the end turns the raw dots and
+// norms into the normalised Hessenberg.  Per Arnoldi step three kernels: the element product of
 // t = D^-1 v_j, the gather of w with its dots, and one pass that orthogonalises,
 // rescales, forms the next t and the new norm.
 template <typename R>
@@ -84,21 +86,27 @@ void smooth(nc_ctx* ctx, int l, bool tr, int k, bool zero_init, cudaStream_t s) 
   R* V = B.V;
   double* Hd = B.Hd;
   if (zero_init) {
-    vinit_basis(n, (const R*)B.b, (const R*)B.diag, V, B.t, Hd + HD_SIG2, ctx->partial, s);
+    vinit_basis(n, (const R*)B.b, (const R*)B.diag, V, B.t, Hd, ctx->partial, s);
   } else {
-    level_apply<R>(ctx, l, tr, B.z, B.t, s);
-    vwaxpy(n, (const R*)B.b, R(-1), (const R*)B.t, V, s);
-    vinit_basis(n, (const R*)V, (const R*)B.diag, V, B.t, Hd + HD_SIG2, ctx->partial, s);
+    Dots<R> res;
+    res.b = B.b;
+    level_apply<R>(ctx, l, tr, B.z, V, s, &res);  // v0 = b - A z
+    vinit_basis(n, (const R*)V, (const R*)B.diag, V, B.t, Hd, ctx->partial, s);
   }
   for (int j = 0; j < k; ++j) {
     R* w = V + (j + 1) * ld;
-    double* hcol = Hd + j * LDH;
-    const Dots<R> dots{j + 1, V, ld, hcol, ctx->partial};
+    Dots<R> dots;
+    dots.k = j + 1;
+    dots.V = V;
+    dots.ld = ld;
+    dots.out = Hd + j * LDH;
+    dots.sig2 = Hd + HD_SIG2;
+    dots.cf = Hd + HD_CF;
+    dots.partial = ctx->partial;
     level_apply<R>(ctx, l, tr, B.t, w, s, &dots);
-    varnoldi_update(n, j + 1, (const R*)V, ld, hcol, Hd + HD_SIG2, (const R*)B.diag, w,
-                    j + 1 < k ? B.t : (R*)nullptr, Hd + HD_SIG2 + j + 1, ctx->partial, s);
+    varnoldi_update(n, j + 1, (const R*)V, ld, (const R*)B.diag, w, j + 1 < k ? B.t : (R*)nullptr, Hd,
+                    j + 1 == k, ctx->partial, s);
   }
-  small_ls(Hd, k, s);
   // z (+)= D^-1 (V y)
   vcombine(n, k, (const R*)V, ld, Hd + HD_Y, (const R*)B.diag, B.z, !zero_init, s);
 }
@@ -115,8 +123,9 @@ void vcycle(nc_ctx* ctx, int l, int nlev, bool tr, const nc_solve_opts& o, cudaS
     return;
   }
   smooth<R>(ctx, l, tr, o.smooth_its, true, s);
-  level_apply<R>(ctx, l, tr, B.z, B.t, s);
-  vwaxpy(5 * L.d.Nn, (const R*)B.b, R(-1), (const R*)B.t, B.r, s);
+  Dots<R> res;
+  res.b = B.b;
+  level_apply<R>(ctx, l, tr, B.z, B.r, s, &res);  // r = b - A z
   Level& C = ctx->lv[l + 1];
   op_restrict<R>(L.d, B.r, C.d, buf<R>(C).b, s);
   vcycle<R>(ctx, l + 1, nlev, tr, o, s);
