@@ -235,8 +235,9 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_march(LevelDev d, March
 // takes of it next: the result is not read back, and no multi-dot is launched (a third
 // of the reduction launches; on a small level a launch costs more than its work).
 // Two accumulators per column; partials fold in the last block.
-template <typename R, int KB>
-__global__ void __launch_bounds__(NODE_THREADS) k_gather_dots(LevelDev d, MarchPlan mp,
+// TH threads a block: 1024 where one block holds every node (nothing to fold then).
+template <typename R, int KB, int TH>
+__global__ void __launch_bounds__(TH) k_gather_dots(LevelDev d, MarchPlan mp,
                                                               const R* __restrict__ Y_,
                                                               const R* __restrict__ xv_,
                                                               R* __restrict__ out, int k,
@@ -251,8 +252,8 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_dots(LevelDev d, MarchP
   R a0[KB], a1[KB];
 #pragma unroll
   for (int q = 0; q < KB; ++q) a0[q] = a1[q] = R(0);
-  for (long long n = blockIdx.x * (long long)NODE_THREADS + threadIdx.x; n < d.Nn;
-       n += (long long)gridDim.x * NODE_THREADS) {
+  for (long long n = blockIdx.x * (long long)TH + threadIdx.x; n < d.Nn;
+       n += (long long)gridDim.x * TH) {
     int i, j, kk;
     node_ijk(d, n, i, j, kk);
     R acc[5] = {R(0), R(0), R(0), R(0), R(0)};
@@ -278,7 +279,7 @@ __global__ void __launch_bounds__(NODE_THREADS) k_gather_dots(LevelDev d, MarchP
   R v[KB];
 #pragma unroll
   for (int q = 0; q < KB; ++q) v[q] = q < k ? a0[q] + a1[q] : R(0);
-  block_values<NODE_THREADS>(v, k, partial);
+  block_values<TH>(v, k, partial);
   if (last_block(ticket))
     fold_values(k, gridDim.x, partial, [&](int q, double t) {
       dots[q] = t;
@@ -445,12 +446,17 @@ static void run_gather(const LevelDev& d, const R* Y, const R* xv, R* out, cudaS
   const unsigned nb = nblocks(d.Nn, NODE_THREADS);
   if (dots && dots->k > 0 && dots->k <= 8) {
     const unsigned rb = nb < RED_BLOCKS_MAX ? nb : RED_BLOCKS_MAX;
-    if (dots->k <= 4)
-      launch(k_gather_dots<R, 4>, rb, NODE_THREADS, 0, s, d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
-             dots->partial, dots->out, dots->sig2, dots->cf, red_ticket(dots->partial));
-    else
-      launch(k_gather_dots<R, 8>, rb, NODE_THREADS, 0, s, d, mp, Y, xv, out, dots->k, dots->V, dots->ld,
-             dots->partial, dots->out, dots->sig2, dots->cf, red_ticket(dots->partial));
+    auto go = [&](auto kernel, unsigned blocks, unsigned threads) {
+      launch(kernel, blocks, threads, 0, s, d, mp, Y, xv, out, dots->k, dots->V, dots->ld, dots->partial,
+             dots->out, dots->sig2, dots->cf, red_ticket(dots->partial));
+    };
+    if constexpr (sizeof(R) == 4) {
+      if (nb > 1 && d.Nn <= 1024) {
+        go(dots->k <= 4 ? k_gather_dots<R, 4, 1024> : k_gather_dots<R, 8, 1024>, 1, 1024);
+        return;
+      }
+    }
+    go(dots->k <= 4 ? k_gather_dots<R, 4, NODE_THREADS> : k_gather_dots<R, 8, NODE_THREADS>, rb, NODE_THREADS);
     return;
   }
   launch(k_gather_march<R, MODE>, nb, NODE_THREADS, 0, s, d, mp, Y, xv, dots ? dots->b : nullptr, out);
