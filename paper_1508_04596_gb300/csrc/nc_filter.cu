@@ -24,7 +24,7 @@
 //    with the update of p, where a sum over the eight elements takes 64;
 //  * k_cg_update takes the steps of x and r with <r, r> and <r, r/d>.
 // FP64 operations bound both (two FP64 lanes per SM).  80x80x160 (1.06M nodes, 19
-// iterations): 1.86 ms, k_cg_apply 67 us and k_cg_update 23 us an iteration; 5.75 ms
+// iterations): 1.68 ms, k_cg_apply 58 us and k_cg_update 20 us an iteration; 5.75 ms
 // with one kernel per vector operation, a 64-term product (146 us) and three host
 // reads per iteration.
 #include <algorithm>
@@ -122,13 +122,16 @@ __device__ __forceinline__ int mirror(int g, int n) {
 }
 
 // p = r/d + beta p_old, q = A p, alpha = <r, r/d> / <p, q>.
-// A block marches a 32 x 8 node tile over zc planes; a plane of p with its halo is
+// A block marches a tw x th node tile over zc planes; a plane of p with its halo is
 // formed in shared memory (two buffers, one barrier per plane), the loads of the
 // next plane in flight meanwhile.  P and Q are a plane's contributions to its own and
 // to the adjacent planes' products.
-constexpr int HTX = 32, HTY = FT / HTX, HW = HTX + 2, HSLOTS = HW * (HTY + 2);
-__global__ void __launch_bounds__(FT) k_cg_apply(LevelDev d, HelmCoef c, int zc, long long items,
-                                                 int tiles_x, int tiles_y,
+constexpr int HSLOTS = 2 * FT;  // nodes of a tile with its halo at most
+struct HelmTile {
+  int tw, th, tiles_x, tiles_y, zc;
+  long long items;  // tiles times marches
+};
+__global__ void __launch_bounds__(FT) k_cg_apply(LevelDev d, HelmCoef c, HelmTile t,
                                                  const double* __restrict__ r,
                                                  const double* __restrict__ p_old,
                                                  double* __restrict__ p_new, double* __restrict__ q,
@@ -137,36 +140,36 @@ __global__ void __launch_bounds__(FT) k_cg_apply(LevelDev d, HelmCoef c, int zc,
   const double beta = s->beta;
   const bool first = s->it == 0;  // p_old is not set yet
   __shared__ double sm[2][HSLOTS];
-  const int tx = threadIdx.x % HTX, ty = threadIdx.x / HTX;
+  const int tx = threadIdx.x % t.tw, ty = threadIdx.x / t.tw;
+  const int hw = t.tw + 2, slots = hw * (t.th + 2);
   const long long sy = d.nx + 1, sz = (long long)(d.nx + 1) * (d.ny + 1);
-  static_assert(HSLOTS <= 2 * FT, "two tile slots per thread");
   double pq = 0.0;
-  for (long long item = blockIdx.x; item < items; item += gridDim.x) {
-    const int bx = (int)(item % tiles_x), by = (int)(item / tiles_x % tiles_y);
-    const int k0 = (int)(item / tiles_x / tiles_y) * zc, k1 = min(k0 + zc, d.nz + 1);
+  for (long long item = blockIdx.x; item < t.items; item += gridDim.x) {
+    const int bx = (int)(item % t.tiles_x), by = (int)(item / t.tiles_x % t.tiles_y);
+    const int k0 = (int)(item / t.tiles_x / t.tiles_y) * t.zc, k1 = min(k0 + t.zc, d.nz + 1);
     long long at[2];  // node of the slot in plane 0
     double wxy[2], wxy2[2];  // 1/d on an inner and on a boundary plane
     bool own[2];      // the slot is a node of this tile
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
-      const int t = threadIdx.x + u * FT, sx = t % HW, s2 = t / HW;
-      const int gi = bx * HTX + sx - 1, gj = by * HTY + s2 - 1;
+      const int q = threadIdx.x + u * FT, sx = q % hw, s2 = q / hw;
+      const int gi = bx * t.tw + sx - 1, gj = by * t.th + s2 - 1;
       const int mi = mirror(gi, d.nx), mj = mirror(gj, d.ny);
       at[u] = mi + sy * mj;
       wxy[u] = c.inv_d * pow2(on_face(mi, d.nx) + on_face(mj, d.ny));
       wxy2[u] = 2.0 * wxy[u];
-      own[u] = sx >= 1 && sx <= HTX && s2 >= 1 && s2 <= HTY && gi <= d.nx && gj <= d.ny;
+      own[u] = sx >= 1 && sx <= t.tw && s2 >= 1 && s2 <= t.th && gi <= d.nx && gj <= d.ny;
     }
-    const bool two = threadIdx.x + FT < HSLOTS;
-    const int i = bx * HTX + tx, j = by * HTY + ty;
-    const bool in = i <= d.nx && j <= d.ny;
+    const bool use[2] = {(int)threadIdx.x < slots, (int)threadIdx.x + FT < slots};
+    const int i = bx * t.tw + tx, j = by * t.th + ty;
+    const bool in = ty < t.th && i <= d.nx && j <= d.ny;
     const int faces_xy = on_face(i, d.nx) + on_face(j, d.ny);
     double rv[2] = {0.0, 0.0}, pv[2] = {0.0, 0.0};
     auto load = [&](int kk) {
       const long long off = sz * mirror(kk, d.nz);
 #pragma unroll
       for (int u = 0; u < 2; ++u)
-        if (u == 0 || two) {
+        if (use[u]) {
           rv[u] = r[at[u] + off];
           pv[u] = first ? 0.0 : p_old[at[u] + off];
         }
@@ -179,17 +182,17 @@ __global__ void __launch_bounds__(FT) k_cg_apply(LevelDev d, HelmCoef c, int zc,
       const bool face = on_face(gk, d.nz);
 #pragma unroll
       for (int u = 0; u < 2; ++u)
-        if (u == 0 || two) {
+        if (use[u]) {
           const double v = rv[u] * (face ? wxy2[u] : wxy[u]) + beta * pv[u];
           b[threadIdx.x + u * FT] = v;
           if (own[u] && kk >= k0 && kk < k1) p_new[at[u] + sz * gk] = v;
         }
       if (kk < k1) load(kk + 1);
       __syncthreads();
-      const double* m = b + (ty + 1) * HW + tx + 1;
+      const double* m = b + ((ty < t.th ? ty : 0) + 1) * hw + tx + 1;
       const double cc = m[0];
-      const double e = (m[-1] + m[1]) + (m[-HW] + m[HW]);
-      const double dg = (m[-HW - 1] + m[-HW + 1]) + (m[HW - 1] + m[HW + 1]);
+      const double e = (m[-1] + m[1]) + (m[-hw] + m[hw]);
+      const double dg = (m[-hw - 1] + m[-hw + 1]) + (m[hw - 1] + m[hw + 1]);
       const double Q = c.w[1] * cc + (c.w[2] * e + c.w[3] * dg);
       if (kk > k0 && in) {
         const int kp = kk - 1;
@@ -222,20 +225,28 @@ __global__ void __launch_bounds__(FT) k_cg_update(LevelDev d, HelmCoef c, const 
                                                   double* __restrict__ r, double* partial, CgState* s) {
   if (s->done) return;
   const double alpha = s->alpha;
-  double rr = 0.0, rz = 0.0;
-  for (long long n = blockIdx.x * (long long)FT + threadIdx.x; n < d.Nn; n += (long long)gridDim.x * FT) {
+  double v2[2] = {0.0, 0.0};  // <r, r>, <r, r/d> d_0
+  const long long gs = (long long)gridDim.x * FT;
+  auto step = [&](long long n, double xv, double pv, double rv, double qv) {
     int i, j, k;
     node_ijk(d, n, i, j, k);
-    x[n] += alpha * p[n];
-    const double v = r[n] - alpha * q[n];
+    x[n] = xv + alpha * pv;
+    const double v = rv - alpha * qv;
     r[n] = v;
-    rr += v * v;
-    rz += v * (v * pow2(on_face(i, d.nx) + on_face(j, d.ny) + on_face(k, d.nz)));
+    v2[0] += v * v;
+    v2[1] += v * (v * pow2(on_face(i, d.nx) + on_face(j, d.ny) + on_face(k, d.nz)));
+  };
+  long long n = blockIdx.x * (long long)FT + threadIdx.x;
+  for (; n + gs < d.Nn; n += 2 * gs) {  // two nodes' loads in flight
+    const long long m = n + gs;
+    const double x0 = x[n], p0 = p[n], r0 = r[n], q0 = q[n];
+    const double x1 = x[m], p1 = p[m], r1 = r[m], q1 = q[m];
+    step(n, x0, p0, r0, q0);
+    step(m, x1, p1, r1, q1);
   }
-  rr = block_fold<false, FT>(rr);
-  if (threadIdx.x == 0) partial[blockIdx.x] = rr;
-  rz = block_fold<false, FT>(rz);
-  if (threadIdx.x == 0) partial[gridDim.x + blockIdx.x] = rz;
+  if (n < d.Nn) step(n, x[n], p[n], r[n], q[n]);
+  block_values<FT>(v2, 2, partial);
+  double rr, rz;
   if (!last_block(&s->ticket)) return;
   rr = fold_partials<false, FT>(gridDim.x, partial);
   rz = fold_partials<false, FT>(gridDim.x, partial + gridDim.x) * c.inv_d;
@@ -265,21 +276,41 @@ __global__ void k_elem_mean(LevelDev d, const double* __restrict__ x, double* __
   g[e] = 0.125 * acc;
 }
 
-// Planes per tile march of k_cg_apply: the count that leaves the busiest SM the least
-// work, a march of zc planes costing zc + 2 halo planes, blocks spread over 152 SMs
+// Tile and march of k_cg_apply.  An FP64 instruction costs a warp the same however few of
+// its lanes hold a node, so the tile (16 to 64 wide, as high as 256 threads allow) is
+// the one that covers the plane in the fewest blocks: 81 x 81 nodes take 27 tiles of 27
+// x 9, 33 of 32 x 8 (67 us an application, 58 now).  A march is as long as leaves the busiest SM
+// the least work, zc planes costing zc + 2 with the halo, blocks spread over 152 SMs
 // (short marches for small grids, where whole columns would leave SMs idle).
-int planes_per_block(long long tiles, int planes) {
-  int best = 1;
+HelmTile helm_tile(const LevelDev& d) {
+  HelmTile t = {};
+  long long least = 0;
+  for (int tw = 16; tw <= 64; ++tw) {
+    const int th = FT / tw;
+    const long long tx = (d.nx + tw) / tw, ty = (d.ny + th) / th;
+    // warps with a node, and the blocks' overhead
+    const long long cost = tx * ty * ((tw * th + 31) / 32 * 4 + 1);
+    if ((tw + 2) * (th + 2) <= HSLOTS && (!least || cost < least)) {
+      least = cost;
+      t.tw = tw;
+      t.th = th;
+      t.tiles_x = (int)tx;
+      t.tiles_y = (int)ty;
+    }
+  }
+  const long long tiles = (long long)t.tiles_x * t.tiles_y;
+  const int planes = d.nz + 1;
   double cost = 1e300;
   for (int zc = 1; zc <= planes && zc <= 64; ++zc) {
     const long long blocks = tiles * ((planes + zc - 1) / zc);
-    const double t = (double)((blocks + 151) / 152) * (zc + 2);
-    if (t < cost) {
-      cost = t;
-      best = zc;
+    const double w = (double)((blocks + 151) / 152) * (zc + 2);
+    if (w < cost) {
+      cost = w;
+      t.zc = zc;
     }
   }
-  return best;
+  t.items = tiles * ((planes + t.zc - 1) / t.zc);
+  return t;
 }
 
 }  // namespace
@@ -305,17 +336,13 @@ extern "C" nc_status nc_filter(nc_ctx* ctx, const double* rho, double* gamma_f, 
   cudaMemsetAsync(cg, 0, sizeof(CgState), s);
   const unsigned vb = (unsigned)std::min<long long>((Nn + FT - 1) / FT, RED_BLOCKS_MAX);
   k_cg_rhs<<<vb, FT, 0, s>>>(d, c, rho, r, x, ctx->partial, cg);
-  const int tiles_x = (d.nx + HTX) / HTX, tiles_y = (d.ny + HTY) / HTY;
-  const long long tiles = (long long)tiles_x * tiles_y;
-  const int zc = planes_per_block(tiles, d.nz + 1);
-  const long long items = tiles * ((d.nz + zc) / zc);
-  const unsigned ab = (unsigned)std::min<long long>(items, (long long)MAX_RESTART * RED_BLOCKS_MAX);
+  const HelmTile tile = helm_tile(d);
+  const unsigned ab = (unsigned)std::min<long long>(tile.items, (long long)MAX_RESTART * RED_BLOCKS_MAX);
   CgState h;
   int m = 0, batch = 16;  // a radius of 2.5 h takes about 19 iterations
   do {
     for (int i = 0; i < batch; ++i, ++m) {
-      k_cg_apply<<<ab, FT, 0, s>>>(d, c, zc, items, tiles_x, tiles_y, r, p[m & 1], p[(m + 1) & 1], q,
-                                   ctx->partial, cg);
+      k_cg_apply<<<ab, FT, 0, s>>>(d, c, tile, r, p[m & 1], p[(m + 1) & 1], q, ctx->partial, cg);
       k_cg_update<<<vb, FT, 0, s>>>(d, c, p[(m + 1) & 1], q, x, r, ctx->partial, cg);
     }
     k_elem_mean<<<fblocks(d.E), FT, 0, s>>>(d, x, gamma_f, cg);

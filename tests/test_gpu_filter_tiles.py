@@ -1,4 +1,4 @@
-"""nc_filter at the edges of its 32 x 8 node tiles and plane marches (node counts one below, at
+"""nc_filter at the edges of its node tiles and plane marches (node counts one below, at
 and one above a tile, one element across, many planes), for radii from 0 (the mass matrix alone)
 to 6 elements, against the oracle's sparse direct solve.
 
