@@ -392,7 +392,7 @@ __global__ void k_coarsen_elem(LevelDev f, const R* __restrict__ gf, LevelDev c,
 // sums per lane) against 40 per element, or per 32 faces with one element across.
 MarchPlan march_plan(const LevelDev& d, bool fp64) {
   const long long slots = fp64 ? 608 : 8 * 152;
-  const double extra = fp64 ? 0.15 : 0.6;
+  const double extra = fp64 ? 0.05 : 0.6;
   MarchPlan p;
   p.stride = 32 % (d.nx + 1) == 0 ? 32 : 31;
   const long long faces = (long long)(d.nx + 1) * d.nz;
