@@ -217,6 +217,7 @@ void nc_destroy(nc_ctx* ctx) {
   for (auto& p : ctx->tmp64) cudaFree(p);
   for (auto& p : ctx->tmp32) cudaFree(p);
   cudaFree(ctx->cjel);
+  cudaFree(ctx->gj);
   for (auto& p : ctx->filt) cudaFree(p);
   cudaFree(ctx->pub_lin);
   cudaFree(ctx->ref_lin);

@@ -7,8 +7,9 @@
 //   1. a kernel computes every column of every element Jacobian J_e in FP64
 //      (the element tangent with unit directions; Dirichlet columns are zero),
 //   2. the host assembles the dense matrix (Dirichlet rows identity, Dirichlet
-//      columns removed from interior rows, the same operator as nc_jvp) and
-//      inverts it by Gauss-Jordan elimination with partial pivoting in FP64,
+//      columns removed from interior rows, the same operator as nc_jvp); it is
+//      inverted by Gauss-Jordan elimination with partial pivoting in FP64, on the host
+//      for the smallest systems, else on the device,
 //   3. the inverse (in the cycle's precision) is applied with one dense
 //      matrix-vector kernel: one warp per row, fixed-order shuffle reduction; the
 //      transpose is stored after it, so that the adjoint's cycle reads rows too (a
@@ -117,6 +118,203 @@ bool gauss_jordan_inverse(std::vector<double>& A, int n) {
   return true;
 }
 
+// ---- the same elimination on the device
+// The largest candidate for a pivot among a block's rows, with its sign.
+struct GjCand {
+  double v;
+  int row, pad;
+};
+constexpr int GJ_W = 8;  // rows per block, a warp each
+
+// Whether candidate (v, row) goes before (w, row2): larger in size, ties to the first row.
+__device__ __forceinline__ bool gj_before(double v, int row, double w, int row2) {
+  return fabs(v) > fabs(w) || (fabs(v) == fabs(w) && row < row2);
+}
+
+// Step p: in -> out (n x n each, n <= 32 NV), a launch per step, a warp per row.  cin
+// holds every block's candidate of column p, cout gets those of column p + 1, perm[p] the
+// pivot row; *bad is set where a pivot vanishes or is not finite.  p = -1 only finds the
+// first candidates.  A step is a chain of three trips to L2 (candidates, pivot row, rows);
+// a row is loaded whole while the candidates are compared, and the one division is done by
+// one warp (a division by every thread costs as much as the update).
+template <int NV>
+__global__ void __launch_bounds__(32 * GJ_W) k_gj_step(int n, int p, const double* in_, double* out,
+                                                       const GjCand* cin_, GjCand* cout, int* perm, int* bad) {
+  chained();
+  const double* const in = fresh(in_);
+  const GjCand* const cin = fresh(cin_);
+  __shared__ double rp[32 * NV];  // the scaled pivot row
+  __shared__ double inv_s;
+  __shared__ int q_s;
+  __shared__ GjCand cand[GJ_W];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, i = blockIdx.x * GJ_W + w;
+  double v[NV];
+#pragma unroll
+  for (int k = 0; k < NV; ++k) v[k] = i < n && 32 * k + lane < n ? in[(size_t)i * n + 32 * k + lane] : 0.0;
+  if (p >= 0) {
+    if (w == 0) {
+      double c = 0.0;
+      int row = n;
+      bool nan = false;
+      for (int b = lane; b < (int)gridDim.x; b += 32) {
+        const GjCand x = cin[b];
+        nan |= x.v != x.v;
+        if (gj_before(x.v, x.row, c, row)) {
+          c = x.v;
+          row = x.row;
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double c2 = __shfl_xor_sync(0xffffffffu, c, o);
+        const int r2 = __shfl_xor_sync(0xffffffffu, row, o);
+        if (gj_before(c2, r2, c, row)) {
+          c = c2;
+          row = r2;
+        }
+      }
+      nan = __any_sync(0xffffffffu, nan);
+      const double inv = 1.0 / c;
+      if (lane == 0) {
+        inv_s = inv;
+        q_s = row < n ? row : p;
+        if (blockIdx.x == 0) {
+          perm[p] = q_s;
+          if (nan || c == 0.0 || !isfinite(c)) *bad = 1;
+        }
+      }
+    }
+    __syncthreads();
+    const int q = q_s;
+    const double inv = inv_s;
+    for (int j = threadIdx.x; j < n; j += 32 * GJ_W) rp[j] = (j == p ? 1.0 : in[(size_t)q * n + j]) * inv;
+    if (i == q && q != p) {  // the row that the interchange puts here
+#pragma unroll
+      for (int k = 0; k < NV; ++k) v[k] = 32 * k + lane < n ? in[(size_t)p * n + 32 * k + lane] : 0.0;
+    }
+    __syncthreads();
+    const double f = i < n ? in[(size_t)(i == q ? p : i) * n + p] : 0.0;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+      const int j = 32 * k + lane;
+      if (j < n) v[k] = i == p ? rp[j] : (j == p ? 0.0 : v[k]) - f * rp[j];
+    }
+    if (i < n) {
+#pragma unroll
+      for (int k = 0; k < NV; ++k)
+        if (32 * k + lane < n) out[(size_t)i * n + 32 * k + lane] = v[k];
+    }
+  }
+  if (lane == 0) cand[w] = GjCand{0.0, n, 0};
+  __syncwarp();
+  if (p + 1 < n && i < n && i >= p + 1) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k)
+      if (32 * k + lane == p + 1) cand[w] = GjCand{v[k], i, 0};
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    GjCand best = cand[0];
+    for (int k = 1; k < GJ_W; ++k)
+      if (cand[k].v != cand[k].v || gj_before(cand[k].v, cand[k].row, best.v, best.row)) best = cand[k];
+    cout[blockIdx.x] = best;
+  }
+}
+
+// Column of the eliminated matrix that each column of the inverse is: the row
+// interchanges undone as column interchanges, in reverse order.
+__global__ void k_gj_columns(int n, const int* perm_, int* map) {
+  chained();
+  const int* const perm = fresh(perm_);
+  extern __shared__ int m[];
+  for (int j = threadIdx.x; j < n; j += blockDim.x) {
+    m[j] = j;
+    m[n + j] = perm[j];
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int p = n - 1; p >= 0; --p) {
+      const int q = m[n + p], t = m[p];
+      m[p] = m[q];
+      m[q] = t;
+    }
+  __syncthreads();
+  for (int j = threadIdx.x; j < n; j += blockDim.x) map[j] = m[j];
+}
+
+// The inverse and its transpose in the cycle's precision.
+template <typename R>
+__global__ void k_gj_store(int n, const double* A_, const int* map_, R* inv) {
+  chained();
+  const double* const A = fresh(A_);
+  const int* const map = fresh(map_);
+  const int j = blockIdx.x * blockDim.x + threadIdx.x, i = blockIdx.y;
+  if (j >= n) return;
+  const R v = R(A[(size_t)i * n + map[j]]);
+  inv[(size_t)i * n + j] = v;
+  inv[(size_t)n * n + (size_t)j * n + i] = v;
+}
+
+// Smallest system inverted on the device.  The device pays 7 to 9 us a pivot (launch and
+// three trips to L2; 2.2 us of it are the n^2 operations at n = 1000), one core 2 n^3
+// operations out of its cache.  Linearisation of a one-level hierarchy, host / device:
+// n = 320 1.2 / 2.2 ms, 400 2.0 / 2.8, 500 4.5 / 3.6, 560 5.6 / 4.6, 750 18 / 6.7,
+// 1000 46 / 10.8 ms.
+constexpr int GJ_DEVICE_MIN = 480;
+static_assert(COARSE_DENSE_MAX <= 32 * 32, "a lane of k_gj_step holds at most 32 entries of a row");
+
+// inv_dev <- the inverse of the host matrix A (overwritten) and its transpose.
+template <typename R>
+nc_status invert(nc_ctx* ctx, std::vector<double>& A, int n, R* inv_dev, const char* singular, cudaStream_t s) {
+  nc_status st;
+  if (n >= GJ_DEVICE_MIN) {
+    const int blocks = (n + GJ_W - 1) / GJ_W;
+    const size_t nn = (size_t)n * n, need = sizeof(double) * 2 * nn + sizeof(GjCand) * 2 * blocks +
+                                            sizeof(int) * (2 * (size_t)n + 1);
+    if (ctx->gj_bytes < need) {
+      void* p = nullptr;
+      if (cudaMalloc(&p, need) == cudaSuccess) {
+        cudaFree(ctx->gj);
+        ctx->gj = p;
+        ctx->gj_bytes = need;
+      } else {
+        cudaGetLastError();  // no room: on the host below
+      }
+    }
+    if (ctx->gj_bytes >= need) {
+      double* M[2] = {(double*)ctx->gj, (double*)ctx->gj + nn};
+      GjCand* C[2] = {(GjCand*)(M[1] + nn), (GjCand*)(M[1] + nn) + blocks};
+      int *perm = (int*)(C[1] + blocks), *map = perm + n, *bad = map + n;
+      cudaMemsetAsync(bad, 0, sizeof(int), s);
+      if ((st = cuda_check(ctx, cudaMemcpyAsync(M[0], A.data(), sizeof(double) * nn, cudaMemcpyHostToDevice, s),
+                           "coarse H2D")) != NC_OK)
+        return st;
+      const auto step = n <= 512 ? k_gj_step<16> : k_gj_step<32>;
+      for (int p = -1; p < n; ++p) {
+        const int a = p & 1, b = (p + 1) & 1;  // step -1 leaves its candidates in C[0]
+        launch(step, blocks, 32 * GJ_W, 0, s, n, p, p < 0 ? M[0] : M[a], M[b], C[a], C[b], perm, bad);
+      }
+      launch(k_gj_columns, 1, 256, 2 * sizeof(int) * n, s, n, perm, map);
+      launch(k_gj_store<R>, dim3((n + 255) / 256, n), 256, 0, s, n, M[n & 1], map, inv_dev);
+      int h = 0;
+      if ((st = cuda_check(ctx, cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, s),
+                           "coarse inverse")) != NC_OK ||
+          (st = cuda_check(ctx, cudaStreamSynchronize(s), "coarse sync")) != NC_OK)
+        return st;
+      return h ? set_err(ctx, NC_ERR_NAN, singular) : NC_OK;
+    }
+  }
+  if (!gauss_jordan_inverse(A, n)) return set_err(ctx, NC_ERR_NAN, singular);
+  std::vector<R> Ar(A.begin(), A.end());
+  Ar.resize((size_t)2 * n * n);
+  for (int i = 0; i < n; ++i)
+    for (int j = 0; j < n; ++j) Ar[(size_t)n * n + (size_t)j * n + i] = Ar[(size_t)i * n + j];
+  if ((st = cuda_check(ctx, cudaMemcpyAsync(inv_dev, Ar.data(), sizeof(R) * Ar.size(),
+                                            cudaMemcpyHostToDevice, s), "coarse H2D")) != NC_OK)
+    return st;
+  return cuda_check(ctx, cudaStreamSynchronize(s), "coarse sync");
+}
+
 }  // namespace
 
 int coarse_dense_dofs(const Level& L) { return (int)(5 * L.d.Nn); }
@@ -177,16 +375,7 @@ nc_status coarse_setup(nc_ctx* ctx, Level& L, const R* x, const R* gam, const R*
         for (int c = 0; c < n; ++c) A[(size_t)r * n + c] = 0.0;
         A[(size_t)r * n + r] = 1.0;
       }
-  if (!gauss_jordan_inverse(A, n))
-    return set_err(ctx, NC_ERR_NAN, "coarsest-level operator is singular");
-  std::vector<R> Ar(A.begin(), A.end());
-  Ar.resize((size_t)2 * n * n);
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) Ar[(size_t)n * n + (size_t)j * n + i] = Ar[(size_t)i * n + j];
-  if ((st = cuda_check(ctx, cudaMemcpyAsync(*inv_dev, Ar.data(), sizeof(R) * Ar.size(),
-                                            cudaMemcpyHostToDevice, s), "coarse H2D")) != NC_OK)
-    return st;
-  return cuda_check(ctx, cudaStreamSynchronize(s), "coarse sync");
+  return invert(ctx, A, n, *inv_dev, "coarsest-level operator is singular", s);
 }
 
 template <typename R>
@@ -221,16 +410,7 @@ nc_status coarse_setup_stencil(nc_ctx* ctx, Level& L, const R* S, R** inv_dev, c
               (double)sh[(size_t)((o * 5 + f) * 5 + g) * Nn + node];
     }
   }
-  if (!gauss_jordan_inverse(A, n))
-    return set_err(ctx, NC_ERR_NAN, "coarsest-level Galerkin operator is singular");
-  std::vector<R> Ar(A.begin(), A.end());
-  Ar.resize((size_t)2 * n * n);
-  for (int i = 0; i < n; ++i)
-    for (int j = 0; j < n; ++j) Ar[(size_t)n * n + (size_t)j * n + i] = Ar[(size_t)i * n + j];
-  if ((st = cuda_check(ctx, cudaMemcpyAsync(*inv_dev, Ar.data(), sizeof(R) * Ar.size(),
-                                            cudaMemcpyHostToDevice, s), "coarse H2D")) != NC_OK)
-    return st;
-  return cuda_check(ctx, cudaStreamSynchronize(s), "coarse sync");
+  return invert(ctx, A, n, *inv_dev, "coarsest-level Galerkin operator is singular", s);
 }
 
 template <typename R>

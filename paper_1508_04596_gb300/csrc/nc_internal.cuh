@@ -164,6 +164,8 @@ struct nc_ctx {
   int ws_ks = 0;              // smoother workspace size allocated
   double* cjel = nullptr;     // coarsest-level element Jacobians (40 x 40 per element)
   long long cjel_elems = 0;
+  void* gj = nullptr;         // the coarsest level's dense inversion on the device
+  size_t gj_bytes = 0;
   cudaStream_t cap = nullptr; // stream used to capture the V-cycle graph
   double* filt[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // filter CG
   double* pub_lin = nullptr;  // linearisation of nc_linearize (level 0, FP64)
