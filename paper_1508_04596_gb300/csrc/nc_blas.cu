@@ -135,19 +135,6 @@ __global__ void k_waxpy(long long n, const R* __restrict__ x, R a, const R* __re
 }
 
 template <typename R, bool VEC>
-__global__ void k_div(long long n, const R* __restrict__ x, const R* __restrict__ d,
-                      R* __restrict__ y) {
-  chunk_loop(n, [&](long long c) {
-    R xv[4], dv[4];
-    ld4<R, VEC>(x, c, xv);
-    ld4<R, VEC>(d, c, dv);
-#pragma unroll
-    for (int u = 0; u < 4; ++u) xv[u] /= dv[u];
-    st4<R, VEC>(y, c, xv);
-  }, [&](long long i) { y[i] = x[i] / d[i]; });
-}
-
-template <typename R, bool VEC>
 __global__ void k_scal(long long n, R a, R* __restrict__ y) {
   chunk_loop(n, [&](long long c) {
     R yv[4];
@@ -573,13 +560,6 @@ void vwaxpy(long long n, const R* x, R a, const R* y, R* w, cudaStream_t s) {
     k_waxpy<R, false><<<map_blocks(n), VT, 0, s>>>(n, x, a, y, w);
 }
 template <typename R>
-void vdiv(long long n, const R* x, const R* d, R* y, cudaStream_t s) {
-  if (al16(x) && al16(d) && al16(y))
-    k_div<R, true><<<map_blocks(n), VT, 0, s>>>(n, x, d, y);
-  else
-    k_div<R, false><<<map_blocks(n), VT, 0, s>>>(n, x, d, y);
-}
-template <typename R>
 void vscal(long long n, R a, R* y, cudaStream_t s) {
   if (al16(y))
     k_scal<R, true><<<map_blocks(n), VT, 0, s>>>(n, a, y);
@@ -672,7 +652,6 @@ template void vcast<double, float>(long long, const float*, double*, cudaStream_
   template void vaxpy<R>(long long, R, const R*, R*, cudaStream_t);                            \
   template void vxpay<R>(long long, const R*, R, R*, cudaStream_t);                            \
   template void vwaxpy<R>(long long, const R*, R, const R*, R*, cudaStream_t);                 \
-  template void vdiv<R>(long long, const R*, const R*, R*, cudaStream_t);                      \
   template void vscal<R>(long long, R, R*, cudaStream_t);                                      \
   template void vmdot<R>(long long, int, const R*, long long, const R*, double*, double*,      \
                          cudaStream_t);                                                        \

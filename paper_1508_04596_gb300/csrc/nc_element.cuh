@@ -21,7 +21,11 @@
 // This header provides, for one element, the residual, its tangent (J v, with
 // the dtau/du_e term of App. B), its adjoint (J^T w), the diagonal of J_e and
 // the design derivative lambda^T dr_e/dgamma_e (with dtau/dgamma_e).  It is
-// plain arithmetic on register arrays, usable from host and device code.
+// plain arithmetic on register arrays, usable from host and device code.  The device
+// operators work on faces of elements that share their stages with the neighbours
+// (nc_march.cuh), on the coefficients and point fluxes below; the whole-element forms
+// (elem_jvp, elem_diag in the dense coarse matrix, the FP32 assembly and the diagonal; the
+// others on the host only) state what these must equal.
 //
 // Scaling.  Point gradients are kept in reference units, h grad (the nodal
 // differences of the tensor-product stages, with no division by h), and so are

@@ -15,6 +15,8 @@
 //    with the element coefficients broadcast to both lanes;
 //  * the test side (test8) mirrors the interpolation: a scalar x stage from
 //    point pairs to node pairs, then packed y and z stages.
+// The marching kernels (nc_march.cuh) take the pair arithmetic and the point fluxes from
+// here; the whole-element products below are the form that the host check compares.
 // The result equals elem_jvp<float> / elem_jtvp<float> up to FP32 rounding
 // (different order of some sums); the host check compares them.
 //

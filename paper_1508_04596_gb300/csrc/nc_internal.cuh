@@ -281,8 +281,6 @@ void vxpay(long long n, const R* x, R a, R* y, cudaStream_t s);  // y = x + a y
 template <typename R>
 void vwaxpy(long long n, const R* x, R a, const R* y, R* w, cudaStream_t s);  // w = x + a y
 template <typename R>
-void vdiv(long long n, const R* x, const R* d, R* y, cudaStream_t s);  // y = x / d
-template <typename R>
 void vscal(long long n, R a, R* y, cudaStream_t s);  // y = a y
 // Multivectors X_i = X + i*ld are stored with ld = mv_ld(n), a multiple of 64
 // elements, so that every column starts on a 256-byte boundary.
