@@ -59,23 +59,32 @@ bool valid_bcs(const nc_params& p, const nc_bcs* b, std::string& why) {
   return true;
 }
 
+// Allocated once, for the finest level, so that a captured nc_assemble stays valid; the
+// allocation itself may fall into a capture.  FP32 can do without (op_assemble), and does
+// so rather than leave less than 8 GB free.
 template <typename R>
-R* assembly_store(nc_ctx* ctx, long long E) {
-  const size_t need = sizeof(R) * (size_t)LIN_SLOTS * (size_t)E;
-  if (ctx->asm_lin_bytes < need) {
-    void* p = nullptr;
-    if (cudaMalloc(&p, need) != cudaSuccess) {
+R* assembly_store(nc_ctx* ctx) {
+  constexpr bool fp32 = sizeof(R) == 4;
+  void*& store = fp32 ? ctx->asm_lin32 : ctx->asm_lin;
+  if (!store) {
+    const size_t need = sizeof(R) * (size_t)LIN_SLOTS * (size_t)ctx->lv[0].d.E;
+    size_t fr = 0, tot = 0;
+    if (fp32 && (cudaMemGetInfo(&fr, &tot) != cudaSuccess || fr < need + ((size_t)8 << 30))) {
       cudaGetLastError();
       return nullptr;
     }
-    cudaFree(ctx->asm_lin);
-    ctx->asm_lin = p;
-    ctx->asm_lin_bytes = need;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (cudaMalloc(&store, need) != cudaSuccess) {
+      cudaGetLastError();
+      store = nullptr;
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
   }
-  return (R*)ctx->asm_lin;
+  return (R*)store;
 }
-template double* assembly_store<double>(nc_ctx*, long long);
-template float* assembly_store<float>(nc_ctx*, long long);
+template double* assembly_store<double>(nc_ctx*);
+template float* assembly_store<float>(nc_ctx*);
 
 }  // namespace nc
 
@@ -222,6 +231,7 @@ void nc_destroy(nc_ctx* ctx) {
   cudaFree(ctx->pub_lin);
   cudaFree(ctx->ref_lin);
   cudaFree(ctx->asm_lin);
+  cudaFree(ctx->asm_lin32);
   cudaFree(ctx->mma_ws);
   if (ctx->cap) cudaStreamDestroy(ctx->cap);
   delete ctx;
@@ -426,13 +436,13 @@ nc_status nc_assemble(nc_ctx* ctx, const void* x, const void* gam, void* S, int 
   const Level& L = ctx->lv[0];
   cudaStream_t s = (cudaStream_t)stream;
   if (prec == NC_FP64) {
-    double* lin = assembly_store<double>(ctx, L.d.E);
+    double* lin = assembly_store<double>(ctx);
     if (!lin) return set_err(ctx, NC_ERR_OOM, "nc_assemble: linearisation store");
     op_linearize<double>(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src, lin, s);
     op_assemble<double>(L.d, L.c64, (const double*)x, (const double*)gam, L.f64.src, lin, (double*)S,
                         ctx->Y, s);
   } else {
-    float* lin = assembly_store<float>(ctx, L.d.E);
+    float* lin = assembly_store<float>(ctx);
     if (lin) op_linearize<float>(L.d, L.c32, (const float*)x, (const float*)gam, L.f32.src, lin, s);
     op_assemble<float>(L.d, L.c32, (const float*)x, (const float*)gam, L.f32.src, lin, (float*)S,
                        (float*)ctx->Y, s);

@@ -169,8 +169,8 @@ struct nc_ctx {
   cudaStream_t cap = nullptr; // stream used to capture the V-cycle graph
   double* filt[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // filter CG
   double* pub_lin = nullptr;  // linearisation of nc_linearize (level 0, FP64)
-  void* asm_lin = nullptr;    // linearisation store of an assembly (FP64: nc_assemble; FP32: any level)
-  size_t asm_lin_bytes = 0;
+  void* asm_lin = nullptr;    // linearisation store of nc_assemble in FP64
+  void* asm_lin32 = nullptr;  // of the FP32 assemblies, all levels in turn
   double* ref_lin = nullptr;  // linearisation of the mixed adjoint's FP64 refinement (level 0)
   void* mma_ws = nullptr;     // coefficient workspace of nc_mma_update
   size_t mma_ws_bytes = 0;
@@ -353,7 +353,7 @@ void op_assemble(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* 
 // The context's linearisation store for assemblies, LIN_SLOTS * E values of R; null if
 // there is no memory for it (nc_api.cu).
 template <typename R>
-R* assembly_store(nc_ctx* ctx, long long E);
+R* assembly_store(nc_ctx* ctx);
 template <typename R>
 void op_stencil(const LevelDev& d, const R* S, bool tr, const R* v, R* out, cudaStream_t s);
 template <typename R>

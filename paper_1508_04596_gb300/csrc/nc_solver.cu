@@ -224,7 +224,7 @@ nc_status linearize(nc_ctx* ctx, int nlev, const double* x, const double* gam, c
       op_stencil_diag<R>(L.d, B.gst, B.diag, s);
     } else if (assembled) {
       R* lin = B.lin;
-      if (!lin && sizeof(R) == sizeof(float)) lin = assembly_store<R>(ctx, L.d.E);
+      if (!lin && sizeof(R) == sizeof(float)) lin = assembly_store<R>(ctx);
       if (lin) op_linearize<R>(L.d, cst<R>(L), B.x, B.gam, B.src, lin, s);
       op_assemble<R>(L.d, cst<R>(L), B.x, B.gam, B.src, lin, B.gst, (R*)ctx->Y, s);
       op_stencil_diag<R>(L.d, B.gst, B.diag, s);

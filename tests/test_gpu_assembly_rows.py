@@ -36,3 +36,25 @@ def test_rows_match_products(dims, g_dir, dt, tol):
             ref = f(x, gam, v).double()
             got = gp.stencil_apply(S, v, transpose=tr).double()
             assert (got - ref).norm() <= tol * ref.norm(), tr
+
+
+def test_first_call_under_capture():
+    """An FP32 assembly captured as a context's first one, replayed after an FP64 assembly."""
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1508_04596_gb300 import nc
+    params, bcs = nc.make_params(12, 7, 9, 1.0 / 12, 1e4, 0.71), nc.cavity_bcs()
+    gp, other = nc.Problem(params, bcs), nc.Problem(params, bcs)
+    rng = np.random.default_rng(5)
+    x = torch.tensor(rng.standard_normal(gp.ndof), dtype=torch.float32, device="cuda")
+    gam = torch.tensor(rng.uniform(0, 1, gp.E), dtype=torch.float32, device="cuda")
+    S = torch.zeros(675 * gp.Nn, dtype=torch.float32, device="cuda")
+    other.assemble(x, gam)  # loads the kernels
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        gp.assemble(x, gam, S)
+    gp.assemble(x.double(), gam.double())
+    x.mul_(0.5)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(S, other.assemble(x, gam))
