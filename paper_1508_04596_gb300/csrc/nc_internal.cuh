@@ -333,6 +333,11 @@ constexpr int HD_SIG2 = HD_Y + LDH;
 constexpr int HD_ISIG = HD_SIG2 + LDH;
 constexpr int HD_CF = HD_ISIG + LDH;
 constexpr int HD_SIZE = HD_CF + LDH;
+// z (+)= Jacobi-GMRES(k) for A z = b on a small level in one kernel (nc_block.cu), and
+// r = b - A z if r is given; false where the level does not qualify.
+constexpr int SMOOTH_BLOCK_MAX = 512;  // elements
+bool smooth_block(const LevelDev& d, const ElemConst<float>& c, const LevelBuf<float>& B, bool tr, int k, bool zero,
+                  float* r, cudaStream_t s);
 // The smoother's small least-squares problem (nc_smooth.cu): Hd[HD_Y..] from the rest.
 void small_ls(double* Hd, int k, cudaStream_t s);
 template <typename R>

@@ -77,12 +77,16 @@ void level_apply(nc_ctx* ctx, int l, bool tr, const R* v, R* out, cudaStream_t s
 // norms into the normalised Hessenberg.  Per Arnoldi step three kernels: the element product of
 // t = D^-1 v_j, the gather of w with its dots, and one pass that orthogonalises,
 // rescales, forms the next t and the new norm.
+// With r the residual b - A z is left there.
 template <typename R>
-void smooth(nc_ctx* ctx, int l, bool tr, int k, bool zero_init, cudaStream_t s) {
+void smooth(nc_ctx* ctx, int l, bool tr, int k, bool zero_init, cudaStream_t s, R* r = nullptr) {
   Level& L = ctx->lv[l];
   LevelBuf<R>& B = buf<R>(L);
   const long long n = 5 * L.d.Nn;
   const long long ld = mv_ld(n);
+  if constexpr (std::is_same<R, float>::value) {
+    if (!B.use_gst && smooth_block(L.d, L.c32, B, tr, k, zero_init, r, s)) return;
+  }
   R* V = B.V;
   double* Hd = B.Hd;
   if (zero_init) {
@@ -109,6 +113,11 @@ void smooth(nc_ctx* ctx, int l, bool tr, int k, bool zero_init, cudaStream_t s) 
   }
   // z (+)= D^-1 (V y)
   vcombine(n, k, (const R*)V, ld, Hd + HD_Y, (const R*)B.diag, B.z, !zero_init, s);
+  if (r) {
+    Dots<R> res;
+    res.b = B.b;
+    level_apply<R>(ctx, l, tr, B.z, r, s, &res);
+  }
 }
 
 template <typename R>
@@ -122,10 +131,7 @@ void vcycle(nc_ctx* ctx, int l, int nlev, bool tr, const nc_solve_opts& o, cudaS
       smooth<R>(ctx, l, tr, o.coarse_its, true, s);
     return;
   }
-  smooth<R>(ctx, l, tr, o.smooth_its, true, s);
-  Dots<R> res;
-  res.b = B.b;
-  level_apply<R>(ctx, l, tr, B.z, B.r, s, &res);  // r = b - A z
+  smooth<R>(ctx, l, tr, o.smooth_its, true, s, B.r);  // r = b - A z
   Level& C = ctx->lv[l + 1];
   op_restrict<R>(L.d, B.r, C.d, buf<R>(C).b, s);
   vcycle<R>(ctx, l + 1, nlev, tr, o, s);
