@@ -51,9 +51,9 @@ PEAK_SOURCE = ("unit counts x max SM clock: 152 SMs x 128 FP32 lanes (2 FP64 FMA
 # DRAM traffic of one launch of the headline element kernel, from an ncu capture
 # at the benchmark's workload; used only while the kernel sources are the ones
 # the capture was taken with (their SHA-256 is recorded beside the figure).
-TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_elem_lin_cached_tall192x192x384_traffic.txt")
+TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_march_jvp_lin_tall192x192x384_traffic.txt")
 KERNEL_SOURCES = [os.path.join(ROOT, "paper_1508_04596_gb300", "csrc", f)
-                  for f in ("nc_kernels.cu", "nc_element.cuh", "nc_internal.cuh")]
+                  for f in ("nc_kernels.cu", "nc_march.cuh", "nc_element.cuh", "nc_internal.cuh")]
 
 
 def parse():
@@ -412,8 +412,8 @@ def run_ours(args, rank, world):
     roof = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak, 3),
             "unit": "TFLOP/s", "frac": round(achieved / peak, 4),
             "traffic": traffic, "traffic_source": traffic_src,
-            "kernel": ("k_elem_lin_cached<double> + k_gather, k_elem_linearize once per step"
-                       if args.prec == "f64" else "k_elem_lin<float> + k_gather"),
+            "kernel": ("k_march<double, JVP_LIN> + k_gather_march, k_march<double, LINEARIZE> once per step"
+                       if args.prec == "f64" else "k_march<float, JVP> + k_gather_march"),
             "achieved_over": "the whole step (element kernel, gather and linearisation)",
             "peak_source": PEAK_SOURCE,
             "peak_probe": extra["alu_probe"][args.prec]["tflops"],
