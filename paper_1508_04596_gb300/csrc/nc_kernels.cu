@@ -21,6 +21,7 @@ namespace {
 
 constexpr int ELEM_THREADS = 128;
 constexpr int NODE_THREADS = 256;
+constexpr unsigned PROLONG_BLOCKS = 8 * 152;  // blocks that fill the GPU: a thread per node from here
 
 inline unsigned nblocks(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
@@ -330,7 +331,8 @@ __global__ void k_source_grad(LevelDev d, const double* __restrict__ src, double
 }
 
 // A thread per node and field (blockIdx.y): with a thread per node the coarse levels
-// are too few threads to hide the latency of 27 x 5 loads (64^3 -> 32^3: 21 us, 9 now).
+// are too few threads to hide the latency of 27 x 5 loads (64^3 -> 32^3: 21 us, 9 now),
+// and on fine ones its registers leave too few warps (192x192x384 429 us, 246).
 template <typename R>
 __global__ void k_restrict(LevelDev f, const R* __restrict__ rf, LevelDev c, R* __restrict__ rc) {
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -341,15 +343,28 @@ __global__ void k_restrict(LevelDev f, const R* __restrict__ rf, LevelDev c, R* 
   rc[q * c.Nn + n] = restrict_value(f, rf + q * f.Nn, q, c.flag[n], I, J, K);
 }
 
-template <typename R>
-__global__ void k_prolong_add(LevelDev c, const R* __restrict__ zc, LevelDev f, R* zf) {
+// A thread per node with Q = 5, per node and field (blockIdx.y) with Q = 1: where the
+// nodes fill the GPU, five threads only repeat the index arithmetic and the branches
+// (192x192x384 482 us, 266 with a thread per node; 96x96x192 63 and 36).
+template <typename R, int Q>
+__global__ void k_prolong_add(LevelDev c, const R* __restrict__ zc, LevelDev f, R* __restrict__ zf) {
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= f.Nn) return;
-  const int q = blockIdx.y;
   int i, j, k;
   node_ijk(f, n, i, j, k);
-  if ((f.flag[n] >> q) & 1) return;
-  zf[q * f.Nn + n] += prolong_value(c, zc + q * c.Nn, i, j, k);
+  const uint8_t fl = f.flag[n];
+  R v[Q], z[Q];
+#pragma unroll
+  for (int u = 0; u < Q; ++u) {
+    const int q = Q * blockIdx.y + u;
+    z[u] = zf[q * f.Nn + n];
+    v[u] = prolong_value(c, zc + q * c.Nn, i, j, k);
+  }
+#pragma unroll
+  for (int u = 0; u < Q; ++u) {
+    const int q = Q * blockIdx.y + u;
+    if (!((fl >> q) & 1)) zf[q * f.Nn + n] = z[u] + v[u];
+  }
 }
 
 template <typename R>
@@ -568,7 +583,11 @@ void op_restrict(const LevelDev& fine, const R* rf, const LevelDev& coarse, R* r
 template <typename R>
 void op_prolong_add(const LevelDev& coarse, const R* zc, const LevelDev& fine, R* zf,
                     cudaStream_t s) {
-  k_prolong_add<R><<<dim3(nblocks(fine.Nn, NODE_THREADS), NF), NODE_THREADS, 0, s>>>(coarse, zc, fine, zf);
+  const unsigned nb = nblocks(fine.Nn, NODE_THREADS);
+  if (nb >= PROLONG_BLOCKS)
+    k_prolong_add<R, NF><<<nb, NODE_THREADS, 0, s>>>(coarse, zc, fine, zf);
+  else
+    k_prolong_add<R, 1><<<dim3(nb, NF), NODE_THREADS, 0, s>>>(coarse, zc, fine, zf);
 }
 template <typename R>
 void op_inject(const LevelDev& fine, const R* xf, const LevelDev& coarse, R* xc, cudaStream_t s) {
