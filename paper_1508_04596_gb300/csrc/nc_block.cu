@@ -36,6 +36,16 @@ struct BlockSmooth {
 // Shared floats: k + 1 basis vectors, t, x and D, then 40 rows per element.
 inline long long block_floats(const LevelDev& d, int k) { return (k + 4LL) * 5 * d.Nn + 40 * d.E; }
 
+struct BlockScalars {
+  double H[BK * (BK + 1)], sig2[BK + 1], isig[BK + 1], y[BK + 1], g[BK + 1];
+  float warp[BW][BK], cf[BK], sc;
+};
+// What the dynamic part may take: 227 KB a block less the scalars.  The attribute that
+// allows it belongs to the kernel, not to a context, and solves on other threads set it
+// too, so every launch sets this value and not its own size.
+constexpr int BLOCK_BYTES = 227 * 1024 - 1280;
+static_assert(sizeof(BlockScalars) <= 1280, "the scalars fit what BLOCK_BYTES leaves");
+
 template <bool TR>
 __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ BlockSmooth a) {
   chained();
@@ -44,9 +54,12 @@ __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ 
   const float* const gam = fresh(a.gam);
   const float* const src = a.src ? fresh(a.src) : nullptr;
   extern __shared__ float sm[];
-  __shared__ float warp[BW][BK];
-  __shared__ double H[BK * (BK + 1)], sig2[BK + 1], isig[BK + 1], y[BK + 1], g[BK + 1];
-  __shared__ float cf[BK], sc;
+  __shared__ BlockScalars sh;
+  auto& H = sh.H;
+  double *const sig2 = sh.sig2, *const isig = sh.isig, *const y = sh.y, *const g = sh.g;
+  auto& warp = sh.warp;
+  float* const cf = sh.cf;
+  float& sc = sh.sc;
   const int Nn = (int)a.d.Nn, N = 5 * Nn, E = (int)a.d.E, k = a.k;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int sx = a.d.nx + 1, sy = a.d.ny + 1;
@@ -218,9 +231,9 @@ __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ 
 bool smooth_block(const LevelDev& d, const ElemConst<float>& c, const LevelBuf<float>& B, bool tr, int k, bool zero,
                   float* r, cudaStream_t s) {
   const long long bytes = 4 * block_floats(d, k);
-  if (k > BK || d.E > SMOOTH_BLOCK_MAX || bytes > 226 * 1024) return false;
+  if (k > BK || d.E > SMOOTH_BLOCK_MAX || bytes > BLOCK_BYTES) return false;
   const auto kernel = tr ? k_smooth_block<true> : k_smooth_block<false>;
-  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) {
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, BLOCK_BYTES) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
