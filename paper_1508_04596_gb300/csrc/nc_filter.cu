@@ -333,6 +333,7 @@ extern "C" nc_status nc_filter(nc_ctx* ctx, const double* rho, double* gamma_f, 
   const HelmCoef c = helm_coef(d.h, radius);
   CgState* cg = (CgState*)ctx->dscal;
   static_assert(sizeof(CgState) <= sizeof(double) * (MAX_RESTART + 2) * 4, "dscal holds the state");
+  cudaGetLastError();  // below, only this call's launches are meant
   cudaMemsetAsync(cg, 0, sizeof(CgState), s);
   const unsigned vb = (unsigned)std::min<long long>((Nn + FT - 1) / FT, RED_BLOCKS_MAX);
   k_cg_rhs<<<vb, FT, 0, s>>>(d, c, rho, r, x, ctx->partial, cg);
@@ -346,7 +347,9 @@ extern "C" nc_status nc_filter(nc_ctx* ctx, const double* rho, double* gamma_f, 
       k_cg_update<<<vb, FT, 0, s>>>(d, c, p[(m + 1) & 1], q, x, r, ctx->partial, cg);
     }
     k_elem_mean<<<fblocks(d.E), FT, 0, s>>>(d, x, gamma_f, cg);
-    if ((st = cuda_check(ctx, cudaMemcpyAsync(&h, cg, sizeof(h), cudaMemcpyDeviceToHost, s),
+    // a refused launch would leave the state, which ends the loop, as it is
+    if ((st = cuda_check(ctx, cudaGetLastError(), "nc_filter")) != NC_OK ||
+        (st = cuda_check(ctx, cudaMemcpyAsync(&h, cg, sizeof(h), cudaMemcpyDeviceToHost, s),
                          "nc_filter")) != NC_OK ||
         (st = cuda_check(ctx, cudaStreamSynchronize(s), "nc_filter")) != NC_OK)
       return st;

@@ -525,6 +525,7 @@ nc_status nc_mma_update(nc_ctx* ctx, long long n, int iter, double* x, double* x
                   1e-5 / (o.xmax - o.xmin), o.df0_scale, f1};
   MmaSearch* srch = (MmaSearch*)ctx->dscal;
   static_assert(sizeof(MmaSearch) <= sizeof(double) * (MAX_RESTART + 2) * 4, "dscal holds the search");
+  cudaGetLastError();  // below, only this call's launches are meant
   cudaMemsetAsync(srch, 0, sizeof(MmaSearch), s);
   double* part = ctx->partial;
   if (store)
@@ -543,8 +544,10 @@ nc_status nc_mma_update(nc_ctx* ctx, long long n, int iter, double* x, double* x
       k_mma_commit<true><<<nb, MT, 0, s>>>(a, w, x, xold1, xold2, part, srch);
     else
       k_mma_commit<false><<<nb, MT, 0, s>>>(a, w, x, xold1, xold2, part, srch);
-    nc_status st = cuda_check(ctx, cudaMemcpyAsync(&h, srch, sizeof(h), cudaMemcpyDeviceToHost, s),
-                              "nc_mma_update");
+    // a refused launch would leave the state, which ends the loop, as it is
+    nc_status st = cuda_check(ctx, cudaGetLastError(), "nc_mma_update");
+    if (st == NC_OK)
+      st = cuda_check(ctx, cudaMemcpyAsync(&h, srch, sizeof(h), cudaMemcpyDeviceToHost, s), "nc_mma_update");
     if (st == NC_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "nc_mma_update");
     if (st != NC_OK) return st;
   } while (!h.done);

@@ -4,6 +4,7 @@
 
 #include <cstdio>
 #include <string>
+#include <vector>
 
 #include "../../paper_1508_04596_gb300/csrc/nc_internal.cuh"
 
@@ -31,9 +32,50 @@ static int smoother_levels() {
   return bad;
 }
 
+// A context on a small grid of the stand-in's memory.
+static nc_ctx* context(int n) {
+  nc_params p = {};
+  p.nx = p.ny = p.nz = n;
+  p.h = 1.0 / n;
+  p.Gr = 1e3;
+  p.Pr = 0.71;
+  p.alpha_max = 1e4;
+  p.q_alpha = p.q_f = 1.0;
+  p.Ck = 0.1;
+  p.g_dir[2] = -1.0;
+  nc_bcs b = {};
+  b.p_pin = -1;
+  nc_ctx* ctx = nullptr;
+  if (nc_setup(&p, &b, &ctx) != NC_OK) std::exit(3);
+  return ctx;
+}
+
+// The calls whose host loop waits for the device: launches that the runtime refuses end
+// them with an error.
+static int device_loops() {
+  int bad = 0;
+  for (int n : {2, 5}) {
+    nc_ctx* ctx = context(n);
+    const long long E = (long long)n * n * n;
+    std::vector<double> v[8];
+    for (auto& q : v) q.assign(E, 0.5);
+    fake::refuse = true;
+    bad += report("nc_filter", nc_filter(ctx, v[0].data(), v[1].data(), 2.5 / n, nullptr) == NC_ERR_CUDA);
+    bad += report("nc_mma_update",
+                  nc_mma_update(ctx, E, 0, v[0].data(), v[1].data(), v[2].data(), v[3].data(), v[4].data(),
+                                v[5].data(), 0.1, v[6].data(), nullptr, nullptr, nullptr, nullptr,
+                                nullptr) == NC_ERR_CUDA);
+    bad += report("no error is left", cudaGetLastError() == cudaSuccess);
+    fake::refuse = false;
+    nc_destroy(ctx);
+  }
+  return bad;
+}
+
 int main(int argc, char** argv) {
   const std::string check = argc > 1 ? argv[1] : "";
   if (check == "smoother_levels") return smoother_levels();
+  if (check == "device_loops") return device_loops();
   std::printf("unknown check\n");
   return 2;
 }
