@@ -225,7 +225,13 @@ __global__ void __launch_bounds__(WARPS * 32, 2) k_march(LevelDev d, ElemConst<R
 
   issue(0, n, fl0);
   issue(1, n + sx, fl);
-  R gam_next = gam[e], src_next = srcs ? srcs[e] : R(0);
+  R gam_next = R(0), src_next = R(0);
+  auto load_design = [&] {
+    if (TR::VEL) return;  // the coefficients come from the store
+    gam_next = fresh(gam)[e];
+    if (srcs) src_next = fresh(srcs)[e];
+  };
+  load_design();
   copies_wait();
   consume(0, fl0, lo, s_lo, uv_lo);
 
@@ -247,8 +253,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) k_march(LevelDev d, ElemConst<R
     e += d.nx;
     if (r + 1 < rows) {
       issue(b + 1 == BUFS ? 0 : b + 1, n + sx, fl);
-      gam_next = gam[e];
-      if (srcs) src_next = srcs[e];
+      load_design();
     }
 
     // ---- element coefficients

@@ -54,7 +54,7 @@ __device__ __forceinline__ void split_chunk(const LevelDev& d, const ElemConst<R
   T dzr[5][2], vr[5][2];  // [field][row]
   R vel[TR::ADJ ? 3 : 1][2][2];
   R S = R(0), uv = R(0);
-  const R g = gam[e], s = srcs ? srcs[e] : R(0);
+  const R g = TR::VEL ? R(0) : fresh(gam)[e], s = TR::VEL || !srcs ? R(0) : fresh(srcs)[e];
 #pragma unroll
   for (int r = 0; r < 2; ++r) {
     uint8_t fl[2] = {0, 0};
