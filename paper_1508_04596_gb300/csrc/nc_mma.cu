@@ -147,6 +147,7 @@ __device__ __forceinline__ MmaCoef mma_coef_y(double xj, double l, double u, dou
   m.q1 = xl2 * (0.001 * a1p + 1.001 * a1m + r);
   m.alpha = fmax(fmax(xmin, l + 0.1 * (xj - l)), xj - move * d);
   m.beta = fmin(fmin(xmax, u - 0.1 * (u - xj)), xj + move * d);
+  m.alpha = fmin(m.alpha, m.beta);  // limits that cross (x far outside the box): the upper one holds
   return m;
 }
 

@@ -1,0 +1,53 @@
+"""nc_mma_update beyond the ordinary: variables outside the box by more than the move limit,
+whose two limits cross (the upper one holds).  Against the oracle; tolerance 1e-10 as in
+test_gpu_design_update.py (a bracket a few units in the last place wide, sums of up to 3e3
+terms, a relative slope of the constraint below 100)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-10
+
+
+@pytest.fixture(scope="module")
+def nc():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1508_04596_gb300 import nc as ncmod
+    return ncmod
+
+
+def update(nc, x, df0, f1, df1, it=0):
+    gp = nc.Problem(nc.make_params(2, 2, 2, 0.5, 1e3, 0.71), nc.cavity_bcs())
+    dev = lambda t: torch.tensor(np.asarray(t, dtype=float), dtype=torch.float64, device="cuda")  # noqa: E731
+    s = [dev(x) for _ in range(5)]
+    lam, chg = gp.mma_update(it, *s, dev(df0), f1, dev(df1))
+    return lam, chg, s[0].cpu().numpy()
+
+
+@pytest.mark.parametrize("n", [300, 3000])
+@pytest.mark.parametrize("side", ["above", "below"])
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_variables_outside_the_box(nc, n, side, sign):
+    from oracle import mma as M
+    rng = np.random.default_rng(n)
+    x = rng.uniform(0.1, 0.9, n)
+    out = rng.uniform(size=n) < 0.1
+    x[out] = rng.uniform(1.25, 1.4, out.sum()) if side == "above" else rng.uniform(-0.4, -0.25, out.sum())
+    df0 = sign * rng.uniform(0.5, 1.5, n) / n
+    df1 = -sign * rng.uniform(0.5, 1.5, n) / n
+    # the constraint value whose multiplier is near 1
+    low, upp = x - 0.5, x + 0.5
+    alpha, beta = M.bounds(x, low, upp, 0.0, 1.0, 0.2)
+    assert (alpha[out] > beta[out]).all()
+    p0, q0 = M.approx_coefficients(x, low, upp, df0, 1.0)
+    p1, q1 = M.approx_coefficients(x, low, upp, df1, 1.0)
+    y = M.y_of_lambda(1.0, low, upp, alpha, beta, p0, q0, p1, q1)
+    f1 = -M.approx_value(0.0, x, y, low, upp, p1, q1)
+    yo, _, _, lo = M.mma_step(0, x, x, x, x, x, f1, df0, df1)
+    lam, chg, X = update(nc, x, df0, f1, df1)
+    assert 0.9 < lo < 1.1 and lam == pytest.approx(lo, rel=TOL)
+    assert np.abs(X - yo).max() <= TOL
+    assert chg == pytest.approx(np.abs(yo - x).max(), abs=TOL)
