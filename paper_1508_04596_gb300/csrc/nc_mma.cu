@@ -172,12 +172,14 @@ __device__ __forceinline__ double mma_y(const MmaCoef& m, double lam) {
   return fmin(fmax((m.l * sP + m.u * sQ) / (sP + sQ), m.alpha), m.beta);
 }
 // Its term of the approximated constraint (P, Q > 0: the approximation adds 1e-5 / d).
+// Where P or Q is infinite (an infinite entry of df0), y is not a number and mma_y gives
+// alpha; the first comparison below is written so that the term goes with it.
 __device__ __forceinline__ double mma_term(const MmaCoef& m, double lam) {
   const double P = m.p0 + lam * m.p1, Q = m.q0 + lam * m.q1;
   const double rP = rsqrt(P), rQ = rsqrt(Q), sP = P * rP, sQ = Q * rQ;
   const double den = sP + sQ, num = m.l * sP + m.u * sQ;  // y = num / den
   const double t = (den * m.w) * (m.p1 * rP + m.q1 * rQ) - m.c;
-  return num <= m.alpha * den ? m.ta : (num >= m.beta * den ? m.tb : t);
+  return !(num > m.alpha * den) ? m.ta : (num >= m.beta * den ? m.tb : t);
 }
 
 // The search for the multiplier.  a is the newest point, b the end of the bracket
@@ -189,10 +191,11 @@ struct MmaSearch {
   unsigned ticket, pad;
 };
 
-// One step of the search: v = f(s.lam).
-__device__ void mma_advance(MmaSearch& s, double v) {
+// One step of the search: v = f(s.lam) = f1 + sum.
+__device__ void mma_advance(MmaSearch& s, double f1, double sum) {
+  const double v = f1 + sum;
   ++s.evals;
-  if (!isfinite(v)) {
+  if (!isfinite(sum)) {
     s.err = s.done = 1;
     return;
   }
@@ -319,7 +322,7 @@ __device__ __forceinline__ void mma_finish(double acc, double f1, double* partia
   const double sum = fold_partials<false, MT>(gridDim.x, partial);
   if (threadIdx.x == 0) {
     MmaSearch t = *s;
-    mma_advance(t, f1 + sum);
+    mma_advance(t, f1, sum);
     *s = t;
   }
 }

@@ -51,3 +51,33 @@ def test_variables_outside_the_box(nc, n, side, sign):
     assert 0.9 < lo < 1.1 and lam == pytest.approx(lo, rel=TOL)
     assert np.abs(X - yo).max() <= TOL
     assert chg == pytest.approx(np.abs(yo - x).max(), abs=TOL)
+
+
+def test_infinite_objective_gradient(nc):
+    """An infinite entry of df0 sends its variable to the lower limit, whatever its sign; the
+    others solve the subproblem with its (constant) term."""
+    from oracle import mma as M
+    rng = np.random.default_rng(8)
+    n = 700
+    x = rng.uniform(0.1, 0.9, n)
+    df0, df1 = rng.uniform(0.5, 1.5, n) / n, -rng.uniform(0.5, 1.5, n) / n
+    bad = np.arange(n) % 50 == 7
+    low, upp = x - 0.5, x + 0.5
+    alpha, _ = M.bounds(x, low, upp, 0.0, 1.0, 0.2)
+    p1, q1 = M.approx_coefficients(x, low, upp, df1, 1.0)
+    t = M.approx_value(0.0, x[bad], alpha[bad], low[bad], upp[bad], p1[bad], q1[bad])
+    f = ~bad
+    yo, _, _, lo = M.mma_step(0, x[f], x[f], x[f], x[f], x[f], 0.02 + t, df0[f], df1[f])
+    assert 1e-3 < lo < 1e3
+    df0[bad] = np.where(np.arange(bad.sum()) % 2, np.inf, -np.inf)
+    lam, chg, X = update(nc, x, df0, 0.02, df1)
+    assert lam == pytest.approx(lo, rel=TOL)
+    assert np.abs(X[f] - yo).max() <= TOL and np.abs(X[bad] - alpha[bad]).max() <= 1e-15
+    with pytest.raises(Exception):  # the constraint's gradient has no such limit
+        update(nc, x, df1, 0.02, df0)
+
+
+def test_constraint_sum_beyond_the_range(nc):
+    """Finite terms whose sum with f1 overflows: violated for every multiplier."""
+    lam, chg, X = update(nc, np.full(4, 0.5), np.full(4, 1.0), 1.2e308, np.full(4, -1e308))
+    assert lam == 2.0 ** 200 and np.abs(X - 0.3).max() <= 1e-15
