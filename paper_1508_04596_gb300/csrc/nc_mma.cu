@@ -131,6 +131,13 @@ struct MmaCoef {
 };
 constexpr int MMA_COEFS = 12;
 
+// Rounds v where it stands: what is computed from it later does not depend on whether it was
+// just computed (and could be contracted into a fused multiply-add) or read back.
+__device__ __forceinline__ double rounded(double v) {
+  asm volatile("" : "+d"(v));
+  return v;
+}
+
 // The coefficients but for w, c, ta and tb, which only the evaluations need.
 __device__ __forceinline__ MmaCoef mma_coef_y(double xj, double l, double u, double a0, double a1,
                                               double xmin, double xmax, double move, double r) {
@@ -141,10 +148,10 @@ __device__ __forceinline__ MmaCoef mma_coef_y(double xj, double l, double u, dou
   MmaCoef m;
   m.l = l;
   m.u = u;
-  m.p0 = ux2 * (1.001 * a0p + 0.001 * a0m + r);
-  m.q0 = xl2 * (0.001 * a0p + 1.001 * a0m + r);
-  m.p1 = ux2 * (1.001 * a1p + 0.001 * a1m + r);
-  m.q1 = xl2 * (0.001 * a1p + 1.001 * a1m + r);
+  m.p0 = rounded(ux2 * (1.001 * a0p + 0.001 * a0m + r));
+  m.q0 = rounded(xl2 * (0.001 * a0p + 1.001 * a0m + r));
+  m.p1 = rounded(ux2 * (1.001 * a1p + 0.001 * a1m + r));
+  m.q1 = rounded(xl2 * (0.001 * a1p + 1.001 * a1m + r));
   m.alpha = fmax(fmax(xmin, l + 0.1 * (xj - l)), xj - move * d);
   m.beta = fmin(fmin(xmax, u - 0.1 * (u - xj)), xj + move * d);
   m.alpha = fmin(m.alpha, m.beta);  // limits that cross (x far outside the box): the upper one holds
@@ -368,7 +375,8 @@ __global__ void __launch_bounds__(MT) k_mma_begin(MmaArgs a, int iter, MmaWs w, 
   mma_finish(acc, a.f1, partial, s);
 }
 
-// One evaluation of the approximated constraint at the search's multiplier.
+// One evaluation of the approximated constraint at the search's multiplier, with the same
+// bits whether the coefficients come from the workspace (STORE) or from the variables.
 template <bool STORE>
 __global__ void __launch_bounds__(MT) k_mma_dual(MmaArgs a, MmaWs w, double* partial, MmaSearch* s) {
   if (s->done) return;
@@ -379,10 +387,21 @@ __global__ void __launch_bounds__(MT) k_mma_dual(MmaArgs a, MmaWs w, double* par
     const long long base = (long long)blockIdx.x * w.seg;
     for (int i = threadIdx.x; i < cnt; i += MT) acc += mma_term(ws_load<true>(w, base + i), lam);
   } else {
-    for (long long j = blockIdx.x * (long long)MT + threadIdx.x; j < a.n; j += (long long)gridDim.x * MT)
-      if (!a.active || a.active[j])
-        acc += mma_term(mma_coef(a.x[j], a.low[j], a.upp[j], a.scale0 * a.df0[j], a.df1[j], a.xmin,
-                                 a.xmax, a.move, a.r), lam);
+    // the same sums in the same order: a term goes to the thread that would read its entry
+    __shared__ double term[MT];
+    int at = 0;  // active variables of the block so far, modulo MT
+    for (long long j0 = blockIdx.x * (long long)MT; j0 < a.n; j0 += (long long)gridDim.x * MT) {
+      const long long j = j0 + threadIdx.x;
+      const bool act = j < a.n && (!a.active || a.active[j]);
+      int total;
+      const int pos = tile_slot(act, total);
+      if (act)
+        term[(at + pos) % MT] = mma_term(mma_coef(a.x[j], a.low[j], a.upp[j], a.scale0 * a.df0[j], a.df1[j],
+                                                  a.xmin, a.xmax, a.move, a.r), lam);
+      __syncthreads();
+      if ((int)(threadIdx.x + MT - at) % MT < total) acc += term[threadIdx.x];
+      at = (at + total) % MT;
+    }
   }
   mma_finish(acc, a.f1, partial, s);
 }

@@ -81,3 +81,35 @@ def test_constraint_sum_beyond_the_range(nc):
     """Finite terms whose sum with f1 overflows: violated for every multiplier."""
     lam, chg, X = update(nc, np.full(4, 0.5), np.full(4, 1.0), 1.2e308, np.full(4, -1e308))
     assert lam == 2.0 ** 200 and np.abs(X - 0.3).max() <= 1e-15
+
+
+@pytest.mark.parametrize("n", [257, 70001, 608 * 256 * 2 + 77])
+@pytest.mark.parametrize("share", [1.0, 0.4, 0.003])
+def test_same_bits_without_the_workspace(nc, n, share):
+    """The update does not depend on how much device memory is free: without the workspace it
+    sums the same terms in the same order."""
+    rng = np.random.default_rng(n)
+    x = rng.uniform(0.1, 0.9, n)
+    xo1 = np.clip(x + 0.05 * rng.standard_normal(n), 0, 1)
+    xo2 = np.clip(xo1 + 0.05 * rng.standard_normal(n), 0, 1)
+    df0, df1 = rng.uniform(0.5, 1.5, n) / n, -rng.uniform(0.5, 1.5, n) / (share * n)
+    act = rng.uniform(size=n) < share
+    act[n // 3] = True
+    dev = lambda t: torch.tensor(t, dtype=torch.float64, device="cuda")  # noqa: E731
+    mask = torch.tensor(act.astype(np.uint8), device="cuda")
+
+    def run():
+        gp = nc.Problem(nc.make_params(2, 2, 2, 0.5, 1e3, 0.71), nc.cavity_bcs())
+        s = [dev(t) for t in (x, xo1, xo2, xo1 - 0.3, xo1 + 0.3)]
+        lam, chg = gp.mma_update(4, *s, dev(df0), 0.02, dev(df1), active=mask)
+        return [lam, chg] + [t.cpu() for t in s]
+
+    with_ws = run()
+    torch.cuda.empty_cache()
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - (6 << 30), dtype=torch.uint8, device="cuda")
+    try:
+        without = run()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert with_ws[:2] == without[:2] and all(torch.equal(a, b) for a, b in zip(with_ws[2:], without[2:]))
