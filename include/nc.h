@@ -176,11 +176,14 @@ nc_status nc_diag(nc_ctx* ctx, const void* x, const void* gamma, void* d, int pr
  * with entries reaching outside the grid 0, Dirichlet rows identity and
  * Dirichlet columns 0 (the same blockdiag(J_II, I) as nc_jvp).  S: DEVICE,
  * 675 Nn values of the precision prec, owned by the caller (5.4 KB per node in
- * FP64).  Built from the element Jacobians: 40 element products with unit
- * directions, each summed into S per node in a fixed order (deterministic); FP64
- * first stores the linearisation (as nc_linearize, in a context-owned store
- * allocated at the first call) and forms the columns from it with the unit
- * direction written out.  x and gamma as for nc_jvp. */
+ * FP64).  Built from the element Jacobians, a row per element, test node and field
+ * at a time, from a linearisation store (as nc_linearize's; 1,248 B per element in FP64,
+ * 624 in FP32) that the context allocates at the first call and keeps; deterministic.
+ * In FP32 the store is not allocated where the device would keep less than 8 GB free;
+ * the context's FP32 assemblies (also those of solves with mixed and assembled) are
+ * then built from 40 element products with unit directions, slower and rounded
+ * differently.  A context decides this once, at its first FP32 assembly.
+ * x and gamma as for nc_jvp. */
 nc_status nc_assemble(nc_ctx* ctx, const void* x, const void* gamma, void* S, int prec,
                       void* stream);
 

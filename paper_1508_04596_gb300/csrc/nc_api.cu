@@ -61,16 +61,18 @@ bool valid_bcs(const nc_params& p, const nc_bcs* b, std::string& why) {
 
 // Allocated once, for the finest level, so that a captured nc_assemble stays valid; the
 // allocation itself may fall into a capture.  FP32 can do without (op_assemble), and does
-// so rather than leave less than 8 GB free.
+// so rather than leave less than 8 GB free.  That rounds differently, so what the first
+// call finds holds for the context: its results do not change with the memory free later.
 template <typename R>
 R* assembly_store(nc_ctx* ctx) {
   constexpr bool fp32 = sizeof(R) == 4;
   void*& store = fp32 ? ctx->asm_lin32 : ctx->asm_lin;
-  if (!store) {
+  if (!store && !(fp32 && ctx->asm_none32)) {
     const size_t need = sizeof(R) * (size_t)LIN_SLOTS * (size_t)ctx->lv[0].d.E;
     size_t fr = 0, tot = 0;
     if (fp32 && (cudaMemGetInfo(&fr, &tot) != cudaSuccess || fr < need + ((size_t)8 << 30))) {
       cudaGetLastError();
+      ctx->asm_none32 = true;
       return nullptr;
     }
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -78,6 +80,7 @@ R* assembly_store(nc_ctx* ctx) {
     if (cudaMalloc(&store, need) != cudaSuccess) {
       cudaGetLastError();
       store = nullptr;
+      ctx->asm_none32 |= fp32;
     }
     cudaThreadExchangeStreamCaptureMode(&mode);
   }

@@ -171,6 +171,7 @@ struct nc_ctx {
   double* pub_lin = nullptr;  // linearisation of nc_linearize (level 0, FP64)
   void* asm_lin = nullptr;    // linearisation store of nc_assemble in FP64
   void* asm_lin32 = nullptr;  // of the FP32 assemblies, all levels in turn
+  bool asm_none32 = false;    // the first FP32 assembly found no room for it
   double* ref_lin = nullptr;  // linearisation of the mixed adjoint's FP64 refinement (level 0)
   void* mma_ws = nullptr;     // coefficient workspace of nc_mma_update
   size_t mma_ws_bytes = 0;
