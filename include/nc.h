@@ -19,6 +19,9 @@
  *    in _host.  Element type: double for NC_FP64, float for NC_FP32.
  *  - Calls enqueue work on `stream` (a cudaStream_t; NULL = legacy default stream)
  *    and return without synchronising, except where a call documents a host result.
+ *  - A context has one set of scratch arrays: the caller orders the calls on it (one
+ *    stream, or streams that wait for each other).  Calls on different contexts need no
+ *    order.
  *  - Inputs are never modified, except arguments named *_inout.
  *  - Errors: every call returns an nc_status; nc_last_error(ctx) gives a message.
  *    The library never aborts and never prints.

@@ -503,6 +503,7 @@ nc_status nc_objective(nc_ctx* ctx, const double* x, double* phi_host, double* d
   else
     op_objective_grad(L.d, g, s);  // mean patch temperature
   // Phi = <dPhi/dx, x> (both objectives are linear in T)
+  red_start(ctx, s);
   vmdot(5 * L.d.Nn, 1, g, 0, x, ctx->dscal, ctx->partial, s);
   if ((st = cuda_check(ctx, cudaMemcpyAsync(phi_host, ctx->dscal, sizeof(double),
                                             cudaMemcpyDeviceToHost, s), "nc_objective")) != NC_OK)

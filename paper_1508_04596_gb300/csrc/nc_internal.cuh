@@ -269,6 +269,11 @@ void op_coarsen_elem(const LevelDev& fine, const R* gf, const LevelDev& coarse, 
 // that finishes last (0 between reductions).
 constexpr long long RED_PARTIALS = (long long)(MAX_RESTART + 2) * RED_BLOCKS_MAX;
 inline unsigned* red_ticket(double* partial) { return (unsigned*)(partial + RED_PARTIALS); }
+// Every public call that reduces starts with this: reductions of two calls that overlapped
+// on one context (the caller's error) may have left a count behind.
+inline void red_start(nc_ctx* ctx, cudaStream_t s) {
+  cudaMemsetAsync(red_ticket(ctx->partial), 0, sizeof(unsigned), s);
+}
 template <typename Rd, typename Rs>
 void vcast(long long n, const Rs* x, Rd* y, cudaStream_t s);
 template <typename R>

@@ -675,6 +675,7 @@ nc_status nc_newton_solve(nc_ctx* ctx, const double* gam, double* x, const nc_so
   nc_default_opts(&o);
   if (opts) o = *opts;
   cudaStream_t s = (cudaStream_t)stream;
+  red_start(ctx, s);
   nc_solve_info info;
   std::memset(&info, 0, sizeof(info));
   const auto t0 = std::chrono::steady_clock::now();
@@ -751,6 +752,7 @@ nc_status nc_arnoldi_orth(nc_ctx* ctx, long long n, int k, const void* V, long l
       (prec != NC_FP64 && prec != NC_FP32))
     return set_err(ctx, NC_ERR_ARG, "nc_arnoldi_orth: invalid argument");
   cudaStream_t s = (cudaStream_t)stream;
+  red_start(ctx, s);
   const int off = MAX_RESTART + 2;
   double* hc = ctx->dscal;  // 2 * off + 1 slots
   if (prec == NC_FP64)
@@ -840,6 +842,7 @@ nc_status nc_adjoint_solve(nc_ctx* ctx, const double* x, const double* gam, cons
   nc_default_opts(&o);
   if (opts) o = *opts;
   cudaStream_t s = (cudaStream_t)stream;
+  red_start(ctx, s);
   nc_solve_info info;
   std::memset(&info, 0, sizeof(info));
   const auto t0 = std::chrono::steady_clock::now();

@@ -72,10 +72,33 @@ static int device_loops() {
   return bad;
 }
 
+// A count that overlapping reductions left in a context's ticket is gone with the next call.
+static int tickets() {
+  int bad = 0;
+  nc_ctx* ctx = context(4);
+  unsigned* const ticket = nc::red_ticket(ctx->partial);
+  const long long n = 5LL * 125, E = 64;
+  std::vector<double> x(n, 0.0), g(E, 0.5), r(n, 0.0), l(n, 0.0);
+  double h[3];
+  nc_solve_info info;
+  auto call = [&](const char* what, auto f) {
+    *ticket = 7;
+    f();
+    bad += report(what, *ticket == 0);
+  };
+  call("nc_arnoldi_orth", [&] { nc_arnoldi_orth(ctx, n, 1, r.data(), n, l.data(), h, NC_FP64, nullptr); });
+  call("nc_objective", [&] { nc_objective(ctx, x.data(), h, r.data(), nullptr); });
+  call("nc_newton_solve", [&] { nc_newton_solve(ctx, g.data(), x.data(), nullptr, &info, nullptr); });
+  call("nc_adjoint_solve", [&] { nc_adjoint_solve(ctx, x.data(), g.data(), r.data(), l.data(), nullptr, &info, nullptr); });
+  nc_destroy(ctx);
+  return bad;
+}
+
 int main(int argc, char** argv) {
   const std::string check = argc > 1 ? argv[1] : "";
   if (check == "smoother_levels") return smoother_levels();
   if (check == "device_loops") return device_loops();
+  if (check == "tickets") return tickets();
   std::printf("unknown check\n");
   return 2;
 }
