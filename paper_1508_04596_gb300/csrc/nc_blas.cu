@@ -168,10 +168,16 @@ __device__ __forceinline__ void sub_cols(const R* __restrict__ X, long long ld, 
   }
 }
 
-// Block-level sum of one value per thread, result valid in thread 0.
+// Block sum of one value per thread -> partial[blockIdx.x].
 template <typename T>
-__device__ __forceinline__ T block_sum(T v) {
-  return block_fold<false, RED_THREADS>(v);
+__device__ __forceinline__ void block_partial(T v, double* partial) {
+  if constexpr (sizeof(T) == 8) {
+    v = block_fold<false, RED_THREADS>(v);
+    if (threadIdx.x == 0) partial[blockIdx.x] = v;
+  } else {
+    const T w[1] = {v};
+    block_values<RED_THREADS>(w, 1, partial);
+  }
 }
 
 // The last block's end of a reduction of cnt values (nc_reduce.cuh).
@@ -342,8 +348,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_arnoldi_update(long long n, int
     w[i] = a;
     if (t) t[i] = a / D[i];
   });
-  const R s = block_sum(acc2);
-  if (threadIdx.x == 0) partial[blockIdx.x] = double(s);
+  block_partial(acc2, partial);
   if (!last_block(ticket)) return;
   fold_values(1, gridDim.x, partial, [&](int, double v) { put_norm(Hd + HD_SIG2 + k, Hd + HD_ISIG + k, v); });
   if (ls) {
@@ -386,8 +391,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_init_basis(long long n, const R
     if (copy) v0[i] = a;
     t[i] = a / D[i];
   });
-  const R s = block_sum(acc2);
-  if (threadIdx.x == 0) partial[blockIdx.x] = double(s);
+  block_partial(acc2, partial);
   finish(1, partial, ticket, [&](int, double v) { put_norm(Hd + HD_SIG2, Hd + HD_ISIG, v); });
 }
 

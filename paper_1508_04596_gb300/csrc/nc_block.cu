@@ -12,7 +12,8 @@
 // at six steps.
 //
 // The arithmetic is that of smooth() in nc_solver.cu: the basis is unnormalised, dots
-// and norms are summed in FP32 in a fixed order and their quotients formed in FP64.
+// and norms are summed in FP32 within a warp, in FP64 over the warps, in a fixed order, and
+// their quotients are formed in FP64.
 #include "nc_element_f2.cuh"
 #include "nc_internal.cuh"
 #include "nc_reduce.cuh"
@@ -24,6 +25,7 @@ namespace {
 
 constexpr int BT = 256, BW = BT / 32;  // one element per thread and pass at 255 registers
 constexpr int BK = 8;                  // largest number of smoothing steps
+static_assert(BW == 8 && BK == 8, "k_smooth_block folds eight values of eight warps, eight lanes each");
 
 struct BlockSmooth {
   LevelDev d;
@@ -109,18 +111,21 @@ __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ 
     for (int f = 0; f < 5; ++f)
       if ((fl >> f) & 1) w[f] = t[f * Nn + n];
   };
+  // The sum over the eight lanes from lane 8 g on, in all of them: the warps' parts of a value.
+  auto fold8 = [&](double v) {
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
   // The squared norm of v_j from its per-thread parts, and its reciprocal root, which the
-  // last thread forms while the others begin the next product.
+  // last warp forms while the others begin the next product.
   auto norm = [&](int j, float s) {
     s = warp_fold<false>(s);
     if (lane == 0) warp[wid][0] = s;
     __syncthreads();
-    if (tid == BT - 1) {
-      float v = 0.0f;
-      for (int w = 0; w < BW; ++w) v += warp[w][0];
-      const double v2 = v;
-      sig2[j] = v2;
-      isig[j] = v2 > 0.0 && v2 < 1e300 ? rsqrt(v2) : 0.0;
+    if (wid == BW - 1) {
+      const double v2 = fold8(warp[lane & 7][0]);
+      if (lane == 0) put_norm(sig2 + j, isig + j, v2);
     }
   };
 
@@ -175,12 +180,14 @@ __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ 
         if (lane == 0) warp[wid][q] = v;
       }
     __syncthreads();
-    if (tid <= j) {
-      float v = 0.0f;
-      for (int m = 0; m < BW; ++m) v += warp[m][tid];
-      H[j * (k + 1) + tid] = v;
-      cf[tid] = (float)(v * isig[tid] * isig[tid]);
-    } else if (tid == 32) {
+    if (tid < 8 * BW) {  // eight lanes a dot
+      const int q = tid >> 3;
+      const double v = fold8(q <= j ? (double)warp[tid & 7][q] : 0.0);
+      if ((tid & 7) == 0 && q <= j) {
+        H[j * (k + 1) + q] = v;
+        cf[q] = (float)(v * isig[q] * isig[q]);
+      }
+    } else if (tid == 8 * BW) {
       sc = (float)isig[j];
     }
     __syncthreads();

@@ -34,7 +34,9 @@ __device__ __forceinline__ T block_fold(T v) {
 }
 
 // Block sums of N values per thread (the first cnt of them) to partial[q * gridDim.x +
-// blockIdx.x].  FP32 folds by shuffles.  An FP64 addition holds a scheduler's unit for
+// blockIdx.x].  FP32 folds by shuffles within a warp and the warps' sums in FP64: a block may
+// hold a whole vector (4,096 elements), whose sum stays in as many bits as that of two
+// blocks.  An FP64 addition holds a scheduler's unit for
 // 64 cycles whatever the number of active lanes, so FP64 values go through shared
 // memory and one warp adds a value's eight warps before its five shuffle steps: 12
 // additions per value and block instead of 45.
@@ -72,11 +74,12 @@ __device__ __forceinline__ void block_values(const T (&v)[N], int cnt, double* p
         if (lane == 0) sh[wid * 8 + q] = t;
       }
     __syncthreads();
-    if ((int)threadIdx.x < cnt) {
-      T t = sh[threadIdx.x];
+    if ((int)(threadIdx.x & ~31u) < cnt * W) {  // W lanes a value
+      const int q = threadIdx.x / W, w = threadIdx.x % W;
+      double t = q < cnt ? double(sh[w * 8 + q]) : 0.0;
 #pragma unroll
-      for (int w = 1; w < W; ++w) t += sh[w * 8 + threadIdx.x];
-      partial[(long long)threadIdx.x * gridDim.x + blockIdx.x] = double(t);
+      for (int o = W / 2; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o, W);
+      if (w == 0 && q < cnt) partial[(long long)q * gridDim.x + blockIdx.x] = t;
     }
   }
 }
