@@ -355,7 +355,7 @@ void vcombine(long long n, int k, const R* X, long long ld, const double* coef, 
 // (n, f) to (n + offset o, g), o = (dx+1) + 3 (dy+1) + 9 (dz+1)
 constexpr int STENCIL_VALUES = 675;
 // S = J(x, gamma) of one level, from its element Jacobians: from the linearisation
-// store `cache` (nc_assemble.cuh), or without one by 40 element products with unit
+// store `cache` (nc_assemble.cuh), or in FP32 without one by 40 element products with unit
 // directions, each summed into S per node; Dirichlet rows identity, Dirichlet columns
 // zero.
 template <typename R>

@@ -75,30 +75,29 @@ __device__ __forceinline__ void store_elem(long long E, long long e, const R out
 // Column col = 5 b + g of every element Jacobian: the element product with the
 // unit direction on unknown g of local node b, or zero where that unknown is
 // Dirichlet (Dirichlet columns are removed).  Re-interpolates the state: the way
-// to assemble where there is no memory for a linearisation store.
-template <typename R>
+// to assemble in FP32 where there is no memory for a linearisation store.
 __global__ void __launch_bounds__(ELEM_THREADS) k_elem_column(
-    LevelDev d, ElemConst<R> c, const R* __restrict__ x, const R* __restrict__ gam,
-    const R* __restrict__ src, int col, R* Y) {
+    LevelDev d, ElemConst<float> c, const float* __restrict__ x, const float* __restrict__ gam,
+    const float* __restrict__ src, int col, float* Y) {
   const long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (e >= d.E) return;
   const int b = col / 5, g = col % 5;
-  R out[5][8];
+  float out[5][8];
   if ((d.flag[elem_node(d, e, b)] >> g) & 1) {
 #pragma unroll
     for (int f = 0; f < 5; ++f)
 #pragma unroll
-      for (int a = 0; a < 8; ++a) out[f][a] = R(0);
+      for (int a = 0; a < 8; ++a) out[f][a] = 0.0f;
     store_elem(d.E, e, out, Y);
     return;
   }
-  R ve[5][8], xe[5][8];
+  float ve[5][8], xe[5][8];
 #pragma unroll
   for (int f = 0; f < 5; ++f)
 #pragma unroll
-    for (int a = 0; a < 8; ++a) ve[f][a] = (f == g && a == b) ? R(1) : R(0);
+    for (int a = 0; a < 8; ++a) ve[f][a] = (f == g && a == b) ? 1.0f : 0.0f;
   load_elem(d, x, e, xe, false);
-  elem_jvp<R>(xe, ve, gam[e], src ? src[e] : R(0), c, out);
+  elem_jvp<float>(xe, ve, gam[e], src ? src[e] : 0.0f, c, out);
   store_elem(d.E, e, out, Y);
 }
 
@@ -108,10 +107,9 @@ __global__ void __launch_bounds__(ELEM_THREADS) k_elem_column(
 // eight distinct offsets, so one launch writes no entry twice; the launches run
 // in column order, so the sums are deterministic.  Dirichlet rows are skipped
 // (they become identity rows afterwards).
-template <typename R>
 __global__ void __launch_bounds__(NODE_THREADS) k_assemble_column(LevelDev d, int col,
-                                                                  const R* __restrict__ Y,
-                                                                  R* __restrict__ S) {
+                                                                  const float* __restrict__ Y,
+                                                                  float* __restrict__ S) {
   const long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (n >= d.Nn) return;
   int i, j, k;
@@ -532,14 +530,18 @@ template <typename R>
 void op_assemble(const LevelDev& d, const ElemConst<R>& c, const R* x, const R* gam, const R* src,
                  const R* cache, R* S, R* Y, cudaStream_t s) {
   cudaMemsetAsync(S, 0, sizeof(R) * (size_t)STENCIL_VALUES * (size_t)d.Nn, s);
-  if (cache) {
-    for (int a = 0; a < 8; ++a) rows::k_assemble_rows<R><<<nblocks(d.E, 128), 128, 0, s>>>(d, c, rows::row_const(c, a), x, cache, a, S);
-  } else {
-    for (int col = 0; col < 40; ++col) {
-      k_elem_column<R><<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src, col, Y);
-      k_assemble_column<R><<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, col, Y, S);
+  if constexpr (sizeof(R) == 4) {
+    if (!cache) {
+      for (int col = 0; col < 40; ++col) {
+        k_elem_column<<<nblocks(d.E, ELEM_THREADS), ELEM_THREADS, 0, s>>>(d, c, x, gam, src, col, Y);
+        k_assemble_column<<<nblocks(d.Nn, NODE_THREADS), NODE_THREADS, 0, s>>>(d, col, Y, S);
+      }
+      stencil_dirichlet<R>(d, S, s);
+      return;
     }
   }
+  for (int a = 0; a < 8; ++a)
+    rows::k_assemble_rows<R><<<nblocks(d.E, 128), 128, 0, s>>>(d, c, rows::row_const(c, a), x, cache, a, S);
   stencil_dirichlet<R>(d, S, s);
 }
 

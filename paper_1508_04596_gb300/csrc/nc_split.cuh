@@ -20,14 +20,18 @@ template <typename R> struct QuadSums {
   R o[4][20][32];
 };
 
-// Warp q of a quad, chunk `w`.  sync() is a barrier of the quad's 128 threads.  FRESH:
-// v was written by other blocks of this kernel (read past L1).
-template <typename R, int K, bool FRESH, typename Sync>
-__device__ __forceinline__ void split_chunk(const LevelDev& d, const ElemConst<R>& c, const MarchPlan& mp,
-                                            long long w, int q, const R* __restrict__ x,
-                                            const R* __restrict__ gam, const R* __restrict__ srcs,
-                                            const R* __restrict__ cache, const R* v, R* Y,
-                                            QuadSums<R>& sums, Sync&& sync) {
+template <typename R, int K>
+__global__ void __launch_bounds__(128) k_split(LevelDev d, ElemConst<R> c, MarchPlan mp,
+                                               const R* __restrict__ x_, const R* __restrict__ gam,
+                                               const R* __restrict__ srcs, const R* __restrict__ cache_,
+                                               const R* __restrict__ v_, R* Y) {
+  chained();
+  const R* const x = fresh(x_);
+  const R* const cache = fresh(cache_);
+  const R* const v = fresh(v_);
+  __shared__ QuadSums<R> sums;
+  const long long w = blockIdx.x;  // the chunk
+  const int q = threadIdx.x >> 5;  // the warp of the quad
   typedef Traits<K> TR;
   typedef typename Stage<R, K>::T T;
   typedef PR<R> P;
@@ -45,10 +49,6 @@ __device__ __forceinline__ void split_chunk(const LevelDev& d, const ElemConst<R
   const long long n = i + sx * (j + (long long)(d.ny + 1) * k);
   const long long e = min(i, d.nx - 1) + (long long)d.nx * (j + (long long)d.ny * k);
   const R c0 = R(GW0), c1 = R(GW1), cy = qy ? c1 : c0, cz = qz ? c1 : c0;
-  auto vec = [&](long long at) -> R {
-    if constexpr (FRESH) return __ldcg(v + at);
-    else return v[at];
-  };
 
   // ---- nodal values, z stage (this warp's plane), row sums of u.u and u.v
   T dzr[5][2], vr[5][2];  // [field][row]
@@ -72,7 +72,7 @@ __device__ __forceinline__ void split_chunk(const LevelDev& d, const ElemConst<R
         R u = R(0), t = R(0);
         if (!TR::DIR || f < 3) u = x[at];
         if (TR::TWO || TR::DIR) {
-          t = vec(at);
+          t = v[at];
           t = masked ? R(0) : t;
         }
         if constexpr (TR::TWO) nod[z] = mk(u, t);
@@ -249,27 +249,13 @@ __device__ __forceinline__ void split_chunk(const LevelDev& d, const ElemConst<R
         sums.o[q][(r * 2 + z) * 5 + f][lane] = o[r][z];
       }
   }
-  sync();
+  __syncthreads();
   // warp q adds the five sums of node row q / 2, corner q % 2
   R* y = Y + w * 2 * (long long)ROW_LEN + (q >> 1) * ROW_LEN + (q & 1) * 160 + lane;
 #pragma unroll
   for (int f = 0; f < 5; ++f)
     y[f * 32] = (sums.o[0][q * 5 + f][lane] + sums.o[1][q * 5 + f][lane]) +
                 (sums.o[2][q * 5 + f][lane] + sums.o[3][q * 5 + f][lane]);
-}
-
-template <typename R, int K>
-__global__ void __launch_bounds__(128) k_split(LevelDev d, ElemConst<R> c, MarchPlan mp,
-                                               const R* __restrict__ x_, const R* __restrict__ gam,
-                                               const R* __restrict__ srcs, const R* __restrict__ cache_,
-                                               const R* __restrict__ v_, R* Y) {
-  chained();
-  const R* const x = fresh(x_);
-  const R* const cache = fresh(cache_);
-  const R* const v = fresh(v_);
-  __shared__ QuadSums<R> sums;
-  split_chunk<R, K, false>(d, c, mp, blockIdx.x, threadIdx.x >> 5, x, gam, srcs, cache, v, Y, sums,
-                           [] { __syncthreads(); });
 }
 
 }  // namespace march
