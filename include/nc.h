@@ -253,7 +253,7 @@ nc_status nc_fma_probe(int prec, int blocks, long long iters, void* out, void* s
  * gamma_f[e] of rho~ (element arrays [E], FP64, device).  The map rho -> gamma_f
  * is symmetric, so the same call applied to dPhi/dgamma_f gives dPhi/drho (the
  * chain rule of the filtered design).  Conjugate gradients with Jacobi
- * preconditioning to a relative residual of 1e-13; workspace (6 node vectors)
+ * preconditioning to a relative residual of 1e-13; workspace (5 node vectors)
  * is allocated at the first call.  Synchronous.  NC_ERR_NAN for a non-finite
  * design, NC_ERR_MAXIT if CG does not converge in 1000 iterations. */
 nc_status nc_filter(nc_ctx* ctx, const double* rho, double* gamma_f, double radius, void* stream);

@@ -8,7 +8,7 @@
 // elem_jtvp_f2) and then nodes.  One SM works on it, so it pays while the product takes
 // less than the launches saved.  An FGMRES iteration of a mixed solve without / with it:
 // 16^3 (levels 8^3 and 4^3 here) 790 / 657 us, 64^3 1998 / 1890; with 4^3 alone 700 and
-// 1927.  6^3 (96^3): 3650 / 3588.  512 elements are what the shared memory holds: 228 KB
+// 1927.  6^3 (96^3): 3650 / 3588.  512 elements are what the shared memory holds: 222 KB
 // at six steps.
 //
 // The arithmetic is that of smooth() in nc_solver.cu: the basis is unnormalised, dots

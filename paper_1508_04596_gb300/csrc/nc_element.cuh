@@ -24,8 +24,8 @@
 // plain arithmetic on register arrays, usable from host and device code.  The device
 // operators work on faces of elements that share their stages with the neighbours
 // (nc_march.cuh), on the coefficients and point fluxes below; the whole-element forms
-// (elem_jvp, elem_diag in the dense coarse matrix, the FP32 assembly and the diagonal; the
-// others on the host only) state what these must equal.
+// (elem_jvp in the dense coarse matrix and in the FP32 assembly without a store, elem_diag
+// in the diagonal; the others on the host only) state what these must equal.
 //
 // Scaling.  Point gradients are kept in reference units, h grad (the nodal
 // differences of the tensor-product stages, with no division by h), and so are

@@ -16,7 +16,8 @@
 //  * the test side (test8) mirrors the interpolation: a scalar x stage from
 //    point pairs to node pairs, then packed y and z stages.
 // The marching kernels (nc_march.cuh) take the pair arithmetic and the point fluxes from
-// here; the whole-element products below are the form that the host check compares.
+// here; the whole-element products below are what the one-block smoother of small levels
+// runs (nc_block.cu) and what the host check compares.
 // The result equals elem_jvp<float> / elem_jtvp<float> up to FP32 rounding
 // (different order of some sums); the host check compares them.
 //

@@ -329,6 +329,9 @@ template <typename R>
 void varnoldi_update(long long n, int k, const R* X, long long ld, const R* D, R* w, R* t, double* Hd,
                      bool ls, double* partial, cudaStream_t s);
 // z = (sum_i coef[i] X_i) / D (D may be null: no division), or z += ... with accumulate
+template <typename R>
+void vcombine(long long n, int k, const R* X, long long ld, const double* coef, const R* D, R* z,
+              bool accumulate, cudaStream_t s);
 // Device scalars of a smoother: the Hessenberg columns of raw dots (leading dimension
 // LDH), the coefficients of the correction, the squared norms of the basis and their
 // reciprocal roots (0 for a vanishing or non-finite norm), and the coefficients
@@ -346,9 +349,6 @@ bool smooth_block(const LevelDev& d, const ElemConst<float>& c, const LevelBuf<f
                   float* r, cudaStream_t s);
 // The smoother's small least-squares problem (nc_smooth.cu): Hd[HD_Y..] from the rest.
 void small_ls(double* Hd, int k, cudaStream_t s);
-template <typename R>
-void vcombine(long long n, int k, const R* X, long long ld, const double* coef, const R* D, R* z,
-              bool accumulate, cudaStream_t s);
 
 // ---- stencil operators (nc_galerkin.cu): assembled level operators and Galerkin
 // coarse operators.  S holds 675 * Nn entries, S[((o*5 + f)*5 + g)*Nn + n] couples

@@ -9,9 +9,10 @@
 // in FP32; with mixed = 0 everything is FP64.
 //
 // The V-cycle and smoother run entirely on the device: their Hessenberg
-// scalars stay in device memory and a one-thread kernel solves the small
-// least-squares problem, so a preconditioner application never waits on the
-// host.
+// scalars stay in device memory and one warp solves the small least-squares
+// problem (at the end of the last update, of the one-block smoother, or beyond
+// eight steps in a kernel of its own), so a preconditioner application never
+// waits on the host.
 #include <chrono>
 #include <cmath>
 #include <cstring>
