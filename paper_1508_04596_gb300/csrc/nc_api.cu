@@ -498,15 +498,16 @@ nc_status nc_objective(nc_ctx* ctx, const double* x, double* phi_host, double* d
     if (!ctx->tmp64[3] && (st = dev_alloc(ctx, &ctx->tmp64[3], 5 * L.d.Nn)) != NC_OK) return st;
     g = ctx->tmp64[3];
   }
+  red_start(ctx, s);
   if (L.d.patch_mode == NC_PATCH_NONE && ctx->src64)
     op_source_grad(L.d, ctx->src64, g, s);  // thermal compliance (Sec. 3.2)
   else
     op_objective_grad(L.d, g, s);  // mean patch temperature
   // Phi = <dPhi/dx, x> (both objectives are linear in T)
-  red_start(ctx, s);
   vmdot(5 * L.d.Nn, 1, g, 0, x, ctx->dscal, ctx->partial, s);
-  if ((st = cuda_check(ctx, cudaMemcpyAsync(phi_host, ctx->dscal, sizeof(double),
-                                            cudaMemcpyDeviceToHost, s), "nc_objective")) != NC_OK)
+  if ((st = cuda_check(ctx, cudaGetLastError(), "nc_objective")) != NC_OK ||
+      (st = cuda_check(ctx, cudaMemcpyAsync(phi_host, ctx->dscal, sizeof(double), cudaMemcpyDeviceToHost, s),
+                       "nc_objective")) != NC_OK)
     return st;
   return cuda_check(ctx, cudaStreamSynchronize(s), "nc_objective");
 }

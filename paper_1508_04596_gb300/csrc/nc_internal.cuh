@@ -270,8 +270,10 @@ void op_coarsen_elem(const LevelDev& fine, const R* gf, const LevelDev& coarse, 
 constexpr long long RED_PARTIALS = (long long)(MAX_RESTART + 2) * RED_BLOCKS_MAX;
 inline unsigned* red_ticket(double* partial) { return (unsigned*)(partial + RED_PARTIALS); }
 // Every public call that reduces starts with this: reductions of two calls that overlapped
-// on one context (the caller's error) may have left a count behind.
+// on one context (the caller's error) may have left a count behind.  Errors of earlier calls
+// are dropped: what cudaGetLastError says at the call's next read is its own launches'.
 inline void red_start(nc_ctx* ctx, cudaStream_t s) {
+  cudaGetLastError();
   cudaMemsetAsync(red_ticket(ctx->partial), 0, sizeof(unsigned), s);
 }
 template <typename Rd, typename Rs>

@@ -351,8 +351,9 @@ void apply_A(nc_ctx* ctx, const LinSolve& ls, const double* v, double* out, cuda
 }
 
 nc_status read_scalar(nc_ctx* ctx, const double* d, double* h, int k, cudaStream_t s) {
-  nc_status st = cuda_check(ctx, cudaMemcpyAsync(h, d, sizeof(double) * k, cudaMemcpyDeviceToHost, s),
-                            "read scalar");
+  nc_status st = cuda_check(ctx, cudaGetLastError(), "launch");
+  if (st != NC_OK) return st;
+  st = cuda_check(ctx, cudaMemcpyAsync(h, d, sizeof(double) * k, cudaMemcpyDeviceToHost, s), "read scalar");
   if (st != NC_OK) return st;
   return cuda_check(ctx, cudaStreamSynchronize(s), "stream sync");
 }

@@ -94,11 +94,34 @@ static int tickets() {
   return bad;
 }
 
+// Calls that read a sum from the device: with every launch refused they end with an error, and
+// not with what the memory happened to hold.
+static int refused_sums() {
+  int bad = 0;
+  nc_ctx* ctx = context(4);
+  const long long n = 5LL * 125, E = 64;
+  std::vector<double> x(n, 0.0), g(E, 0.5), r(n, 0.0), l(n, 0.0);
+  double h[3];
+  nc_solve_info info;
+  fake::refuse = true;
+  bad += report("nc_arnoldi_orth", nc_arnoldi_orth(ctx, n, 1, r.data(), n, l.data(), h, NC_FP64, nullptr) == NC_ERR_CUDA);
+  bad += report("nc_objective", nc_objective(ctx, x.data(), h, r.data(), nullptr) == NC_ERR_CUDA);
+  bad += report("nc_newton_solve",
+                nc_newton_solve(ctx, g.data(), x.data(), nullptr, &info, nullptr) == NC_ERR_CUDA &&
+                    info.status == NC_ERR_CUDA);
+  bad += report("nc_adjoint_solve",
+                nc_adjoint_solve(ctx, x.data(), g.data(), r.data(), l.data(), nullptr, &info, nullptr) == NC_ERR_CUDA);
+  fake::refuse = false;
+  nc_destroy(ctx);
+  return bad;
+}
+
 int main(int argc, char** argv) {
   const std::string check = argc > 1 ? argv[1] : "";
   if (check == "smoother_levels") return smoother_levels();
   if (check == "device_loops") return device_loops();
   if (check == "tickets") return tickets();
+  if (check == "refused_sums") return refused_sums();
   std::printf("unknown check\n");
   return 2;
 }
