@@ -237,6 +237,8 @@ void nc_destroy(nc_ctx* ctx) {
   cudaFree(ctx->asm_lin32);
   cudaFree(ctx->mma_ws);
   if (ctx->cap) cudaStreamDestroy(ctx->cap);
+  cudaFreeHost(ctx->pin);
+  if (ctx->ev) cudaEventDestroy(ctx->ev);
   delete ctx;
 }
 
@@ -293,7 +295,9 @@ nc_status nc_setup(const nc_params* prm, const nc_bcs* bcs, nc_ctx** out) {
   if ((st = dev_alloc(ctx, &ctx->Y, scratch_len(L0.d.E))) != NC_OK) { nc_destroy(ctx); return st; }
   if ((st = dev_alloc(ctx, &ctx->partial, RED_PARTIALS + 1)) != NC_OK ||
       (st = cuda_check(ctx, cudaMemset(red_ticket(ctx->partial), 0, sizeof(double)), "cudaMemset")) != NC_OK ||
-      (st = dev_alloc(ctx, &ctx->dscal, (long long)(MAX_RESTART + 2) * 4)) != NC_OK) {
+      (st = dev_alloc(ctx, &ctx->dscal, (long long)(MAX_RESTART + 2) * 4)) != NC_OK ||
+      (st = cuda_check(ctx, cudaMallocHost(&ctx->pin, PIN_BYTES), "cudaMallocHost")) != NC_OK ||
+      (st = cuda_check(ctx, cudaEventCreateWithFlags(&ctx->ev, cudaEventDisableTiming), "cudaEventCreate")) != NC_OK) {
     nc_destroy(ctx);
     return st;
   }

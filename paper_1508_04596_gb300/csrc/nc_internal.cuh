@@ -167,6 +167,8 @@ struct nc_ctx {
   void* gj = nullptr;         // the coarsest level's dense inversion on the device
   size_t gj_bytes = 0;
   cudaStream_t cap = nullptr; // stream used to capture the V-cycle graph
+  void* pin = nullptr;        // page-locked memory for scalars read while the stream goes on
+  cudaEvent_t ev = nullptr;   // marks that read
   double* filt[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // filter CG
   double* pub_lin = nullptr;  // linearisation of nc_linearize (level 0, FP64)
   void* asm_lin = nullptr;    // linearisation store of nc_assemble in FP64
@@ -268,6 +270,7 @@ void op_coarsen_elem(const LevelDev& fine, const R* gf, const LevelDev& coarse, 
 // Reduction scratch (nc_ctx::partial): the partials, then the ticket of the block
 // that finishes last (0 between reductions).
 constexpr long long RED_PARTIALS = (long long)(MAX_RESTART + 2) * RED_BLOCKS_MAX;
+constexpr size_t PIN_BYTES = 256;  // nc_ctx::pin
 inline unsigned* red_ticket(double* partial) { return (unsigned*)(partial + RED_PARTIALS); }
 // Every public call that reduces starts with this: reductions of two calls that overlapped
 // on one context (the caller's error) may have left a count behind.  Errors of earlier calls

@@ -453,12 +453,13 @@ __global__ void k_design_map(long long n, const double* in, const unsigned char*
 
 inline unsigned grid1(long long n) { return (unsigned)((n + MT - 1) / MT); }
 
-nc_status read_sync(nc_ctx* ctx, const double* d, double* h, int k, cudaStream_t s,
-                    const char* what) {
-  nc_status st = cuda_check(ctx, cudaMemcpyAsync(h, d, sizeof(double) * k, cudaMemcpyDeviceToHost, s), what);
-  if (st != NC_OK) return st;
-  return cuda_check(ctx, cudaStreamSynchronize(s), what);
+// A read of device memory to ctx->pin that does not hold up what is enqueued after it:
+// read_end waits for the copy, not for the stream.
+nc_status read_begin(nc_ctx* ctx, const void* d, size_t bytes, cudaStream_t s, const char* what) {
+  const nc_status st = cuda_check(ctx, cudaMemcpyAsync(ctx->pin, d, bytes, cudaMemcpyDeviceToHost, s), what);
+  return st != NC_OK ? st : cuda_check(ctx, cudaEventRecord(ctx->ev, s), what);
 }
+nc_status read_end(nc_ctx* ctx, const char* what) { return cuda_check(ctx, cudaEventSynchronize(ctx->ev), what); }
 
 // The coefficient workspace of nc_mma_update, kept by the context (grown when a
 // larger problem asks).  False if the device would keep less than 8 GB free: the
@@ -520,10 +521,12 @@ nc_status nc_volume(nc_ctx* ctx, long long n, const double* gamma, const unsigne
   unsigned* ticket = (unsigned*)(ctx->dscal + 2);
   cudaMemsetAsync(ticket, 0, sizeof(unsigned), s);
   k_volume<<<mma_blocks(n), MT, 0, s>>>(n, gamma, active, ctx->partial, ctx->dscal, ticket);
+  // the host waits for the sums alone; the gradient is left on the stream
+  nc_status st = read_begin(ctx, ctx->dscal, 2 * sizeof(double), s, "nc_volume");
   if (dgdgamma) k_volume_grad<<<grid1(n), MT, 0, s>>>(n, active, ctx->dscal, vf, dgdgamma);
-  double sc[2];
-  nc_status st = read_sync(ctx, ctx->dscal, sc, 2, s, "nc_volume");
+  if (st == NC_OK) st = read_end(ctx, "nc_volume");
   if (st != NC_OK) return st;
+  const double* const sc = (const double*)ctx->pin;
   if (!(sc[1] > 0.0)) return set_err(ctx, NC_ERR_ARG, "nc_volume: no active variable");
   *g_host = sc[0] * (1.0 / (vf * sc[1])) - 1.0;
   return cuda_check(ctx, cudaGetLastError(), "nc_volume");

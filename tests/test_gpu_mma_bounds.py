@@ -113,3 +113,24 @@ def test_same_bits_without_the_workspace(nc, n, share):
         del hold
         torch.cuda.empty_cache()
     assert with_ws[:2] == without[:2] and all(torch.equal(a, b) for a, b in zip(with_ws[2:], without[2:]))
+
+
+@pytest.mark.parametrize("n", [1, 300, 608 * 256 * 3 + 5])
+def test_volume_gradient_is_left_on_the_stream(nc, n):
+    """The value is there when the call returns, the gradient in stream order; calls one after
+    another on different designs do not disturb each other."""
+    from oracle import mma as M
+    rng = np.random.default_rng(n)
+    gp = nc.Problem(nc.make_params(2, 2, 2, 0.5, 1e3, 0.71), nc.cavity_bcs())
+    dev = lambda t: torch.tensor(t, dtype=torch.float64, device="cuda")  # noqa: E731
+    xs = [rng.uniform(0, 1, n) for _ in range(3)]
+    acts = [np.arange(n) % (k + 1) == 0 for k in range(3)]
+    masks = [torch.tensor(a.astype(np.uint8), device="cuda") for a in acts]
+    gam, grads = [dev(x) for x in xs], [torch.empty(n, dtype=torch.float64, device="cuda") for _ in xs]
+    got = [gp.volume(g, m, 0.3, grad=d) for g, m, d in zip(gam, masks, grads)]
+    for x, a, g, d in zip(xs, acts, got, grads):
+        ref, dref = M.volume_constraint(x, a, 0.3)
+        assert g == pytest.approx(ref, rel=1e-12, abs=1e-12)
+        assert np.allclose(d.cpu().numpy(), dref, rtol=1e-14, atol=0)
+    with pytest.raises(Exception):
+        gp.volume(gam[0], torch.zeros_like(masks[0]), 0.3, grad=grads[0])
