@@ -51,8 +51,10 @@ namespace {
 
 constexpr int MT = 256;
 // Passes enqueued between two reads of the search's state: the search takes 10-15
-// evaluations, and one that finds it ended costs about 2 us.
-constexpr int MMA_BATCH = 16;
+// evaluations, and one that finds it ended costs about 2 us.  Where the constraint holds
+// without a multiplier there is nothing to search for: the host reads what the first
+// evaluation found while MMA_FIRST passes keep the GPU busy, and only then enqueues the rest.
+constexpr int MMA_FIRST = 2, MMA_BATCH = 14;
 
 // Blocks of a reduction over n variables: four per SM at most (FP64 square roots and
 // divisions are long dependent chains), a partition that depends only on n.
@@ -558,20 +560,30 @@ nc_status nc_mma_update(nc_ctx* ctx, long long n, int iter, double* x, double* x
     k_mma_begin<true><<<nb, MT, 0, s>>>(a, iter, w, part, srch);
   else
     k_mma_begin<false><<<nb, MT, 0, s>>>(a, iter, w, part, srch);
-  MmaSearch h;
-  do {  // most searches end within the first batch; a pass after the end costs its launch
-    for (int i = 0; i < MMA_BATCH; ++i) {
+  static_assert(sizeof(MmaSearch) <= PIN_BYTES, "ctx->pin holds the search");
+  auto search = [&](int passes) {
+    for (int i = 0; i < passes; ++i) {
       if (store)
         k_mma_dual<true><<<nb, MT, 0, s>>>(a, w, part, srch);
       else
         k_mma_dual<false><<<nb, MT, 0, s>>>(a, w, part, srch);
     }
+  };
+  nc_status st = read_begin(ctx, srch, sizeof(MmaSearch), s, "nc_mma_update");
+  if (st != NC_OK) return st;
+  search(MMA_FIRST);
+  if ((st = read_end(ctx, "nc_mma_update")) != NC_OK) return st;
+  int passes = ((const MmaSearch*)ctx->pin)->done ? 0 : MMA_BATCH;
+  MmaSearch h;
+  do {  // most searches end within the first batch; a pass after the end costs its launch
+    search(passes);
+    passes = MMA_BATCH;
     if (store)
       k_mma_commit<true><<<nb, MT, 0, s>>>(a, w, x, xold1, xold2, part, srch);
     else
       k_mma_commit<false><<<nb, MT, 0, s>>>(a, w, x, xold1, xold2, part, srch);
     // a refused launch would leave the state, which ends the loop, as it is
-    nc_status st = cuda_check(ctx, cudaGetLastError(), "nc_mma_update");
+    st = cuda_check(ctx, cudaGetLastError(), "nc_mma_update");
     if (st == NC_OK)
       st = cuda_check(ctx, cudaMemcpyAsync(&h, srch, sizeof(h), cudaMemcpyDeviceToHost, s), "nc_mma_update");
     if (st == NC_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "nc_mma_update");

@@ -134,3 +134,22 @@ def test_volume_gradient_is_left_on_the_stream(nc, n):
         assert np.allclose(d.cpu().numpy(), dref, rtol=1e-14, atol=0)
     with pytest.raises(Exception):
         gp.volume(gam[0], torch.zeros_like(masks[0]), 0.3, grad=grads[0])
+
+
+@pytest.mark.parametrize("n", [1, 300, 70001])
+@pytest.mark.parametrize("slack", [0.5, 0.0])
+def test_constraint_that_holds_without_a_multiplier(nc, n, slack):
+    """The first evaluation ends the search: lambda = 0, the history shifted once."""
+    from oracle import mma as M
+    rng = np.random.default_rng(n)
+    x = rng.uniform(0.1, 0.9, n)
+    df0, df1 = -rng.uniform(0.5, 1.5, n) / n, -rng.uniform(0.5, 1.5, n) / n
+    yo, _, _, lo = M.mma_step(0, x, x, x, x, x, -slack, df0, df1)
+    assert lo == 0.0
+    gp = nc.Problem(nc.make_params(2, 2, 2, 0.5, 1e3, 0.71), nc.cavity_bcs())
+    dev = lambda t: torch.tensor(t, dtype=torch.float64, device="cuda")  # noqa: E731
+    s = [dev(x), dev(x + 1), dev(x + 2), dev(x), dev(x)]
+    lam, chg = gp.mma_update(0, *s, dev(df0), -slack, dev(df1))
+    assert lam == 0.0 and chg == pytest.approx(np.abs(yo - x).max(), abs=TOL)
+    assert np.abs(s[0].cpu().numpy() - yo).max() <= 1e-14
+    assert np.array_equal(s[1].cpu().numpy(), x) and np.array_equal(s[2].cpu().numpy(), x + 1)
