@@ -116,12 +116,60 @@ static int refused_sums() {
   return bad;
 }
 
+// The marching plan of a grid: the cheapest of all run lengths by its rule (a plain search), sums
+// that fit the element scratch, and every face row covered.
+static int plans() {
+  int bad = 0;
+  auto up = [](long long a, long long b) { return (a + b - 1) / b; };
+  auto check = [&](int nx, int ny, int nz, bool fp64) {
+    nc::LevelDev d = {};
+    d.nx = nx;
+    d.ny = ny;
+    d.nz = nz;
+    d.E = (long long)nx * ny * nz;
+    d.Nn = (nx + 1LL) * (ny + 1) * (nz + 1);
+    const nc::MarchPlan p = nc::march_plan(d, fp64);
+    const long long stride = 32 % (nx + 1) == 0 ? 32 : 31, faces = (nx + 1LL) * nz, slots = fp64 ? 608 : 8 * 152;
+    const double extra = fp64 ? 0.05 : 0.6;
+    auto steps = [&](int rc, long long warps) {
+      const long long turns = up(warps, slots);
+      return (rc + extra) * (fp64 && turns == 1 ? 1.12 : (double)turns);
+    };
+    int rc = 1;
+    double cost = steps(1, up(faces * ny, stride));
+    for (int r = 2; r <= 24 && r <= ny; ++r) {
+      const long long warps = up(faces, stride) * up(ny, r);
+      if (steps(r, warps) < cost && warps * (r + 1) * 320 <= nc::scratch_len(d.E)) {
+        rc = r;
+        cost = steps(r, warps);
+      }
+    }
+    const bool ok = p.rc == rc && p.stride == stride && p.flat == (rc == 1) && p.runs == up(ny, rc) &&
+                    p.nchunk == up(p.flat ? faces * ny : faces, stride) && p.scratch() <= nc::scratch_len(d.E);
+    if (!ok) bad += report((std::to_string(nx) + "x" + std::to_string(ny) + "x" + std::to_string(nz)).c_str(), false);
+  };
+  for (bool fp64 : {false, true}) {
+    for (int nx = 1; nx <= 34; ++nx)
+      for (int ny = 1; ny <= 30; ++ny)
+        for (int nz = 1; nz <= 12; ++nz) check(nx, ny, nz, fp64);
+    unsigned s = 12345;
+    auto next = [&](int hi) { return 1 + (int)((s = s * 1664525u + 1013904223u) >> 8) % hi; };
+    for (int t = 0; t < 20000; ++t) {
+      check(next(400), next(400), next(400), fp64);
+      check(next(6), next(40), next(200000), fp64);
+      check(next(300000), next(6), next(6), fp64);
+    }
+  }
+  return bad;
+}
+
 int main(int argc, char** argv) {
   const std::string check = argc > 1 ? argv[1] : "";
   if (check == "smoother_levels") return smoother_levels();
   if (check == "device_loops") return device_loops();
   if (check == "tickets") return tickets();
   if (check == "refused_sums") return refused_sums();
+  if (check == "plans") return plans();
   std::printf("unknown check\n");
   return 2;
 }

@@ -26,7 +26,7 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("check", ["smoother_levels", "device_loops", "tickets", "refused_sums"])
+@pytest.mark.parametrize("check", ["smoother_levels", "device_loops", "tickets", "refused_sums", "plans"])
 def test_host_side(program, check):
     r = subprocess.run([program, check], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
