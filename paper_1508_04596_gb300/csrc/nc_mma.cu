@@ -133,12 +133,10 @@ struct MmaCoef {
 };
 constexpr int MMA_COEFS = 12;
 
-// Rounds v where it stands: what is computed from it later does not depend on whether it was
-// just computed (and could be contracted into a fused multiply-add) or read back.
-__device__ __forceinline__ double rounded(double v) {
-  asm volatile("" : "+d"(v));
-  return v;
-}
+// The arithmetic from here to mma_term names its fused multiply-adds and its rounded products:
+// left to the compiler, kernels that read the coefficients and kernels that form them fuse
+// different operations, and the design would depend on which of them ran.
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 
 // The coefficients but for w, c, ta and tb, which only the evaluations need.
 __device__ __forceinline__ MmaCoef mma_coef_y(double xj, double l, double u, double a0, double a1,
@@ -146,23 +144,23 @@ __device__ __forceinline__ MmaCoef mma_coef_y(double xj, double l, double u, dou
   const double d = xmax - xmin;
   const double a0p = fmax(a0, 0.0), a0m = fmax(-a0, 0.0);
   const double a1p = fmax(a1, 0.0), a1m = fmax(-a1, 0.0);
-  const double ux2 = (u - xj) * (u - xj), xl2 = (xj - l) * (xj - l);
+  const double ux = u - xj, xl = xj - l, ux2 = mul(ux, ux), xl2 = mul(xl, xl);
   MmaCoef m;
   m.l = l;
   m.u = u;
-  m.p0 = rounded(ux2 * (1.001 * a0p + 0.001 * a0m + r));
-  m.q0 = rounded(xl2 * (0.001 * a0p + 1.001 * a0m + r));
-  m.p1 = rounded(ux2 * (1.001 * a1p + 0.001 * a1m + r));
-  m.q1 = rounded(xl2 * (0.001 * a1p + 1.001 * a1m + r));
-  m.alpha = fmax(fmax(xmin, l + 0.1 * (xj - l)), xj - move * d);
-  m.beta = fmin(fmin(xmax, u - 0.1 * (u - xj)), xj + move * d);
+  m.p0 = mul(ux2, fma(1.001, a0p, fma(0.001, a0m, r)));
+  m.q0 = mul(xl2, fma(0.001, a0p, fma(1.001, a0m, r)));
+  m.p1 = mul(ux2, fma(1.001, a1p, fma(0.001, a1m, r)));
+  m.q1 = mul(xl2, fma(0.001, a1p, fma(1.001, a1m, r)));
+  m.alpha = fmax(fmax(xmin, fma(0.1, xl, l)), fma(-move, d, xj));
+  m.beta = fmin(fmin(xmax, fma(-0.1, ux, u)), fma(move, d, xj));
   m.alpha = fmin(m.alpha, m.beta);  // limits that cross (x far outside the box): the upper one holds
   return m;
 }
 
 __device__ __forceinline__ double mma_term_at(const MmaCoef& m, double y) {
   const double a = m.u - y, b = y - m.l;
-  return (m.p1 * b + m.q1 * a) / (a * b);
+  return fma(m.p1, b, mul(m.q1, a)) / mul(a, b);
 }
 
 __device__ __forceinline__ MmaCoef mma_coef(double xj, double l, double u, double a0, double a1,
@@ -177,18 +175,18 @@ __device__ __forceinline__ MmaCoef mma_coef(double xj, double l, double u, doubl
 
 // Minimiser y_j(lam) of the separable Lagrangian, clipped to [alpha, beta].
 __device__ __forceinline__ double mma_y(const MmaCoef& m, double lam) {
-  const double sP = sqrt(m.p0 + lam * m.p1), sQ = sqrt(m.q0 + lam * m.q1);
-  return fmin(fmax((m.l * sP + m.u * sQ) / (sP + sQ), m.alpha), m.beta);
+  const double sP = sqrt(fma(lam, m.p1, m.p0)), sQ = sqrt(fma(lam, m.q1, m.q0));
+  return fmin(fmax(fma(m.l, sP, mul(m.u, sQ)) / (sP + sQ), m.alpha), m.beta);
 }
 // Its term of the approximated constraint (P, Q > 0: the approximation adds 1e-5 / d).
 // Where P or Q is infinite (an infinite entry of df0), y is not a number and mma_y gives
 // alpha; the first comparison below is written so that the term goes with it.
 __device__ __forceinline__ double mma_term(const MmaCoef& m, double lam) {
-  const double P = m.p0 + lam * m.p1, Q = m.q0 + lam * m.q1;
-  const double rP = rsqrt(P), rQ = rsqrt(Q), sP = P * rP, sQ = Q * rQ;
-  const double den = sP + sQ, num = m.l * sP + m.u * sQ;  // y = num / den
-  const double t = (den * m.w) * (m.p1 * rP + m.q1 * rQ) - m.c;
-  return !(num > m.alpha * den) ? m.ta : (num >= m.beta * den ? m.tb : t);
+  const double P = fma(lam, m.p1, m.p0), Q = fma(lam, m.q1, m.q0);
+  const double rP = rsqrt(P), rQ = rsqrt(Q), sP = mul(P, rP), sQ = mul(Q, rQ);
+  const double den = sP + sQ, num = fma(m.l, sP, mul(m.u, sQ));  // y = num / den
+  const double t = fma(mul(den, m.w), fma(m.p1, rP, mul(m.q1, rQ)), -m.c);
+  return !(num > mul(m.alpha, den)) ? m.ta : (num >= mul(m.beta, den) ? m.tb : t);
 }
 
 // The search for the multiplier.  a is the newest point, b the end of the bracket
