@@ -421,9 +421,7 @@ MarchPlan march_plan(const LevelDev& d, bool fp64) {
   MarchPlan q = p;
   q.flat = 0;
   q.nchunk = (faces + p.stride - 1) / p.stride;
-  // (a run costs at least one turn of its rows: the small grids, whose calls the host bounds,
-  // end here at once)
-  for (q.rc = 2; q.rc <= 24 && q.rc <= d.ny && q.rc + extra < cost; ++q.rc) {
+  for (q.rc = 2; q.rc <= 24 && q.rc <= d.ny; ++q.rc) {
     q.runs = (d.ny + q.rc - 1) / q.rc;
     const double t = steps(q);
     if (t < cost && q.scratch() <= scratch_len(d.E)) {
