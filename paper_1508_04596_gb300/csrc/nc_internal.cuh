@@ -167,6 +167,8 @@ struct nc_ctx {
   void* gj = nullptr;         // the coarsest level's dense inversion on the device
   size_t gj_bytes = 0;
   cudaStream_t cap = nullptr; // stream used to capture the V-cycle graph
+  cudaStream_t red_stream = nullptr;  // the stream of the first call that reduces
+  int red_streams = 0;        // streams of such calls so far, 2 for more than one
   void* pin = nullptr;        // page-locked memory for scalars read while the stream goes on
   cudaEvent_t ev = nullptr;   // marks that read
   double* filt[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // filter CG
@@ -272,12 +274,16 @@ void op_coarsen_elem(const LevelDev& fine, const R* gf, const LevelDev& coarse, 
 constexpr long long RED_PARTIALS = (long long)(MAX_RESTART + 2) * RED_BLOCKS_MAX;
 constexpr size_t PIN_BYTES = 256;  // nc_ctx::pin
 inline unsigned* red_ticket(double* partial) { return (unsigned*)(partial + RED_PARTIALS); }
-// Every public call that reduces starts with this: reductions of two calls that overlapped
-// on one context (the caller's error) may have left a count behind.  Errors of earlier calls
-// are dropped: what cudaGetLastError says at the call's next read is its own launches'.
+// Every public call that reduces starts with this.  Reductions of two calls that overlap on
+// one context (the caller's error) may leave a count behind; they need two streams, so a
+// context that has seen a second stream clears its ticket at every call (1 us, which a
+// small orthogonalisation would notice).  Errors of earlier calls are dropped: what
+// cudaGetLastError says at the call's next read is its own launches'.
 inline void red_start(nc_ctx* ctx, cudaStream_t s) {
   cudaGetLastError();
-  cudaMemsetAsync(red_ticket(ctx->partial), 0, sizeof(unsigned), s);
+  if (ctx->red_streams == 0) ctx->red_stream = s;
+  if (ctx->red_streams < 2) ctx->red_streams = ctx->red_stream == s ? 1 : 2;
+  if (ctx->red_streams == 2) cudaMemsetAsync(red_ticket(ctx->partial), 0, sizeof(unsigned), s);
 }
 template <typename Rd, typename Rs>
 void vcast(long long n, const Rs* x, Rd* y, cudaStream_t s);

@@ -72,24 +72,29 @@ static int device_loops() {
   return bad;
 }
 
-// A count that overlapping reductions left in a context's ticket is gone with the next call.
+// A count that overlapping reductions (calls on two streams) left in a context's ticket is gone
+// with the next call, on whichever stream.
 static int tickets() {
   int bad = 0;
   nc_ctx* ctx = context(4);
+  const cudaStream_t first = (cudaStream_t)16, second = (cudaStream_t)32;
   unsigned* const ticket = nc::red_ticket(ctx->partial);
   const long long n = 5LL * 125, E = 64;
   std::vector<double> x(n, 0.0), g(E, 0.5), r(n, 0.0), l(n, 0.0);
   double h[3];
   nc_solve_info info;
+  nc_arnoldi_orth(ctx, n, 1, r.data(), n, l.data(), h, NC_FP64, first);
   auto call = [&](const char* what, auto f) {
-    *ticket = 7;
-    f();
-    bad += report(what, *ticket == 0);
+    for (cudaStream_t s : {second, second, first}) {
+      *ticket = 7;
+      f(s);
+      bad += report(what, *ticket == 0);
+    }
   };
-  call("nc_arnoldi_orth", [&] { nc_arnoldi_orth(ctx, n, 1, r.data(), n, l.data(), h, NC_FP64, nullptr); });
-  call("nc_objective", [&] { nc_objective(ctx, x.data(), h, r.data(), nullptr); });
-  call("nc_newton_solve", [&] { nc_newton_solve(ctx, g.data(), x.data(), nullptr, &info, nullptr); });
-  call("nc_adjoint_solve", [&] { nc_adjoint_solve(ctx, x.data(), g.data(), r.data(), l.data(), nullptr, &info, nullptr); });
+  call("nc_arnoldi_orth", [&](cudaStream_t s) { nc_arnoldi_orth(ctx, n, 1, r.data(), n, l.data(), h, NC_FP64, s); });
+  call("nc_objective", [&](cudaStream_t s) { nc_objective(ctx, x.data(), h, r.data(), s); });
+  call("nc_newton_solve", [&](cudaStream_t s) { nc_newton_solve(ctx, g.data(), x.data(), nullptr, &info, s); });
+  call("nc_adjoint_solve", [&](cudaStream_t s) { nc_adjoint_solve(ctx, x.data(), g.data(), r.data(), l.data(), nullptr, &info, s); });
   nc_destroy(ctx);
   return bad;
 }
