@@ -133,9 +133,10 @@ struct MmaCoef {
 };
 constexpr int MMA_COEFS = 12;
 
-// The arithmetic from here to mma_term names its fused multiply-adds and its rounded products:
-// left to the compiler, kernels that read the coefficients and kernels that form them fuse
-// different operations, and the design would depend on which of them ran.
+// The arithmetic from here to mma_term names its rounded products and fuses only where it says
+// so (the evaluations, which the FP64 pipe bounds): left to the compiler, kernels that read the
+// coefficients and kernels that form them fuse different operations, and the design would
+// depend on which of them ran.
 __device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
 
 // The coefficients but for w, c, ta and tb, which only the evaluations need.
@@ -148,12 +149,12 @@ __device__ __forceinline__ MmaCoef mma_coef_y(double xj, double l, double u, dou
   MmaCoef m;
   m.l = l;
   m.u = u;
-  m.p0 = mul(ux2, fma(1.001, a0p, fma(0.001, a0m, r)));
-  m.q0 = mul(xl2, fma(0.001, a0p, fma(1.001, a0m, r)));
-  m.p1 = mul(ux2, fma(1.001, a1p, fma(0.001, a1m, r)));
-  m.q1 = mul(xl2, fma(0.001, a1p, fma(1.001, a1m, r)));
-  m.alpha = fmax(fmax(xmin, fma(0.1, xl, l)), fma(-move, d, xj));
-  m.beta = fmin(fmin(xmax, fma(-0.1, ux, u)), fma(move, d, xj));
+  m.p0 = mul(ux2, mul(1.001, a0p) + mul(0.001, a0m) + r);
+  m.q0 = mul(xl2, mul(0.001, a0p) + mul(1.001, a0m) + r);
+  m.p1 = mul(ux2, mul(1.001, a1p) + mul(0.001, a1m) + r);
+  m.q1 = mul(xl2, mul(0.001, a1p) + mul(1.001, a1m) + r);
+  m.alpha = fmax(fmax(xmin, l + mul(0.1, xl)), xj - mul(move, d));
+  m.beta = fmin(fmin(xmax, u - mul(0.1, ux)), xj + mul(move, d));
   m.alpha = fmin(m.alpha, m.beta);  // limits that cross (x far outside the box): the upper one holds
   return m;
 }
@@ -175,8 +176,8 @@ __device__ __forceinline__ MmaCoef mma_coef(double xj, double l, double u, doubl
 
 // Minimiser y_j(lam) of the separable Lagrangian, clipped to [alpha, beta].
 __device__ __forceinline__ double mma_y(const MmaCoef& m, double lam) {
-  const double sP = sqrt(fma(lam, m.p1, m.p0)), sQ = sqrt(fma(lam, m.q1, m.q0));
-  return fmin(fmax(fma(m.l, sP, mul(m.u, sQ)) / (sP + sQ), m.alpha), m.beta);
+  const double sP = sqrt(m.p0 + mul(lam, m.p1)), sQ = sqrt(m.q0 + mul(lam, m.q1));
+  return fmin(fmax((mul(m.l, sP) + mul(m.u, sQ)) / (sP + sQ), m.alpha), m.beta);
 }
 // Its term of the approximated constraint (P, Q > 0: the approximation adds 1e-5 / d).
 // Where P or Q is infinite (an infinite entry of df0), y is not a number and mma_y gives
