@@ -40,10 +40,14 @@ inline unsigned map_blocks(long long n) {
   return (unsigned)b;
 }
 
-// One block up to 4,096 elements: four chunks a thread cost less than another block's
-// fence, atomic and second read (2 us of the 4 a small reduction takes).
+// One block up to 4,096 elements in FP64: four chunks a thread cost less than another block's
+// fence, atomic and second read (2 us of the 4 a small reduction takes).  In FP32 a block
+// sums no more than WIDE_FROM elements: its sum is FP32, those of blocks meet in FP64.
+template <typename R>
 inline int red_blocks(long long n) {
-  long long b = n <= 4096 ? 1 : (n + RED_THREADS * 8 - 1) / (RED_THREADS * 8);
+  const long long per = RED_THREADS * 8;
+  static_assert(WIDE_FROM == RED_THREADS * 8, "an ordinary block's elements");
+  long long b = sizeof(R) == 8 && n <= 2 * per ? 1 : (n + per - 1) / per;
   if (b < 1) b = 1;
   if (b > RED_BLOCKS_MAX) b = RED_BLOCKS_MAX;
   return (int)b;
@@ -168,16 +172,10 @@ __device__ __forceinline__ void sub_cols(const R* __restrict__ X, long long ld, 
   }
 }
 
-// Block sum of one value per thread -> partial[blockIdx.x].
+// Block-level sum of one value per thread, result valid in thread 0.
 template <typename T>
-__device__ __forceinline__ void block_partial(T v, double* partial) {
-  if constexpr (sizeof(T) == 8) {
-    v = block_fold<false, RED_THREADS>(v);
-    if (threadIdx.x == 0) partial[blockIdx.x] = v;
-  } else {
-    const T w[1] = {v};
-    block_values<RED_THREADS>(w, 1, partial);
-  }
+__device__ __forceinline__ T block_sum(T v) {
+  return block_fold<false, RED_THREADS>(v);
 }
 
 // The last block's end of a reduction of cnt values (nc_reduce.cuh).
@@ -348,7 +346,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_arnoldi_update(long long n, int
     w[i] = a;
     if (t) t[i] = a / D[i];
   });
-  block_partial(acc2, partial);
+  const R s = block_sum(acc2);
+  if (threadIdx.x == 0) partial[blockIdx.x] = double(s);
   if (!last_block(ticket)) return;
   fold_values(1, gridDim.x, partial, [&](int, double v) { put_norm(Hd + HD_SIG2 + k, Hd + HD_ISIG + k, v); });
   if (ls) {
@@ -391,7 +390,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_init_basis(long long n, const R
     if (copy) v0[i] = a;
     t[i] = a / D[i];
   });
-  block_partial(acc2, partial);
+  const R s = block_sum(acc2);
+  if (threadIdx.x == 0) partial[blockIdx.x] = double(s);
   finish(1, partial, ticket, [&](int, double v) { put_norm(Hd + HD_SIG2, Hd + HD_ISIG, v); });
 }
 
@@ -573,7 +573,7 @@ void vscal(long long n, R a, R* y, cudaStream_t s) {
 template <typename R>
 static void mdot(long long n, int k, const R* X, long long ld, const R* y, int self, double* out,
                  const double* sig2, double* cf, double* partial, cudaStream_t s) {
-  const int nb = red_blocks(n);
+  const int nb = red_blocks<R>(n);
   if ((k == 0 || mv_aligned(X, ld)) && al16(y))
     k_mdot<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, y, self, partial, out, sig2, cf,
                                                red_ticket(partial));
@@ -599,7 +599,7 @@ void vmdot_cf(long long n, int k, const R* X, long long ld, const R* y, double* 
 template <typename R>
 void vinit_basis(long long n, const R* r, const R* D, R* v0, R* t, double* Hd, double* partial,
                  cudaStream_t s) {
-  const int nb = red_blocks(n);
+  const int nb = red_blocks<R>(n);
   if (al16(r) && al16(D) && al16(v0) && al16(t))
     k_init_basis<R, true><<<nb, RED_THREADS, 0, s>>>(n, r, D, v0, t, Hd, partial, red_ticket(partial));
   else
@@ -608,7 +608,7 @@ void vinit_basis(long long n, const R* r, const R* D, R* v0, R* t, double* Hd, d
 template <typename R>
 void varnoldi_update(long long n, int k, const R* X, long long ld, const R* D, R* w, R* t, double* Hd,
                      bool ls, double* partial, cudaStream_t s) {
-  const int nb = red_blocks(n), fused = ls && k <= LS_MAX;
+  const int nb = red_blocks<R>(n), fused = ls && k <= LS_MAX;
   if (mv_aligned(X, ld) && al16(D) && al16(w) && al16(t))
     k_arnoldi_update<R, true><<<nb, RED_THREADS, 0, s>>>(n, k, X, ld, D, w, t, Hd, fused, partial,
                                                          red_ticket(partial));

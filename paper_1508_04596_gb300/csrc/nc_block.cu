@@ -12,8 +12,8 @@
 // at six steps.
 //
 // The arithmetic is that of smooth() in nc_solver.cu: the basis is unnormalised, dots
-// and norms are summed in FP32 within a warp, in FP64 over the warps, in a fixed order, and
-// their quotients are formed in FP64.
+// and norms are summed in FP32 in a fixed order (over the warps in FP64 where the level has
+// more unknowns than one block of the general kernels sums) and their quotients formed in FP64.
 #include "nc_element_f2.cuh"
 #include "nc_internal.cuh"
 #include "nc_reduce.cuh"
@@ -111,8 +111,16 @@ __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ 
     for (int f = 0; f < 5; ++f)
       if ((fl >> f) & 1) w[f] = t[f * Nn + n];
   };
-  // The sum over the eight lanes from lane 8 g on, in all of them: the warps' parts of a value.
-  auto fold8 = [&](double v) {
+  const bool wide = N > WIDE_FROM;
+  // The warps' parts of value q, summed: by every lane, or with `wide` by eight lanes together
+  // (lane & 7 the warp), valid in all of them.
+  auto over_warps = [&](int q) -> double {
+    if (!wide) {
+      float v = 0.0f;
+      for (int m = 0; m < BW; ++m) v += warp[m][q];
+      return v;
+    }
+    double v = warp[lane & 7][q];
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
@@ -124,7 +132,7 @@ __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ 
     if (lane == 0) warp[wid][0] = s;
     __syncthreads();
     if (wid == BW - 1) {
-      const double v2 = fold8(warp[lane & 7][0]);
+      const double v2 = over_warps(0);
       if (lane == 0) put_norm(sig2 + j, isig + j, v2);
     }
   };
@@ -182,7 +190,7 @@ __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ 
     __syncthreads();
     if (tid < 8 * BW) {  // eight lanes a dot
       const int q = tid >> 3;
-      const double v = fold8(q <= j ? (double)warp[tid & 7][q] : 0.0);
+      const double v = over_warps(q);  // not used beyond j
       if ((tid & 7) == 0 && q <= j) {
         H[j * (k + 1) + q] = v;
         cf[q] = (float)(v * isig[q] * isig[q]);

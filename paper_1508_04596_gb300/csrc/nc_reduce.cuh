@@ -34,18 +34,19 @@ __device__ __forceinline__ T block_fold(T v) {
 }
 
 // Block sums of N values per thread (the first cnt of them) to partial[q * gridDim.x +
-// blockIdx.x].  FP32 folds by shuffles within a warp and the warps' sums in FP64: a block may
-// hold a whole vector (4,096 elements), whose sum stays in as many bits as that of two
-// blocks.  An FP64 addition holds a scheduler's unit for
-// 64 cycles whatever the number of active lanes, so FP64 values go through shared
-// memory and one warp adds a value's eight warps before its five shuffle steps: 12
-// additions per value and block instead of 45.
+// blockIdx.x].  FP32 folds by shuffles; in a block of more than eight warps, which may hold
+// more than the WIDE_FROM elements of an ordinary one, the warps' sums meet in FP64, so that
+// the sum keeps the bits that it has over several blocks.  An FP64 addition holds a
+// scheduler's unit for 64 cycles whatever the number of active lanes, so FP64 values go
+// through shared memory and one warp adds a value's eight warps before its five shuffle
+// steps: 12 additions per value and block instead of 45.
 // N <= 8.
 template <int THREADS, typename T>
 __device__ __forceinline__ T* block_buffer() {  // one for every N
   __shared__ T sh[sizeof(T) == 8 ? 8 * THREADS : 8 * (THREADS / 32)];
   return sh;
 }
+constexpr int WIDE_FROM = 2048;
 template <int THREADS, int N, typename T>
 __device__ __forceinline__ void block_values(const T (&v)[N], int cnt, double* partial) {
   static_assert(N <= 8, "the buffer holds 8 values");
@@ -74,7 +75,14 @@ __device__ __forceinline__ void block_values(const T (&v)[N], int cnt, double* p
         if (lane == 0) sh[wid * 8 + q] = t;
       }
     __syncthreads();
-    if ((int)(threadIdx.x & ~31u) < cnt * W) {  // W lanes a value
+    if constexpr (W <= 8) {
+      if ((int)threadIdx.x < cnt) {
+        T t = sh[threadIdx.x];
+#pragma unroll
+        for (int w = 1; w < W; ++w) t += sh[w * 8 + threadIdx.x];
+        partial[(long long)threadIdx.x * gridDim.x + blockIdx.x] = double(t);
+      }
+    } else if ((int)(threadIdx.x & ~31u) < cnt * W) {  // W lanes a value
       const int q = threadIdx.x / W, w = threadIdx.x % W;
       double t = q < cnt ? double(sh[w * 8 + q]) : 0.0;
 #pragma unroll
