@@ -20,11 +20,13 @@
 // enqueues batches of iterations (those after convergence return at once).
 //  * k_cg_apply forms p = r / d + beta p on the fly while it loads its tile, then
 //    q = A p and <p, q>: per plane, the four edge and four corner neighbours are
-//    summed once and meet their weights afterwards, 15 FP64 operations per node
-//    with the update of p, where a sum over the eight elements takes 64;
-//  * k_cg_update takes the steps of x and r with <r, r> and <r, r/d>.
-// FP64 operations bound both (two FP64 lanes per SM).  80x80x160 (1.06M nodes, 19
-// iterations): 1.68 ms, k_cg_apply 58 us and k_cg_update 20 us an iteration; 5.75 ms
+//    summed once and meet their weights afterwards, 15 FP64 operations per node and 2
+//    per slot of the tile for p (23 per node with the halo), where a sum over the
+//    eight elements takes 64;
+//  * k_cg_update takes the steps of x and r with <r, r> and <r, r/d>, 5 per node.
+// FP64 operations bound both (two FP64 lanes per SM): k_cg_apply keeps the pipe 78 % busy
+// on the SMs that have a tile, k_cg_update, which waits for L2 as well, 70 %.  80x80x160
+// (1.06M nodes, 19 iterations): 1.68 ms, k_cg_apply 58 us and k_cg_update 21 us an iteration; 5.75 ms
 // with one kernel per vector operation, a 64-term product (146 us) and three host
 // reads per iteration.
 #include <algorithm>
