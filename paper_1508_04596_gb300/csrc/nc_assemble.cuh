@@ -115,8 +115,8 @@ RowConst<R> row_const(const ElemConst<R>& c, int a) {
   return k;
 }
 
-// FP64 keeps 168 registers (three blocks; 7.5 ms at 64^3 against 7.6 with two), FP32
-// takes 255 (1.3 ms against 1.8 with three, 2.3 with four).
+// FP64 keeps 168 registers (three blocks), FP32 takes 255 (two).  The whole assembly at 64^3 in
+// FP64: 6.89 ms, 6.82 with two blocks; in FP32: 1.49 ms, 1.41 with three, 2.20 with four.
 template <typename R>
 __global__ void __launch_bounds__(128, sizeof(R) == 8 ? 3 : 2)
     k_assemble_rows(LevelDev d, ElemConst<R> c, RowConst<R> kc, const R* __restrict__ x,
