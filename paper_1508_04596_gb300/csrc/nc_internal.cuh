@@ -169,8 +169,8 @@ struct nc_ctx {
   cudaStream_t cap = nullptr; // stream used to capture the V-cycle graph
   cudaStream_t red_stream = nullptr;  // the stream of the first call that reduces
   int red_streams = 0;        // streams of such calls so far, 2 for more than one
-  void* pin = nullptr;        // page-locked memory for scalars read while the stream goes on
-  cudaEvent_t ev = nullptr;   // marks that read
+  void* pin = nullptr;        // page-locked memory that kernels write scalars for the host to
+  cudaEvent_t ev = nullptr;   // recorded after such a kernel, while the stream goes on
   double* filt[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // filter CG
   double* pub_lin = nullptr;  // linearisation of nc_linearize (level 0, FP64)
   void* asm_lin = nullptr;    // linearisation store of nc_assemble in FP64

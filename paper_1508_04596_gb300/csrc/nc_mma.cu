@@ -71,10 +71,11 @@ __device__ __forceinline__ void block_partial(double v, double* partial) {
   if (threadIdx.x == 0) partial[blockIdx.x] = v;
 }
 
-// out[0], out[1]: sums of (1 - gamma_e) and of the active count over the variables
+// out[0], out[1]: sums of (1 - gamma_e) and of the active count over the variables; the same to
+// page-locked memory
 __global__ void __launch_bounds__(MT) k_volume(long long n, const double* __restrict__ g,
                                                const unsigned char* __restrict__ active,
-                                               double* partial, double* out, unsigned* ticket) {
+                                               double* partial, double* out, double* host, unsigned* ticket) {
   double acc = 0.0, cnt = 0.0;
   for (long long j = blockIdx.x * (long long)MT + threadIdx.x; j < n; j += (long long)gridDim.x * MT) {
     if (active && !active[j]) continue;
@@ -87,8 +88,8 @@ __global__ void __launch_bounds__(MT) k_volume(long long n, const double* __rest
   const double s0 = fold_partials<false, MT>(gridDim.x, partial);
   const double s1 = fold_partials<false, MT>(gridDim.x, partial + gridDim.x);
   if (threadIdx.x == 0) {
-    out[0] = s0;
-    out[1] = s1;
+    out[0] = host[0] = s0;
+    out[1] = host[1] = s1;
   }
 }
 
@@ -324,8 +325,9 @@ __device__ __forceinline__ MmaCoef ws_load(const MmaWs& w, long long i) {
   return m;
 }
 
-// The last block's part of an evaluation pass: fold the partials, step the search.
-__device__ __forceinline__ void mma_finish(double acc, double f1, double* partial, MmaSearch* s) {
+// The last block's part of an evaluation pass: fold the partials, step the search; its end
+// (lam, err, done) goes to page-locked memory too.
+__device__ __forceinline__ void mma_finish(double acc, double f1, double* partial, MmaSearch* s, MmaSearch* host) {
   block_partial<false>(acc, partial);
   if (!last_block(&s->ticket)) return;
   const double sum = fold_partials<false, MT>(gridDim.x, partial);
@@ -333,6 +335,11 @@ __device__ __forceinline__ void mma_finish(double acc, double f1, double* partia
     MmaSearch t = *s;
     mma_advance(t, f1, sum);
     *s = t;
+    if (t.done) {
+      host->lam = t.lam;
+      host->err = t.err;
+      host->done = t.done;
+    }
   }
 }
 
@@ -348,7 +355,7 @@ struct MmaArgs {
 // first evaluation, at lam = 0.
 template <bool STORE>
 __global__ void __launch_bounds__(MT) k_mma_begin(MmaArgs a, int iter, MmaWs w, double* partial,
-                                                  MmaSearch* s) {
+                                                  MmaSearch* s, MmaSearch* host) {
   double acc = 0.0;
   const long long base = (long long)blockIdx.x * w.seg;
   long long cnt = 0;
@@ -374,13 +381,16 @@ __global__ void __launch_bounds__(MT) k_mma_begin(MmaArgs a, int iter, MmaWs w, 
     cnt += total;
   }
   if (STORE && threadIdx.x == 0) w.cnt[blockIdx.x] = (int)cnt;
-  mma_finish(acc, a.f1, partial, s);
+  mma_finish(acc, a.f1, partial, s, host);
 }
 
 // One evaluation of the approximated constraint at the search's multiplier, with the same
-// bits whether the coefficients come from the workspace (STORE) or from the variables.
+// bits whether the coefficients come from the workspace (STORE) or from the variables.  Three
+// blocks per SM: at two (92 registers) 110,592 variables take a second wave, 950 us instead of
+// 855 for an update of about 50 passes.
 template <bool STORE>
-__global__ void __launch_bounds__(MT) k_mma_dual(MmaArgs a, MmaWs w, double* partial, MmaSearch* s) {
+__global__ void __launch_bounds__(MT, 3) k_mma_dual(MmaArgs a, MmaWs w, double* partial, MmaSearch* s,
+                                                 MmaSearch* host) {
   if (s->done) return;
   const double lam = s->lam;
   double acc = 0.0;
@@ -405,14 +415,15 @@ __global__ void __launch_bounds__(MT) k_mma_dual(MmaArgs a, MmaWs w, double* par
       at = (at + total) % MT;
     }
   }
-  mma_finish(acc, a.f1, partial, s);
+  mma_finish(acc, a.f1, partial, s, host);
 }
 
 // x^{k+1} = y(lam) once the search has ended; the previous iterates shift;
-// s->change = max |y - x|.
+// host->change = max |y - x|.
 template <bool STORE>
 __global__ void __launch_bounds__(MT) k_mma_commit(MmaArgs a, MmaWs w, double* x, double* xo1,
-                                                   double* xo2, double* partial, MmaSearch* s) {
+                                                   double* xo2, double* partial, MmaSearch* s,
+                                                   MmaSearch* host) {
   if (!s->done || s->err) return;
   const double lam = s->lam;
   double mx = 0.0;
@@ -439,7 +450,7 @@ __global__ void __launch_bounds__(MT) k_mma_commit(MmaArgs a, MmaWs w, double* x
   block_partial<true>(mx, partial);
   if (!last_block(&s->ticket)) return;
   const double v = fold_partials<true, MT>(gridDim.x, partial);
-  if (threadIdx.x == 0) s->change = v;
+  if (threadIdx.x == 0) host->change = v;
 }
 
 // out = clamp(in, lo, hi) on active entries, fixed (or 0) elsewhere
@@ -454,14 +465,6 @@ __global__ void k_design_map(long long n, const double* in, const unsigned char*
 }
 
 inline unsigned grid1(long long n) { return (unsigned)((n + MT - 1) / MT); }
-
-// A read of device memory to ctx->pin that does not hold up what is enqueued after it:
-// read_end waits for the copy, not for the stream.
-nc_status read_begin(nc_ctx* ctx, const void* d, size_t bytes, cudaStream_t s, const char* what) {
-  const nc_status st = cuda_check(ctx, cudaMemcpyAsync(ctx->pin, d, bytes, cudaMemcpyDeviceToHost, s), what);
-  return st != NC_OK ? st : cuda_check(ctx, cudaEventRecord(ctx->ev, s), what);
-}
-nc_status read_end(nc_ctx* ctx, const char* what) { return cuda_check(ctx, cudaEventSynchronize(ctx->ev), what); }
 
 // The coefficient workspace of nc_mma_update, kept by the context (grown when a
 // larger problem asks).  False if the device would keep less than 8 GB free: the
@@ -522,16 +525,17 @@ nc_status nc_volume(nc_ctx* ctx, long long n, const double* gamma, const unsigne
   cudaStream_t s = (cudaStream_t)stream;
   unsigned* ticket = (unsigned*)(ctx->dscal + 2);
   cudaMemsetAsync(ticket, 0, sizeof(unsigned), s);
-  k_volume<<<mma_blocks(n), MT, 0, s>>>(n, gamma, active, ctx->partial, ctx->dscal, ticket);
+  double* const sc = (double*)ctx->pin;
+  k_volume<<<mma_blocks(n), MT, 0, s>>>(n, gamma, active, ctx->partial, ctx->dscal, sc, ticket);
   // the host waits for the sums alone; the gradient is left on the stream
-  nc_status st = read_begin(ctx, ctx->dscal, 2 * sizeof(double), s, "nc_volume");
+  nc_status st = cuda_check(ctx, cudaEventRecord(ctx->ev, s), "nc_volume");
   if (dgdgamma) k_volume_grad<<<grid1(n), MT, 0, s>>>(n, active, ctx->dscal, vf, dgdgamma);
-  if (st == NC_OK) st = read_end(ctx, "nc_volume");
+  if (st == NC_OK) st = cuda_check(ctx, cudaEventSynchronize(ctx->ev), "nc_volume");
+  if (st == NC_OK) st = cuda_check(ctx, cudaGetLastError(), "nc_volume");
   if (st != NC_OK) return st;
-  const double* const sc = (const double*)ctx->pin;
   if (!(sc[1] > 0.0)) return set_err(ctx, NC_ERR_ARG, "nc_volume: no active variable");
   *g_host = sc[0] * (1.0 / (vf * sc[1])) - 1.0;
-  return cuda_check(ctx, cudaGetLastError(), "nc_volume");
+  return NC_OK;
 }
 
 nc_status nc_mma_update(nc_ctx* ctx, long long n, int iter, double* x, double* xold1,
@@ -556,42 +560,46 @@ nc_status nc_mma_update(nc_ctx* ctx, long long n, int iter, double* x, double* x
   cudaGetLastError();  // below, only this call's launches are meant
   cudaMemsetAsync(srch, 0, sizeof(MmaSearch), s);
   double* part = ctx->partial;
-  if (store)
-    k_mma_begin<true><<<nb, MT, 0, s>>>(a, iter, w, part, srch);
-  else
-    k_mma_begin<false><<<nb, MT, 0, s>>>(a, iter, w, part, srch);
+  // the end of the search and the change, written by the kernels: a copy between the first
+  // evaluation and the next would cost a small update 4 to 8 %
+  MmaSearch* const h = (MmaSearch*)ctx->pin;
   static_assert(sizeof(MmaSearch) <= PIN_BYTES, "ctx->pin holds the search");
+  *h = MmaSearch{};
+  if (store)
+    k_mma_begin<true><<<nb, MT, 0, s>>>(a, iter, w, part, srch, h);
+  else
+    k_mma_begin<false><<<nb, MT, 0, s>>>(a, iter, w, part, srch, h);
   auto search = [&](int passes) {
     for (int i = 0; i < passes; ++i) {
       if (store)
-        k_mma_dual<true><<<nb, MT, 0, s>>>(a, w, part, srch);
+        k_mma_dual<true><<<nb, MT, 0, s>>>(a, w, part, srch, h);
       else
-        k_mma_dual<false><<<nb, MT, 0, s>>>(a, w, part, srch);
+        k_mma_dual<false><<<nb, MT, 0, s>>>(a, w, part, srch, h);
     }
   };
-  nc_status st = read_begin(ctx, srch, sizeof(MmaSearch), s, "nc_mma_update");
-  if (st != NC_OK) return st;
+  nc_status st = cuda_check(ctx, cudaEventRecord(ctx->ev, s), "nc_mma_update");
   search(MMA_FIRST);
-  if ((st = read_end(ctx, "nc_mma_update")) != NC_OK) return st;
-  int passes = ((const MmaSearch*)ctx->pin)->done ? 0 : MMA_BATCH;
-  MmaSearch h;
+  if (st == NC_OK) st = cuda_check(ctx, cudaEventSynchronize(ctx->ev), "nc_mma_update");
+  int passes = h->done ? 0 : MMA_BATCH;
   do {  // most searches end within the first batch; a pass after the end costs its launch
-    search(passes);
-    passes = MMA_BATCH;
-    if (store)
-      k_mma_commit<true><<<nb, MT, 0, s>>>(a, w, x, xold1, xold2, part, srch);
-    else
-      k_mma_commit<false><<<nb, MT, 0, s>>>(a, w, x, xold1, xold2, part, srch);
-    // a refused launch would leave the state, which ends the loop, as it is
-    st = cuda_check(ctx, cudaGetLastError(), "nc_mma_update");
-    if (st == NC_OK)
-      st = cuda_check(ctx, cudaMemcpyAsync(&h, srch, sizeof(h), cudaMemcpyDeviceToHost, s), "nc_mma_update");
-    if (st == NC_OK) st = cuda_check(ctx, cudaStreamSynchronize(s), "nc_mma_update");
+    if (st == NC_OK) {
+      search(passes);
+      passes = MMA_BATCH;
+      if (store)
+        k_mma_commit<true><<<nb, MT, 0, s>>>(a, w, x, xold1, xold2, part, srch, h);
+      else
+        k_mma_commit<false><<<nb, MT, 0, s>>>(a, w, x, xold1, xold2, part, srch, h);
+      // a refused launch would leave the state, which ends the loop, as it is
+      st = cuda_check(ctx, cudaGetLastError(), "nc_mma_update");
+    }
+    // on an error too: no pass may write to h after the call
+    const nc_status done = cuda_check(ctx, cudaStreamSynchronize(s), "nc_mma_update");
+    if (st == NC_OK) st = done;
     if (st != NC_OK) return st;
-  } while (!h.done);
-  if (h.err) return set_err(ctx, NC_ERR_NAN, "nc_mma_update: non-finite value");
-  if (lambda_host) *lambda_host = h.lam;
-  if (change_host) *change_host = h.change;
+  } while (!h->done);
+  if (h->err) return set_err(ctx, NC_ERR_NAN, "nc_mma_update: non-finite value");
+  if (lambda_host) *lambda_host = h->lam;
+  if (change_host) *change_host = h->change;
   return NC_OK;
 }
 

@@ -65,6 +65,8 @@ static int device_loops() {
                   nc_mma_update(ctx, E, 0, v[0].data(), v[1].data(), v[2].data(), v[3].data(), v[4].data(),
                                 v[5].data(), 0.1, v[6].data(), nullptr, nullptr, nullptr, nullptr,
                                 nullptr) == NC_ERR_CUDA);
+    double g;
+    bad += report("nc_volume", nc_volume(ctx, E, v[0].data(), nullptr, 0.05, &g, v[1].data(), nullptr) == NC_ERR_CUDA);
     bad += report("no error is left", cudaGetLastError() == cudaSuccess);
     fake::refuse = false;
     nc_destroy(ctx);
