@@ -77,10 +77,11 @@ __device__ __forceinline__ int on_face(int i, int n) { return i == 0 || i == n; 
 // 2^b, from the exponent bits (an integer conversion would take the FP64 pipe)
 __device__ __forceinline__ double pow2(int b) { return __hiloint2double((1023 + b) << 20, 0); }
 
-// b_n = sum over the node's elements of rho_e h^3 / 8; r = b, x = 0, <b, b>, <b, b/d>.
+// b_n = sum over the node's elements of rho_e h^3 / 8; r = b, x = 0, <b, b>, <b, b/d>;
+// whether there is nothing to solve goes to page-locked memory too.
 __global__ void __launch_bounds__(FT) k_cg_rhs(LevelDev d, HelmCoef c, const double* __restrict__ rho,
                                                double* __restrict__ r, double* __restrict__ x,
-                                               double* partial, CgState* s) {
+                                               double* partial, CgState* s, int* host_done) {
   const double w = d.h * d.h * d.h * 0.125;
   double bb = 0.0, bz = 0.0;
   for (long long n = blockIdx.x * (long long)FT + threadIdx.x; n < d.Nn; n += (long long)gridDim.x * FT) {
@@ -112,7 +113,7 @@ __global__ void __launch_bounds__(FT) k_cg_rhs(LevelDev d, HelmCoef c, const dou
     s->rz = bz * c.inv_d;
     s->beta = 0.0;
     s->it = 0;
-    s->done = !isfinite(bb) ? 3 : (bb > 0.0 ? 0 : 1);
+    *host_done = s->done = !isfinite(bb) ? 3 : (bb > 0.0 ? 0 : 1);
   }
 }
 
@@ -224,7 +225,8 @@ __global__ void __launch_bounds__(FT) k_cg_apply(LevelDev d, HelmCoef c, HelmTil
 // x += alpha p, r -= alpha q, beta = the ratio of the new <r, r/d> to the old.
 __global__ void __launch_bounds__(FT) k_cg_update(LevelDev d, HelmCoef c, const double* __restrict__ p,
                                                   const double* __restrict__ q, double* __restrict__ x,
-                                                  double* __restrict__ r, double* partial, CgState* s) {
+                                                  double* __restrict__ r, double* partial, CgState* s,
+                                                  int* host_done) {
   if (s->done) return;
   const double alpha = s->alpha;
   double v2[2] = {0.0, 0.0};  // <r, r>, <r, r/d> d_0
@@ -256,8 +258,9 @@ __global__ void __launch_bounds__(FT) k_cg_update(LevelDev d, HelmCoef c, const 
     s->rr = rr;
     s->beta = rz / s->rz;
     s->rz = rz;
-    if (++s->it >= CG_MAX_IT) s->done = 2;
-    if (rr <= s->tol2) s->done = 1;
+    const int it = s->it + 1, done = rr <= s->tol2 ? 1 : it >= CG_MAX_IT ? 2 : 0;
+    s->it = it;
+    if (done) *host_done = s->done = done;
   }
 }
 
@@ -338,23 +341,29 @@ extern "C" nc_status nc_filter(nc_ctx* ctx, const double* rho, double* gamma_f, 
   cudaGetLastError();  // below, only this call's launches are meant
   cudaMemsetAsync(cg, 0, sizeof(CgState), s);
   const unsigned vb = (unsigned)std::min<long long>((Nn + FT - 1) / FT, RED_BLOCKS_MAX);
-  k_cg_rhs<<<vb, FT, 0, s>>>(d, c, rho, r, x, ctx->partial, cg);
+  // The end of the solve, which the host looks at while it enqueues: a field that needs few
+  // iterations (none, if it is zero) does not pay for the launches of a batch.
+  volatile int* const ended = (int*)ctx->pin;
+  *ended = 0;
+  k_cg_rhs<<<vb, FT, 0, s>>>(d, c, rho, r, x, ctx->partial, cg, (int*)ended);
   const HelmTile tile = helm_tile(d);
   const unsigned ab = (unsigned)std::min<long long>(tile.items, (long long)MAX_RESTART * RED_BLOCKS_MAX);
   CgState h;
   int m = 0, batch = 16;  // a radius of 2.5 h takes about 19 iterations
   do {
-    for (int i = 0; i < batch; ++i, ++m) {
+    for (int i = 0; i < batch && !*ended; ++i, ++m) {
       k_cg_apply<<<ab, FT, 0, s>>>(d, c, tile, r, p[m & 1], p[(m + 1) & 1], q, ctx->partial, cg);
-      k_cg_update<<<vb, FT, 0, s>>>(d, c, p[(m + 1) & 1], q, x, r, ctx->partial, cg);
+      k_cg_update<<<vb, FT, 0, s>>>(d, c, p[(m + 1) & 1], q, x, r, ctx->partial, cg, (int*)ended);
     }
     k_elem_mean<<<fblocks(d.E), FT, 0, s>>>(d, x, gamma_f, cg);
     // a refused launch would leave the state, which ends the loop, as it is
-    if ((st = cuda_check(ctx, cudaGetLastError(), "nc_filter")) != NC_OK ||
-        (st = cuda_check(ctx, cudaMemcpyAsync(&h, cg, sizeof(h), cudaMemcpyDeviceToHost, s),
-                         "nc_filter")) != NC_OK ||
-        (st = cuda_check(ctx, cudaStreamSynchronize(s), "nc_filter")) != NC_OK)
-      return st;
+    st = cuda_check(ctx, cudaGetLastError(), "nc_filter");
+    if (st == NC_OK)
+      st = cuda_check(ctx, cudaMemcpyAsync(&h, cg, sizeof(h), cudaMemcpyDeviceToHost, s), "nc_filter");
+    // on an error too: no kernel may write to `ended` after the call
+    const nc_status done = cuda_check(ctx, cudaStreamSynchronize(s), "nc_filter");
+    if (st == NC_OK) st = done;
+    if (st != NC_OK) return st;
     // the rest at the rate seen so far
     const double rate = std::log(h.rr / h.bb) / m;
     const double need = rate < 0.0 ? std::log(h.tol2 / h.rr) / rate + 1.0 : 32.0;
