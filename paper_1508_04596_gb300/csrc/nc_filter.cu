@@ -15,9 +15,10 @@
 // halved the same way.  The SPD system is solved by Jacobi-preconditioned
 // conjugate gradients in FP64.
 //
-// An iteration is two kernels, and no scalar returns to the host: alpha, beta and
+// An iteration is two kernels, and none waits for the host: alpha, beta and
 // the stopping test are taken by the block that ends a reduction, and the host
-// enqueues batches of iterations (those after convergence return at once).
+// enqueues batches of iterations, fewer where it sees the end meanwhile (those after
+// convergence return at once).
 //  * k_cg_apply forms p = r / d + beta p on the fly while it loads its tile, then
 //    q = A p and <p, q>: per plane, the four edge and four corner neighbours are
 //    summed once and meet their weights afterwards, 15 FP64 operations per node and 2
