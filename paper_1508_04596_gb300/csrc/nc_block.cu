@@ -45,8 +45,8 @@ struct BlockScalars {
 // What the dynamic part may take: 227 KB a block less the scalars.  The attribute that
 // allows it belongs to the kernel, not to a context, and solves on other threads set it
 // too, so every launch sets this value and not its own size.
-constexpr int BLOCK_BYTES = 227 * 1024 - 1280;
-static_assert(sizeof(BlockScalars) <= 1280, "the scalars fit what BLOCK_BYTES leaves");
+constexpr int BLOCK_BYTES = 227 * 1024 - 1168;
+static_assert(sizeof(BlockScalars) <= 1168, "the scalars fit what BLOCK_BYTES leaves");
 
 template <bool TR>
 __global__ void __launch_bounds__(BT, 1) k_smooth_block(const __grid_constant__ BlockSmooth a) {

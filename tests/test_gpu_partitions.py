@@ -81,11 +81,12 @@ def test_runs_of_rows(nc, dims, dt, rows):
 def block_takes(dims, its):
     """Whether the one-block smoother takes a level (the rule of smooth_block)."""
     E, Nn = np.prod(dims), np.prod([n + 1 for n in dims])
-    return its <= 8 and E <= 512 and 4 * ((its + 4) * 5 * Nn + 40 * E) <= 227 * 1024 - 1280
+    return its <= 8 and E <= 512 and 4 * ((its + 4) * 5 * Nn + 40 * E) <= 227 * 1024 - 1168
 
 
 @pytest.mark.parametrize("dims,its", [((16, 16, 2), 1), ((32, 16, 1), 1), ((8, 8, 8), 6), ((13, 12, 3), 6),
-                                      ((8, 8, 7), 8), ((16, 16, 1), 8), ((1, 3, 70), 8)])
+                                      ((8, 8, 7), 8), ((16, 16, 1), 8), ((1, 3, 70), 8),
+                                      ((8, 5, 12), 7), ((1, 262, 1), 5)])
 def test_block_smoother_largest_grids(nc, dims, its):
     assert block_takes(dims, its)
     nx, ny, nz = dims
